@@ -314,16 +314,17 @@ ag_status ag_set_gains(ag_ctx* ctx, const float* gains12);
  * (position tracking, Sec. I after Lee et al. 2011; body velocity, Eqs. 6-9;
  * attitude and thrust, Eqs. 1-2; each with the attitude law of Sec. IV-A
  * Eqs. 3-5; or a direct wrench), allocation with clamp and lag, and
- * semi-implicit Euler, without collision tests; records a checkpoint (state +
- * motors) every record_every steps; and writes
+ * semi-implicit Euler, without collision tests; records every step, or a
+ * checkpoint (state + motors) every record_every steps (see ag_backward); and
+ * writes
  *   loss[i] = sum_{t=1..n_steps} w_pos |p_t - p_goal_i|^2 + w_omega |Omega_t|^2
  * (x_t = the state after step t; p_goal float[3][n_envs]). saturated (may be
  * NULL) flags environments in which some motor command was clamped during
  * the rollout; there the gradient uses the clamp's subgradient 0. Requires
  * semi-implicit Euler, one substep per step and no obstacles (else
  * AG_ERR_UNSUPPORTED); AG_ERR_INVALID for n_steps outside 1 .. 2^30, NULL
- * p_goal or loss; AG_ERR_OOM (context still usable) when the checkpoints do
- * not fit. Does not synchronise. Commands, body parameters and gains must not
+ * p_goal or loss; AG_ERR_OOM (context still usable, nothing recorded) when the
+ * checkpoints do not fit. Does not synchronise. Commands, body parameters and gains must not
  * change until ag_backward has run. */
 ag_status ag_rollout_loss(ag_ctx* ctx, uint32_t n_steps, float w_pos, float w_omega, const float* p_goal,
                           float* loss, uint8_t* saturated);
@@ -343,12 +344,12 @@ ag_status ag_rollout_loss(ag_ctx* ctx, uint32_t n_steps, float w_pos, float w_om
  * heading, body x axis vertical) the gradient is that of the fallback
  * branch. Returns AG_ERR_STATE if nothing was recorded.
  * The reverse sweep needs every step's start state again. ag_rollout_loss
- * allocates a tape of the whole horizon (n_steps x 21 floats per
- * environment) when it fits in device memory and in hbm_budget_bytes; then
- * one launch recomputes every checkpoint segment's states into it in
- * parallel before the sweep. Otherwise the tape holds one segment
- * (record_every x 21 floats per environment) and the sweep recomputes the
- * segments one after another. The two agree to float32 rounding. */
+ * allocates a tape of the whole horizon ((n_steps + 1) x 16 floats per
+ * environment) when it fits in device memory and in hbm_budget_bytes, and
+ * writes it as it records. Otherwise it keeps the checkpoints, the tape holds
+ * one segment (record_every x 16 floats per environment) and the sweep
+ * recomputes the segments one after another. The two agree to float32
+ * rounding. */
 ag_status ag_backward(ag_ctx* ctx, const float* loss_weights, float* grad_x0, float* grad_gains,
                       float* grad_gains_per_env, float* grad_targets);
 

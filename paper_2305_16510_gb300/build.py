@@ -26,8 +26,8 @@ CUDA_SOURCES = ["ag_api.cu", "ag_api_task.cu", "ag_api_adjoint.cu", "ag_api_noal
 # multiply-add explicit (fmaf, __ffma2_rn): the compiler contracts nothing
 # else, so each kernel that runs the per-vehicle step (fused, unfused,
 # serving, task; each mode-specialised copy) rounds exactly as the source
-# says, and they agree bit for bit.
-NO_CONTRACTION = {"fleet_kernels.cu", "serve.cu", "task.cu", "depth.cu"}
+# says, and they agree bit for bit. adjoint.cu's record runs the same step.
+NO_CONTRACTION = {"fleet_kernels.cu", "serve.cu", "task.cu", "depth.cu", "adjoint.cu"}
 
 
 def _nvcc() -> str:

@@ -3,31 +3,41 @@
 // Objective (per environment i, over a recorded rollout of H steps):
 //   L_i = sum_{t=1..H} ( w_pos |p_t - p_goal,i|^2 + w_omega |Omega_t|^2 ),
 // with x_t the state after step t. Gradients are taken with respect to the
-// initial state x_0 (13 numbers per environment) and the 12 diagonal
-// controller gains (k_x, k_v, k_R, k_Omega), shared by the fleet.
-//
-// Gradients also go to each environment's four command targets.
+// initial state x_0 (13 numbers per environment), the 12 diagonal controller
+// gains (k_x, k_v, k_R, k_Omega), shared by the fleet, and each environment's
+// four command targets.
 //
 // The differentiated step is the controller of the environment's command mode
 // (position tracking, Sec. I after Lee et al. 2011; body velocity, Eqs. 6-9;
 // attitude and thrust, Eqs. 1-2; or a direct wrench) with the attitude law
 // of Sec. IV-A (Eqs. 3-5), rotor allocation with per-motor clamp (subgradient
 // 0 on a clamped motor) and first-order lag, and the semi-implicit Euler
-// update with quaternion renormalisation. Reverse mode is written out by hand, operation by
-// operation in reverse order; the comments name the forward line each block
-// inverts.
+// update with quaternion renormalisation. Reverse mode is written out by hand;
+// the comments name the forward line each block inverts.
 //
-// Memory: the forward kernel stores a checkpoint (state + motors) every K
-// steps. The backward pass needs every step's start state again. When a tape
-// of the whole horizon fits (AdjointBuffers::full_tape), one launch with a
-// thread per (vehicle, segment) recomputes every segment's step-start states
-// from its checkpoint into the tape at once, and the reverse sweep then reads
-// them; otherwise the sweep walks the segments from the last to the first and
-// recomputes each segment's states into a one-segment tape itself. Either way
-// the sweep recomputes each step's intermediates in registers before
-// back-propagating through it. Per-vehicle gain gradients are summed over the
-// fleet by a deterministic two-level reduction (fixed block order, fixed tree
-// order).
+// What is recorded. A step's reverse needs its start state (13 floats), the
+// realised thrust W.f and which motors passed the clamp (one bit each): 15
+// words, kept as four float4 per vehicle and step (64 bytes), so the record
+// stores and the sweep loads four 16-byte words per step and nothing of the
+// allocation, the lag or the integration is computed again. The end state of
+// a step is the next entry's start state. The record writes every entry as
+// it goes when a tape of the whole horizon fits (AdjointBuffers::full_tape);
+// otherwise it keeps a checkpoint (state + motors) every K steps and the sweep
+// recomputes one segment's entries at a time.
+//
+// Thread slot s handles environment order[s] (grouped by rotor type and
+// command mode, as in the fused step): a warp runs one mode's code. Tape,
+// checkpoints and the norm of q_0 are kept in slot order, so their rows are
+// read and written coalesced whatever the modes are.
+//
+// Attitude adjoint. The adjoint of the unit quaternion is carried as the
+// 3-vector g of the right perturbation q -> q (1, delta / 2): the step's
+// q' = q c / |c|, c = (1, h/2 Omega'), turns it by R(c), and every use of
+// R = R(q) adds a short body-frame vector to it. That replaces the adjoints
+// of q (4), of R's nine entries and of the normalisation.
+//
+// The file is compiled without implicit contraction and every fused
+// multiply-add is explicit, so the record rounds alike in both forms.
 #include <cstdint>
 #include <cuda_runtime.h>
 
@@ -37,452 +47,80 @@
 namespace agk {
 namespace {
 
-// ----------------------------------------------------------------- forward --
-template <int NROT> struct Xs {  // differentiable state of one vehicle
-  V3 p, v;
-  Q4 q;
-  V3 w;
+// One vehicle during the forward rollout.
+template <int NROT> struct Vehicle {
+  VState s;
   float u[NROT];
 };
 
-// Command of one environment over a recorded rollout: its mode, its four
-// targets and the sines and cosines of its angle targets, taken once.
-//   position: (c0, s0) = (cos, sin) psi_d
-//   attitude: (c0, s0) = (cos, sin) phi_d, (c1, s1) = (cos, sin) theta_d
-struct Cmd {
-  float t[4];
-  float c0, s0, c1, s1;
-};
-
-// Intermediates of one forward step, kept for its backward pass.
-template <int NROT> struct Step {
-  float R[3][3];
-  V3 Rd[3];          // columns b1d, b2d, b3d of R_d
-  V3 eR, eW;
-  float f;           // commanded collective thrust
-  float rate;        // commanded yaw rate (velocity, attitude): R_d Omega_d = rate e_3
-  // position
-  V3 a, c, b1c;      // a is also the vehicle-frame acceleration of the velocity mode
-  float ian, icn;    // 1/|a| (0 when |a| <= 1e-9: b3d = e3), 1/|c|
-  bool turned;       // heading fallback (b1c turned by 90 degrees) taken
-  // current yaw and tilt (velocity, attitude)
-  float cps, sps, ir;  // (cos, sin) psi = (R00, R10) * ir; ir = 0 when R00 = R10 = 0
-  V3 B[3];             // columns of R_y(theta_d) R_x(phi_d)
-  V3 vV;               // velocity in the yaw frame
-  float irxz, ianv;    // 1/|(a_x, a_z)|, 1/|a| (both 0 when a_x = a_z = 0)
-  // allocation and integration
-  float pre[NROT];   // A^+ (f, M) before the clamp
-  bool pass[NROT];   // 0 < pre < u_max: the clamp passes the gradient
-  float uc[NROT];    // clamped command
-  Wrench4 M;         // commanded (f, M)
-  Wrench4 W;         // realised wrench
-  V3 vn, wn, pn;
-  Q4 qt, qn;
-  float iqtn;        // 1/|q_t|
-};
-
-struct Gains { V3 kx, kv, kR, kW; };
-
-__device__ __forceinline__ Gains gains_of(const StepParams& P) {
-  return {{P.kx[0], P.kx[1], P.kx[2]}, {P.kv[0], P.kv[1], P.kv[2]}, {P.kR[0], P.kR[1], P.kR[2]},
-          {P.kW[0], P.kW[1], P.kW[2]}};
-}
-
-// One recorded step: the controller of mode MODE -> allocation/clamp/lag ->
-// SIE. x must hold a unit quaternion.
-//   position (Sec. I, Lee 2011): a = -k_x (p - p_d) - k_v v + g e3, f = m a.b3,
-//     b3d = a/|a|, b2d = (b3d x b1c)/|.|, b1d = b2d x b3d, Omega_d = 0
-//   velocity (Eqs. 6-9): v^V = R_psi^T v, a = k_v (v_d - v^V) + g e3,
-//     f = m a.(R_psi^T b3), R_y(theta_d) R_x(phi_d) e3 = a/|a|
-//   attitude (Eqs. 1-2): phi_d, theta_d, psi_dot_d, f given
-//   velocity and attitude: R_d = R_psi R_y(theta_d) R_x(phi_d) with psi the
-//     current yaw, and R_d Omega_d (Eq. 2) = psi_dot_d e3
-//   Eqs. 3-5: e_R = 1/2 vee(R_d^T R - R^T R_d), e_W = W - R^T R_d Omega_d,
-//     M = -k_R e_R - k_W e_W + W x J W
-//   wrench: (f, M) = the targets
-template <int NROT, int MODE>
-__device__ __forceinline__ void forward_step(const Xs<NROT>& x, const Cmd& cm, const Body& b, const Gains& g,
-                                             const StepParams& P, Step<NROT>& S, Xs<NROT>& xn) {
-  constexpr int T = NROT == 4 ? 0 : (NROT == 6 ? 1 : 2);
-  rotation(x.q, S.R);
-  const V3 b3 = {S.R[0][2], S.R[1][2], S.R[2][2]};
-  const V3 JW = {b.jx * x.w.x, b.jy * x.w.y, b.jz * x.w.z};
-  const V3 gyro = cross(x.w, JW);
-  if (MODE == kModeWrench) {
-    S.M = {cm.t[0], cm.t[1], cm.t[2], cm.t[3]};
-  } else {
-    if (MODE == kModePosition) {
-      S.a = {-g.kx.x * (x.p.x - cm.t[0]) - g.kv.x * x.v.x, -g.kx.y * (x.p.y - cm.t[1]) - g.kv.y * x.v.y,
-             -g.kx.z * (x.p.z - cm.t[2]) - g.kv.z * x.v.z + kGravity};
-      S.f = b.m * dot(S.a, b3);
-      const float a2 = dot(S.a, S.a);
-      S.ian = a2 > 1e-18f ? rsqrt_ftz(a2) : 0.f;
-      const V3 b3d = S.ian > 0.f ? S.ian * S.a : V3{0.f, 0.f, 1.f};
-      S.b1c = {cm.c0, cm.s0, 0.f};
-      S.c = cross(b3d, S.b1c);
-      float c2 = dot(S.c, S.c);
-      S.turned = !(c2 > 1e-18f);
-      if (S.turned) {  // commanded thrust along the heading: use the heading turned by 90 degrees
-        S.b1c = {-cm.s0, cm.c0, 0.f};
-        S.c = cross(b3d, S.b1c);
-        c2 = dot(S.c, S.c);  // near 1
-      }
-      S.icn = rsqrt_ftz(c2);
-      const V3 b2d = S.icn * S.c;
-      S.Rd[0] = cross(b2d, b3d);
-      S.Rd[1] = b2d;
-      S.Rd[2] = b3d;
-      S.rate = 0.f;
-    } else {
-      const float rho2 = S.R[0][0] * S.R[0][0] + S.R[1][0] * S.R[1][0];
-      S.ir = rho2 >= kMinNormal ? rsqrt_ftz(rho2) : 0.f;
-      S.cps = S.ir > 0.f ? S.R[0][0] * S.ir : 1.f;
-      S.sps = S.ir > 0.f ? S.R[1][0] * S.ir : 0.f;
-      float cphi, sphi, cth, sth;
-      if (MODE == kModeBodyVel) {
-        S.vV = {S.cps * x.v.x + S.sps * x.v.y, -S.sps * x.v.x + S.cps * x.v.y, x.v.z};
-        S.a = {g.kv.x * (cm.t[0] - S.vV.x), g.kv.y * (cm.t[1] - S.vV.y), g.kv.z * (cm.t[2] - S.vV.z) + kGravity};
-        const V3 b3V = {S.cps * b3.x + S.sps * b3.y, -S.sps * b3.x + S.cps * b3.y, b3.z};
-        S.f = b.m * dot(S.a, b3V);
-        const float rxz2 = S.a.x * S.a.x + S.a.z * S.a.z;
-        const float an2 = rxz2 + S.a.y * S.a.y;
-        S.irxz = 0.f;
-        S.ianv = 0.f;
-        cth = 1.f; sth = 0.f; cphi = 1.f; sphi = 0.f;
-        if (rxz2 >= kMinNormal) {
-          S.irxz = rsqrt_ftz(rxz2);
-          S.ianv = rsqrt_ftz(an2);
-          cth = S.a.z * S.irxz;
-          sth = S.a.x * S.irxz;
-          cphi = rxz2 * S.irxz * S.ianv;
-          sphi = -S.a.y * S.ianv;
-        } else if (an2 > 0.f) {  // a along +-y: phi_d = atan2(-a_y, 0), theta_d = atan2(0, 0) = 0
-          cphi = 0.f;
-          sphi = S.a.y > 0.f ? -1.f : 1.f;
-        }
-        S.rate = cm.t[3];
-      } else {
-        cphi = cm.c0; sphi = cm.s0; cth = cm.c1; sth = cm.s1;
-        S.rate = cm.t[2];
-        S.f = cm.t[3];
-      }
-      S.B[0] = {cth, 0.f, -sth};
-      S.B[1] = {sth * sphi, cphi, cth * sphi};
-      S.B[2] = {sth * cphi, -sphi, cth * cphi};
-#pragma unroll
-      for (int j = 0; j < 3; ++j)
-        S.Rd[j] = {S.cps * S.B[j].x - S.sps * S.B[j].y, S.sps * S.B[j].x + S.cps * S.B[j].y, S.B[j].z};
-    }
-    // E = R_d^T R: E_ij = col_i(R_d) . col_j(R)
-    auto col = [&](int j) { return V3{S.R[0][j], S.R[1][j], S.R[2][j]}; };
-    S.eR = {0.5f * (dot(S.Rd[2], col(1)) - dot(S.Rd[1], col(2))),
-            0.5f * (dot(S.Rd[0], col(2)) - dot(S.Rd[2], col(0))),
-            0.5f * (dot(S.Rd[1], col(0)) - dot(S.Rd[0], col(1)))};
-    S.eW = {x.w.x - S.rate * S.R[2][0], x.w.y - S.rate * S.R[2][1], x.w.z - S.rate * S.R[2][2]};
-    S.M = {S.f, -g.kR.x * S.eR.x - g.kW.x * S.eW.x + gyro.x, -g.kR.y * S.eR.y - g.kW.y * S.eW.y + gyro.y,
-           -g.kR.z * S.eR.z - g.kW.z * S.eW.z + gyro.z};
-  }
-  S.W = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll
-  for (int i = 0; i < NROT; ++i) {
-    S.pre[i] = P.Ap[T][i][0] * S.M.f + P.Ap[T][i][1] * S.M.mx + P.Ap[T][i][2] * S.M.my + P.Ap[T][i][3] * S.M.mz;
-    S.pass[i] = S.pre[i] > 0.f && S.pre[i] < P.u_max;
-    S.uc[i] = fminf(fmaxf(S.pre[i], 0.f), P.u_max);
-    xn.u[i] = x.u[i] + P.alpha * (S.uc[i] - x.u[i]);
-    S.W.f += P.A[T][0][i] * xn.u[i];
-    S.W.mx += P.A[T][1][i] * xn.u[i];
-    S.W.my += P.A[T][2][i] * xn.u[i];
-    S.W.mz += P.A[T][3][i] * xn.u[i];
-  }
-  const float h = P.h;
-  const float fm = S.W.f * b.inv_m, dm = P.drag * b.inv_m;
-  S.vn = {x.v.x + h * (fm * b3.x - dm * x.v.x), x.v.y + h * (fm * b3.y - dm * x.v.y),
-          x.v.z + h * (fm * b3.z - dm * x.v.z - kGravity)};
-  S.wn = {x.w.x + h * b.ijx * (S.W.mx - gyro.x), x.w.y + h * b.ijy * (S.W.my - gyro.y),
-          x.w.z + h * b.ijz * (S.W.mz - gyro.z)};
-  S.pn = x.p + h * S.vn;
-  const float hh = 0.5f * h;
-  const Q4& q = x.q;
-  const V3& w = S.wn;
-  S.qt = {q.w - hh * (q.x * w.x + q.y * w.y + q.z * w.z), q.x + hh * (q.w * w.x + q.y * w.z - q.z * w.y),
-          q.y + hh * (q.w * w.y - q.x * w.z + q.z * w.x), q.z + hh * (q.w * w.z + q.x * w.y - q.y * w.x)};
-  S.iqtn = rsqrt_ftz(S.qt.w * S.qt.w + S.qt.x * S.qt.x + S.qt.y * S.qt.y + S.qt.z * S.qt.z);
-  const float iq = S.iqtn;
-  S.qn = {S.qt.w * iq, S.qt.x * iq, S.qt.y * iq, S.qt.z * iq};
-  xn.p = S.pn;
-  xn.v = S.vn;
-  xn.w = S.wn;
-  xn.q = S.qn;
-}
-
-// ---------------------------------------------------------------- backward --
-template <int NROT> struct Adj {  // adjoint of the state after a step
+// ------------------------------------------------------------------- tape --
+// Entry of a step: (p, v.x) (v.y, v.z, Omega.x, Omega.y) (q) (Omega.z, W.f, pass bits, 0).
+struct TapeStep {
   V3 p, v;
   Q4 q;
   V3 w;
-  float u[NROT];
+  float wf;
+  uint32_t pass;
 };
 
-struct GainAdj { V3 kx, kv, kR, kW; };
-
-// d(a x b): a_bar += b x y_bar, b_bar += y_bar x a
-__device__ __forceinline__ void cross_bwd(V3 a, V3 b, V3 ybar, V3& abar, V3& bbar) {
-  abar = abar + cross(b, ybar);
-  bbar = bbar + cross(ybar, a);
+__device__ __forceinline__ void store_entry(float4* __restrict__ e, size_t n, const VState& s, float wf, uint32_t pass) {
+  e[0] = make_float4(s.p.x, s.p.y, s.p.z, s.v.x);
+  e[n] = make_float4(s.v.y, s.v.z, s.w.x, s.w.y);
+  e[2 * n] = make_float4(s.q.w, s.q.x, s.q.y, s.q.z);
+  e[3 * n] = make_float4(s.w.z, wf, __uint_as_float(pass), 0.f);
 }
 
-// y = x / |x| (1 / |x| = in): x_bar += in (y_bar - y (y . y_bar))
-__device__ __forceinline__ V3 normalize_bwd(V3 y, float in, V3 ybar) {
-  const float d = dot(y, ybar);
-  return in * (ybar - d * y);
+__device__ __forceinline__ TapeStep unpack(float4 a, float4 b, float4 c, float4 d) {
+  return {{a.x, a.y, a.z}, {a.w, b.x, b.y}, {c.x, c.y, c.z, c.w}, {b.z, b.w, d.x}, d.y, __float_as_uint(d.z)};
 }
 
-// Reverse of forward_step. On entry lam is the adjoint of (x_{t+1}, u_{t+1})
-// including this step's loss term; on exit it is the adjoint of (x_t, u_t).
-// Gain adjoints accumulate into gb, target adjoints into tb.
+// ---------------------------------------------------------------- forward --
+// One recorded step from s (unit quaternion): controller -> allocation, clamp
+// and lag -> semi-implicit Euler, the fused step's own functions.
 template <int NROT, int MODE>
-__device__ __forceinline__ void backward_step(const Xs<NROT>& x, const Cmd& cm, const Body& b, const Gains& g,
-                                              const StepParams& P, const Step<NROT>& S, Adj<NROT>& lam, GainAdj& gb,
-                                              float (&tb)[4]) {
-  constexpr int T = NROT == 4 ? 0 : (NROT == 6 ? 1 : 2);
-  const float h = P.h, hh = 0.5f * h;
-  const Q4& q = x.q;
-  // q_n = q_t / |q_t|
-  Q4 qtb;
-  {
-    const float d = S.qn.w * lam.q.w + S.qn.x * lam.q.x + S.qn.y * lam.q.y + S.qn.z * lam.q.z;
-    const float iq = S.iqtn;
-    qtb = {iq * (lam.q.w - d * S.qn.w), iq * (lam.q.x - d * S.qn.x), iq * (lam.q.y - d * S.qn.y),
-           iq * (lam.q.z - d * S.qn.z)};
-  }
-  // q_t = q + hh q (x) (0, w_n): linear in q and in w_n
-  const V3& w = S.wn;
-  Q4 qb = {qtb.w + hh * (qtb.x * w.x + qtb.y * w.y + qtb.z * w.z),
-           qtb.x + hh * (-qtb.w * w.x + qtb.y * (-w.z) + qtb.z * w.y),
-           qtb.y + hh * (-qtb.w * w.y + qtb.x * w.z - qtb.z * w.x),
-           qtb.z + hh * (-qtb.w * w.z - qtb.x * w.y + qtb.y * w.x)};
-  V3 wnb = lam.w;
-  wnb.x += hh * (-q.x * qtb.w + q.w * qtb.x + q.z * qtb.y - q.y * qtb.z);
-  wnb.y += hh * (-q.y * qtb.w - q.z * qtb.x + q.w * qtb.y + q.x * qtb.z);
-  wnb.z += hh * (-q.z * qtb.w + q.y * qtb.x - q.x * qtb.y + q.w * qtb.z);
-  // p_n = p + h v_n
-  V3 pb = lam.p;
-  V3 vnb = lam.v + h * lam.p;
-  // v_n = v + h (W.f/m b3 - (c/m) v + g)
-  const float dm = P.drag * b.inv_m;
-  V3 vb = (1.f - h * dm) * vnb;
-  const V3 b3 = {S.R[0][2], S.R[1][2], S.R[2][2]};
-  Wrench4 Wb;
-  Wb.f = h * b.inv_m * dot(b3, vnb);
-  V3 Rcb[3] = {{0.f, 0.f, 0.f}, {0.f, 0.f, 0.f}, (h * S.W.f * b.inv_m) * vnb};  // adjoints of the columns of R
-  // w_n = w + h J^-1 (W.M - gyro(w)), gyro(w) = w x (J w)
-  const V3 JW = {b.jx * x.w.x, b.jy * x.w.y, b.jz * x.w.z};
-  V3 wb = wnb;
-  const V3 jinv_wnb = {h * b.ijx * wnb.x, h * b.ijy * wnb.y, h * b.ijz * wnb.z};
-  Wb.mx = jinv_wnb.x;
-  Wb.my = jinv_wnb.y;
-  Wb.mz = jinv_wnb.z;
-  V3 gyrob = {-jinv_wnb.x, -jinv_wnb.y, -jinv_wnb.z};
-  // u_{t+1} = u + alpha (uc - u), W = A u_{t+1}
-  float ub[NROT], ucb[NROT];
-#pragma unroll
-  for (int i = 0; i < NROT; ++i) {
-    const float un_b = lam.u[i] + P.A[T][0][i] * Wb.f + P.A[T][1][i] * Wb.mx + P.A[T][2][i] * Wb.my +
-                       P.A[T][3][i] * Wb.mz;
-    ub[i] = (1.f - P.alpha) * un_b;
-    ucb[i] = S.pass[i] ? P.alpha * un_b : 0.f;
-  }
-  // pre = A^+ (f, M)
-  Wrench4 Mb = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll
-  for (int i = 0; i < NROT; ++i) {
-    Mb.f += P.Ap[T][i][0] * ucb[i];
-    Mb.mx += P.Ap[T][i][1] * ucb[i];
-    Mb.my += P.Ap[T][i][2] * ucb[i];
-    Mb.mz += P.Ap[T][i][3] * ucb[i];
-  }
-  if (MODE == kModeWrench) {
-    tb[0] += Mb.f; tb[1] += Mb.mx; tb[2] += Mb.my; tb[3] += Mb.mz;
-  } else {
-    // M = -k_R e_R - k_W e_W + gyro(w)
-    const V3 Mmb = {Mb.mx, Mb.my, Mb.mz};
-    gyrob = gyrob + Mmb;
-    const V3 eRb = {-g.kR.x * Mb.mx, -g.kR.y * Mb.my, -g.kR.z * Mb.mz};
-    const V3 eWb = {-g.kW.x * Mb.mx, -g.kW.y * Mb.my, -g.kW.z * Mb.mz};
-    gb.kR = gb.kR - V3{S.eR.x * Mb.mx, S.eR.y * Mb.my, S.eR.z * Mb.mz};
-    gb.kW = gb.kW - V3{S.eW.x * Mb.mx, S.eW.y * Mb.my, S.eW.z * Mb.mz};
-    // e_W = w - rate (R20, R21, R22)
-    wb = wb + eWb;
-    Rcb[0].z -= S.rate * eWb.x;
-    Rcb[1].z -= S.rate * eWb.y;
-    Rcb[2].z -= S.rate * eWb.z;
-    const float rateb = -(S.R[2][0] * eWb.x + S.R[2][1] * eWb.y + S.R[2][2] * eWb.z);
-    // e_R = 1/2 (E21 - E12, E02 - E20, E10 - E01), E_ij = Rd_i . R_j
-    V3 Rdb[3] = {{0.f, 0.f, 0.f}, {0.f, 0.f, 0.f}, {0.f, 0.f, 0.f}};
-    const V3 Rc[3] = {{S.R[0][0], S.R[1][0], S.R[2][0]}, {S.R[0][1], S.R[1][1], S.R[2][1]}, b3};
-    auto Eb = [&](int i, int j, float e) {  // E_ij gets adjoint e
-      Rdb[i] = Rdb[i] + e * Rc[j];
-      Rcb[j] = Rcb[j] + e * S.Rd[i];
-    };
-    Eb(2, 1, 0.5f * eRb.x); Eb(1, 2, -0.5f * eRb.x);
-    Eb(0, 2, 0.5f * eRb.y); Eb(2, 0, -0.5f * eRb.y);
-    Eb(1, 0, 0.5f * eRb.z); Eb(0, 1, -0.5f * eRb.z);
-    if (MODE == kModePosition) {
-      // f = m a . b3
-      V3 ab = (b.m * Mb.f) * b3;
-      Rcb[2] = Rcb[2] + (b.m * Mb.f) * S.a;
-      // b1d = b2d x b3d
-      V3 b2db = Rdb[1], b3db = Rdb[2];
-      cross_bwd(S.Rd[1], S.Rd[2], Rdb[0], b2db, b3db);
-      // b2d = c / |c|,  c = b3d x b1c
-      const V3 cb = normalize_bwd(S.Rd[1], S.icn, b2db);
-      V3 b1cb = {0.f, 0.f, 0.f};
-      cross_bwd(S.Rd[2], S.b1c, cb, b3db, b1cb);
-      // b3d = a / |a| (constant e3 in the degenerate case |a| = 0)
-      if (S.ian > 0.f) ab = ab + normalize_bwd(S.Rd[2], S.ian, b3db);
-      // a = -k_x (p - p_d) - k_v v + g e3
-      const V3 ex = {x.p.x - cm.t[0], x.p.y - cm.t[1], x.p.z - cm.t[2]};
-      pb = pb - V3{g.kx.x * ab.x, g.kx.y * ab.y, g.kx.z * ab.z};
-      vb = vb - V3{g.kv.x * ab.x, g.kv.y * ab.y, g.kv.z * ab.z};
-      gb.kx = gb.kx - V3{ex.x * ab.x, ex.y * ab.y, ex.z * ab.z};
-      gb.kv = gb.kv - V3{x.v.x * ab.x, x.v.y * ab.y, x.v.z * ab.z};
-      tb[0] += g.kx.x * ab.x;
-      tb[1] += g.kx.y * ab.y;
-      tb[2] += g.kx.z * ab.z;
-      // b1c = (cos psi_d, sin psi_d, 0), or (-sin psi_d, cos psi_d, 0) when turned
-      tb[3] += S.turned ? -cm.c0 * b1cb.x - cm.s0 * b1cb.y : -cm.s0 * b1cb.x + cm.c0 * b1cb.y;
-    } else {
-      // R_d = R_psi B: adjoints of B's columns and of (cos psi, sin psi)
-      V3 Bb[3];
-      float cpb = 0.f, spb = 0.f;
-#pragma unroll
-      for (int j = 0; j < 3; ++j) {
-        Bb[j] = {S.cps * Rdb[j].x + S.sps * Rdb[j].y, -S.sps * Rdb[j].x + S.cps * Rdb[j].y, Rdb[j].z};
-        cpb += Rdb[j].x * S.B[j].x + Rdb[j].y * S.B[j].y;
-        spb += -Rdb[j].x * S.B[j].y + Rdb[j].y * S.B[j].x;
-      }
-      if (MODE == kModeAttThrust) {
-        // B = R_y(theta_d) R_x(phi_d): columns (ct, 0, -st), (st sp, cp, ct sp), (st cp, -sp, ct cp)
-        const float cp = cm.c0, sp = cm.s0, ct = cm.c1, st = cm.s1;
-        const float thb = Bb[0].x * -st + Bb[0].z * -ct + Bb[1].x * (ct * sp) + Bb[1].z * (-st * sp) +
-                          Bb[2].x * (ct * cp) + Bb[2].z * (-st * cp);
-        const float phb = Bb[1].x * (st * cp) + Bb[1].y * -sp + Bb[1].z * (ct * cp) + Bb[2].x * (-st * sp) +
-                          Bb[2].y * -cp + Bb[2].z * (-ct * sp);
-        tb[0] += phb;
-        tb[1] += thb;
-        tb[2] += rateb;
-        tb[3] += Mb.f;
-      } else {
-        // f = m a . b3V, b3V = R_psi^T b3
-        const V3 b3V = {S.cps * b3.x + S.sps * b3.y, -S.sps * b3.x + S.cps * b3.y, b3.z};
-        V3 ab = (b.m * Mb.f) * b3V;
-        const V3 b3Vb = (b.m * Mb.f) * S.a;
-        Rcb[2].x += S.cps * b3Vb.x - S.sps * b3Vb.y;
-        Rcb[2].y += S.sps * b3Vb.x + S.cps * b3Vb.y;
-        Rcb[2].z += b3Vb.z;
-        cpb += b3.x * b3Vb.x + b3.y * b3Vb.y;
-        spb += b3.y * b3Vb.x - b3.x * b3Vb.y;
-        // B from a: B_2 = a/|a|, B_0 = (a_z, 0, -a_x)/|(a_x, a_z)|, B_1 = B_2 x B_0 (constant when a_x = a_z = 0)
-        if (S.irxz > 0.f) {
-          V3 B2b = Bb[2], B0b = Bb[0];
-          cross_bwd(S.B[2], S.B[0], Bb[1], B2b, B0b);
-          const V3 wbar = normalize_bwd(S.B[0], S.irxz, B0b);
-          ab.z += wbar.x;
-          ab.x -= wbar.z;
-          ab = ab + normalize_bwd(S.B[2], S.ianv, B2b);
-        }
-        // a = k_v (v_d - v^V) + g e3
-        const V3 vVb = {-g.kv.x * ab.x, -g.kv.y * ab.y, -g.kv.z * ab.z};
-        tb[0] += g.kv.x * ab.x;
-        tb[1] += g.kv.y * ab.y;
-        tb[2] += g.kv.z * ab.z;
-        gb.kv = gb.kv + V3{(cm.t[0] - S.vV.x) * ab.x, (cm.t[1] - S.vV.y) * ab.y, (cm.t[2] - S.vV.z) * ab.z};
-        // v^V = R_psi^T v
-        vb.x += S.cps * vVb.x - S.sps * vVb.y;
-        vb.y += S.sps * vVb.x + S.cps * vVb.y;
-        vb.z += vVb.z;
-        cpb += x.v.x * vVb.x + x.v.y * vVb.y;
-        spb += x.v.y * vVb.x - x.v.x * vVb.y;
-        tb[3] += rateb;
-      }
-      // (cos psi, sin psi) = (R00, R10) / |(R00, R10)|
-      if (S.ir > 0.f) {
-        const float d = S.cps * cpb + S.sps * spb;
-        Rcb[0].x += S.ir * (cpb - d * S.cps);
-        Rcb[0].y += S.ir * (spb - d * S.sps);
-      }
-    }
-  }
-  // gyro = w x (J w): w_bar += (J w) x g_bar + J (g_bar x w)
-  {
-    V3 jwb = {0.f, 0.f, 0.f};
-    cross_bwd(x.w, JW, gyrob, wb, jwb);
-    wb = wb + V3{b.jx * jwb.x, b.jy * jwb.y, b.jz * jwb.z};
-  }
-  // R = R(q), unit-quaternion formula; Rcb[j] is the adjoint of column j
-  {
-    const float w0 = q.w, x0 = q.x, y0 = q.y, z0 = q.z;
-    const float R00 = Rcb[0].x, R10 = Rcb[0].y, R20 = Rcb[0].z;
-    const float R01 = Rcb[1].x, R11 = Rcb[1].y, R21 = Rcb[1].z;
-    const float R02 = Rcb[2].x, R12 = Rcb[2].y, R22 = Rcb[2].z;
-    // R00 = 1-2(y2+z2), R01 = 2(xy-wz), R02 = 2(xz+wy), R10 = 2(xy+wz), R11 = 1-2(x2+z2),
-    // R12 = 2(yz-wx), R20 = 2(xz-wy), R21 = 2(yz+wx), R22 = 1-2(x2+y2)
-    qb.w += 2.f * (-z0 * R01 + y0 * R02 + z0 * R10 - x0 * R12 - y0 * R20 + x0 * R21);
-    qb.x += 2.f * (y0 * R01 + z0 * R02 + y0 * R10 - 2.f * x0 * R11 - w0 * R12 + z0 * R20 + w0 * R21 -
-                   2.f * x0 * R22);
-    qb.y += 2.f * (-2.f * y0 * R00 + x0 * R01 + w0 * R02 + x0 * R10 + z0 * R12 - w0 * R20 + z0 * R21 -
-                   2.f * y0 * R22);
-    qb.z += 2.f * (-2.f * z0 * R00 - w0 * R01 + x0 * R02 + w0 * R10 - 2.f * z0 * R11 + y0 * R12 + x0 * R20 +
-                   y0 * R21);
-  }
-  lam.p = pb;
-  lam.v = vb;
-  lam.q = qb;
-  lam.w = wb;
-#pragma unroll
-  for (int i = 0; i < NROT; ++i) lam.u[i] = ub[i];
+__device__ __forceinline__ void forward_step(Vehicle<NROT>& x, const Command& cm, const Body& b, const StepParams& P,
+                                             float& wf, uint32_t& pass) {
+  V3 b3;
+  const Wrench4 cmd = controller(x.s, cm, b, P, b3);
+  const Wrench4 W = allocate<NROT>(cmd, x.u, P, &pass);
+  wf = W.f;
+  step_sie<true>(x.s, b3, W, b, P.drag, P.h);
 }
 
-// ----------------------------------------------------------------- kernels --
 template <int NROT>
-__device__ __forceinline__ void load_x(const float* st, const float* mot, uint32_t n, uint32_t i, Xs<NROT>& x) {
-  x.p = {st[0 * n + i], st[1 * n + i], st[2 * n + i]};
-  x.v = {st[3 * n + i], st[4 * n + i], st[5 * n + i]};
-  x.q = {st[6 * n + i], st[7 * n + i], st[8 * n + i], st[9 * n + i]};
-  x.w = {st[10 * n + i], st[11 * n + i], st[12 * n + i]};
+__device__ __forceinline__ void load_vehicle(const float* st, const float* mot, uint32_t n, uint32_t i, Vehicle<NROT>& x) {
+  x.s.p = {st[0 * n + i], st[1 * n + i], st[2 * n + i]};
+  x.s.v = {st[3 * n + i], st[4 * n + i], st[5 * n + i]};
+  x.s.q = {st[6 * n + i], st[7 * n + i], st[8 * n + i], st[9 * n + i]};
+  x.s.w = {st[10 * n + i], st[11 * n + i], st[12 * n + i]};
 #pragma unroll
   for (int k = 0; k < NROT; ++k) x.u[k] = mot[k * n + i];
 }
 
 template <int NROT>
-__device__ __forceinline__ void store_x(float* st, float* mot, uint32_t n, uint32_t i, const Xs<NROT>& x) {
-  st[0 * n + i] = x.p.x; st[1 * n + i] = x.p.y; st[2 * n + i] = x.p.z;
-  st[3 * n + i] = x.v.x; st[4 * n + i] = x.v.y; st[5 * n + i] = x.v.z;
-  st[6 * n + i] = x.q.w; st[7 * n + i] = x.q.x; st[8 * n + i] = x.q.y; st[9 * n + i] = x.q.z;
-  st[10 * n + i] = x.w.x; st[11 * n + i] = x.w.y; st[12 * n + i] = x.w.z;
+__device__ __forceinline__ void store_vehicle(float* st, float* mot, uint32_t n, uint32_t i, const Vehicle<NROT>& x) {
+  const VState& s = x.s;
+  st[0 * n + i] = s.p.x; st[1 * n + i] = s.p.y; st[2 * n + i] = s.p.z;
+  st[3 * n + i] = s.v.x; st[4 * n + i] = s.v.y; st[5 * n + i] = s.v.z;
+  st[6 * n + i] = s.q.w; st[7 * n + i] = s.q.x; st[8 * n + i] = s.q.y; st[9 * n + i] = s.q.z;
+  st[10 * n + i] = s.w.x; st[11 * n + i] = s.w.y; st[12 * n + i] = s.w.z;
 #pragma unroll
   for (int k = 0; k < NROT; ++k) mot[k * n + i] = x.u[k];
 }
 
-__device__ __forceinline__ Body body_at(const float* bd, uint32_t n, uint32_t i) {
-  return make_body(bd[i], bd[n + i], bd[2 * n + i], bd[3 * n + i]);
+__device__ __forceinline__ Body body_at(const AdjointBuffers& ab, uint32_t i) {
+  const uint32_t n = ab.n;
+  return make_body(ab.body[i], ab.body[n + i], ab.body[2 * n + i], ab.body[3 * n + i]);
 }
 
 __device__ __forceinline__ int rotors_of(const AdjointBuffers& ab, uint32_t i) {
   return i < ab.n_quad ? 4 : (i < ab.n_quad + ab.n_hexa ? 6 : 8);
 }
 
-__device__ __forceinline__ Cmd load_cmd(const AdjointBuffers& ab, uint32_t i, int mode) {
+template <int MODE> __device__ __forceinline__ Command command_at(const AdjointBuffers& ab, uint32_t i) {
   const uint32_t n = ab.n;
-  Cmd cm;
-#pragma unroll
-  for (int k = 0; k < 4; ++k) cm.t[k] = ab.targets[k * n + i];
-  cm.c0 = 1.f; cm.s0 = 0.f; cm.c1 = 1.f; cm.s1 = 0.f;
-  if (mode == kModePosition) sincosf(cm.t[3], &cm.s0, &cm.c0);
-  if (mode == kModeAttThrust) {
-    sincosf(cm.t[0], &cm.s0, &cm.c0);
-    sincosf(cm.t[1], &cm.s1, &cm.c1);
-  }
+  Command cm = prepare_command(MODE, ab.targets[i], ab.targets[n + i], ab.targets[2 * n + i], ab.targets[3 * n + i]);
+  cm.mode = MODE;
   return cm;
 }
 
@@ -491,319 +129,533 @@ __device__ __forceinline__ int mode_of(const AdjointBuffers& ab, uint32_t i) {
   return m > kModeWrench ? kModeWrench : m;
 }
 
-// Forward recording: n_steps steps from the fleet state, checkpoint (state,
-// motors) every K steps into ckpt[s][13 + 8][n], loss per env, final state
-// written back, saturation flag per env.
-template <int NROT, int MODE>
-__device__ void record_one(const AdjointBuffers& ab, const StepParams& P, uint32_t i) {
-  const uint32_t n = ab.n;
-  Xs<NROT> x;
-  load_x(ab.state, ab.motors, n, i, x);
-  store_x(ab.ckpt, ab.ckpt + 13 * n, n, i, x);  // checkpoint 0 keeps the raw (possibly non-unit) q_0
-  normalize(x.q);
-  const Body b = body_at(ab.body, n, i);
-  const Gains g = gains_of(P);
-  const Cmd cm = load_cmd(ab, i, MODE);
-  const V3 goal = {ab.p_goal[i], ab.p_goal[n + i], ab.p_goal[2 * n + i]};
-  float loss = 0.f;
-  bool saturated = false;
-  for (int t = 0; t < ab.n_steps; ++t) {
-    if (t > 0 && t % ab.K == 0)
-      store_x(ab.ckpt + (size_t)(t / ab.K) * 21 * n, ab.ckpt + (size_t)(t / ab.K) * 21 * n + 13 * n, n, i, x);
-    Step<NROT> S;
-    Xs<NROT> xn;
-    forward_step<NROT, MODE>(x, cm, b, g, P, S, xn);
-#pragma unroll
-    for (int k = 0; k < NROT; ++k) saturated |= !S.pass[k];
-    x = xn;
-    const V3 e = x.p - goal;
-    loss += ab.w_pos * dot(e, e) + ab.w_omega * dot(x.w, x.w);
+// Calls f.template run<NROT, MODE>() for environment i's airframe and mode.
+template <int NROT, class F> __device__ __forceinline__ void by_mode(int mode, const F& f) {
+  switch (mode) {
+    case kModePosition: f.template run<NROT, kModePosition>(); break;
+    case kModeBodyVel: f.template run<NROT, kModeBodyVel>(); break;
+    case kModeAttThrust: f.template run<NROT, kModeAttThrust>(); break;
+    default: f.template run<NROT, kModeWrench>(); break;
   }
-  store_x(ab.state, ab.motors, n, i, x);
-  ab.loss[i] = loss;
-  ab.saturated[i] = saturated ? 1 : 0;
+}
+template <class F> __device__ __forceinline__ void by_airframe_and_mode(int rotors, int mode, const F& f) {
+  if (rotors == 4) by_mode<4>(mode, f);
+  else if (rotors == 6) by_mode<6>(mode, f);
+  else by_mode<8>(mode, f);
 }
 
-template <int NROT>
-__device__ __forceinline__ void record_mode(const AdjointBuffers& ab, const StepParams& P, uint32_t i) {
-  switch (mode_of(ab, i)) {
-    case kModePosition: record_one<NROT, kModePosition>(ab, P, i); break;
-    case kModeBodyVel: record_one<NROT, kModeBodyVel>(ab, P, i); break;
-    case kModeAttThrust: record_one<NROT, kModeAttThrust>(ab, P, i); break;
-    default: record_one<NROT, kModeWrench>(ab, P, i); break;
+// Forward recording of slot's environment: n_steps steps from the fleet state,
+// tape entries (FULL_TAPE) or checkpoints every K steps, loss, final state,
+// saturation flag.
+template <bool FULL_TAPE> struct Record {
+  const AdjointBuffers& ab;
+  const StepParams& P;
+  uint32_t slot, env;
+  template <int NROT, int MODE> __device__ __forceinline__ void run() const {
+    const uint32_t n = ab.n;
+    Vehicle<NROT> x;
+    load_vehicle(ab.state, ab.motors, n, env, x);
+    ab.inv_q0[slot] = 1.f / sqrtf(dot4(x.s.q));
+    normalize(x.s.q);
+    const Body b = body_at(ab, env);
+    const Command cm = command_at<MODE>(ab, env);
+    const V3 goal = {ab.p_goal[env], ab.p_goal[n + env], ab.p_goal[2 * n + env]};
+    float loss = 0.f;
+    uint32_t all_pass = (1u << NROT) - 1u;
+    float4* entry = ab.tape + slot;
+    float* ckpt = ab.ckpt;
+    int to_ckpt = 0;
+    for (int t = 0; t < ab.n_steps; ++t) {
+      if (!FULL_TAPE && to_ckpt-- == 0) {
+        store_vehicle(ckpt, ckpt + 13 * (size_t)n, n, slot, x);
+        ckpt += 21 * (size_t)n;
+        to_ckpt = ab.K - 1;
+      }
+      const VState start = x.s;
+      float wf;
+      uint32_t pass = 0;
+      forward_step<NROT, MODE>(x, cm, b, P, wf, pass);
+      all_pass &= pass;
+      if (FULL_TAPE) {
+        store_entry(entry, n, start, wf, pass);
+        entry += 4 * (size_t)n;
+      }
+      const V3 e = x.s.p - goal;
+      loss += fmaf(ab.w_omega, dot(x.s.w, x.s.w), ab.w_pos * dot(e, e));
+    }
+    if (FULL_TAPE) store_entry(entry, n, x.s, 0.f, 0u);  // entry H: the end state
+    store_vehicle(ab.state, ab.motors, n, env, x);
+    ab.loss[env] = loss;
+    ab.saturated[env] = all_pass == (1u << NROT) - 1u ? 0 : 1;
   }
-}
+};
 
 // One warp per block: the fleet's warps spread evenly over the SMs (a
 // 65,536-vehicle fleet puts 13 or 14 on each of 152 SMs, where 128-thread
-// blocks would put 12 on some and 16 on others).
+// blocks would put 12 on some and 16 on others). Writing the tape here costs
+// little beside the step: 65,536 quads x 256 steps take 192 us at 5.3 TB/s of
+// tape, against 176 us without it and another 194 us to recompute it later.
 constexpr int kRecordBlock = 32;
+template <bool FULL_TAPE>
 __global__ void __launch_bounds__(kRecordBlock) k_record(AdjointBuffers ab, StepParams P) {
-  const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= ab.n) return;
-  const int nr = rotors_of(ab, i);
-  if (nr == 4) record_mode<4>(ab, P, i);
-  else if (nr == 6) record_mode<6>(ab, P, i);
-  else record_mode<8>(ab, P, i);
+  const uint32_t slot = blockIdx.x * blockDim.x + threadIdx.x;
+  if (slot >= ab.n) return;
+  const uint32_t env = ab.order[slot];
+  by_airframe_and_mode(rotors_of(ab, env), mode_of(ab, env), Record<FULL_TAPE>{ab, P, slot, env});
 }
 
-// Adjoint state of one vehicle during the reverse sweep.
-template <int NROT> struct SweepState {
-  Adj<NROT> lam;
-  GainAdj gb;
+// ---------------------------------------------------------------- backward --
+// Adjoint state of one vehicle during the reverse sweep: of the state after a
+// step (g: the attitude's right perturbation), of the gains and the targets.
+template <int NROT> struct Adj {
+  V3 p, v, g, w;
+  float u[NROT];
+};
+struct ParamAdj {
+  V3 kx, kv, kR, kW;
   float tb[4];
 };
 
-template <int NROT> __device__ __forceinline__ void sweep_init(SweepState<NROT>& z) {
-  z.lam.p = z.lam.v = z.lam.w = {0.f, 0.f, 0.f};
-  z.lam.q = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll
-  for (int k = 0; k < NROT; ++k) z.lam.u[k] = 0.f;
-  z.gb.kx = z.gb.kv = z.gb.kR = z.gb.kW = {0.f, 0.f, 0.f};
-  z.tb[0] = z.tb[1] = z.tb[2] = z.tb[3] = 0.f;
+__device__ __forceinline__ V3 mul3(V3 a, V3 b) { return {a.x * b.x, a.y * b.y, a.z * b.z}; }
+__device__ __forceinline__ V3 fma3(float s, V3 a, V3 c) { return {fmaf(s, a.x, c.x), fmaf(s, a.y, c.y), fmaf(s, a.z, c.z)}; }
+__device__ __forceinline__ V3 fma33(V3 a, V3 b, V3 c) { return {fmaf(a.x, b.x, c.x), fmaf(a.y, b.y, c.y), fmaf(a.z, b.z, c.z)}; }
+__device__ __forceinline__ V3 neg3(V3 a) { return {-a.x, -a.y, -a.z}; }
+// c + a x b
+__device__ __forceinline__ V3 cross_add(V3 a, V3 b, V3 c) {
+  return {fmaf(a.y, b.z, fmaf(-a.z, b.y, c.x)), fmaf(a.z, b.x, fmaf(-a.x, b.z, c.y)), fmaf(a.x, b.y, fmaf(-a.y, b.x, c.z))};
+}
+// c + x_bar of y = x / |x| (1 / |x| = in): in (y_bar - y (y . y_bar))
+__device__ __forceinline__ V3 normalize_bwd_add(V3 y, float in, V3 ybar, V3 c) {
+  const float d = dot(y, ybar);
+  return fma3(in, fma3(-d, y, ybar), c);
 }
 
-// One step of the reverse sweep from its start state x: recompute the step's
-// intermediates, add the step's loss term (it acts on x_{t+1}), back-propagate.
+// Reverse of forward_step from its tape entry x and the position and body
+// rate after it. On entry z is the adjoint of (x_{t+1}, u_{t+1}) without this
+// step's loss term, on exit that of (x_t, u_t). cp2 and cw2 are 2 w_pos and
+// 2 w_omega times the environment's loss weight.
 template <int NROT, int MODE>
-__device__ __forceinline__ void sweep_step(const AdjointBuffers& ab, const StepParams& P, const Xs<NROT>& x,
-                                           const Cmd& cm, const Body& b, const Gains& g, V3 goal, float wgt,
-                                           SweepState<NROT>& z) {
-  Step<NROT> S;
-  Xs<NROT> xn;
-  forward_step<NROT, MODE>(x, cm, b, g, P, S, xn);
-  const V3 e = xn.p - goal;
-  z.lam.p = z.lam.p + (2.f * ab.w_pos * wgt) * e;
-  z.lam.w = z.lam.w + (2.f * ab.w_omega * wgt) * xn.w;
-  backward_step<NROT, MODE>(x, cm, b, g, P, S, z.lam, z.gb, z.tb);
-}
-
-// Writes vehicle i's gradients. The kernel normalised q_0 at load
-// (q_hat = q0 / |q0|), so the quaternion adjoint is mapped back through that.
-template <int NROT>
-__device__ __forceinline__ void sweep_finish(const AdjointBuffers& ab, uint32_t i, SweepState<NROT>& z) {
-  const uint32_t n = ab.n;
-  Adj<NROT>& lam = z.lam;
+__device__ __forceinline__ void backward_step(const TapeStep& x, V3 pn, V3 wn, const Command& cm, const Body& b,
+                                              const StepParams& P, V3 goal, float cp2, float cw2, Adj<NROT>& z,
+                                              ParamAdj& gb) {
+  constexpr int T = NROT == 4 ? 0 : (NROT == 6 ? 1 : 2);
+  const float h = P.h;
+  // the loss term of x_{t+1}
+  const V3 pb = fma3(cp2, pn - goal, z.p);
+  V3 wb = fma3(cw2, wn, z.w);
+  // q' = q (1, hw) / s with hw = h/2 Omega', s^2 = 1 + |hw|^2:
+  // Omega'_bar += h / s^2 (g + hw x g), g <- R(c) g = g + 2 / s^2 (hw x g + hw x (hw x g))
+  const V3 hw = (0.5f * h) * wn;
+  const float is2 = rcp_ftz(fmaf(hw.z, hw.z, fmaf(hw.y, hw.y, fmaf(hw.x, hw.x, 1.f))));
+  const V3 t1 = cross(hw, z.g);
+  wb = fma3(h * is2, z.g + t1, wb);  // now the adjoint of Omega' (and of Omega through Omega' = Omega + ...)
+  V3 g = fma3(2.f * is2, cross_add(hw, t1, t1), z.g);
+  // p' = p + h v';  v' = v + h (W.f/m b3 - (c/m) v + g e3)
+  const V3 vnb = fma3(h, pb, z.v);
+  const float him = h * b.inv_m;
+  V3 vb = fmaf(-him, P.drag, 1.f) * vnb;
+  float R[3][3];
+  rotation(x.q, R);
+  const V3 r0 = {R[0][0], R[1][0], R[2][0]}, r1 = {R[0][1], R[1][1], R[2][1]}, r2 = {R[0][2], R[1][2], R[2][2]};
+  const float Wfb = him * dot(r2, vnb);
+  V3 tilt = (him * x.wf) * vnb;  // world adjoint of b3: g gets e3 x (R^T tilt) once all its terms are in
+  // Omega' = Omega + h J^-1 (W.M - gyro)
+  const V3 wmb = {(h * b.ijx) * wb.x, (h * b.ijy) * wb.y, (h * b.ijz) * wb.z};
+  // u' = u + alpha (clamp(A^+ (f, M)) - u), W = A u': motors as FP32 pairs, the commanded wrench's adjoint as
+  // (f, M_x) and (M_y, M_z)
+  float2 Ma = make_float2(0.f, 0.f), Mc = make_float2(0.f, 0.f);
   {
-    const Q4 q0 = {ab.ckpt[6 * n + i], ab.ckpt[7 * n + i], ab.ckpt[8 * n + i], ab.ckpt[9 * n + i]};
-    const float nq = sqrtf(q0.w * q0.w + q0.x * q0.x + q0.y * q0.y + q0.z * q0.z);
-    const Q4 qh = {q0.w / nq, q0.x / nq, q0.y / nq, q0.z / nq};
-    const float d = qh.w * lam.q.w + qh.x * lam.q.x + qh.y * lam.q.y + qh.z * lam.q.z;
-    lam.q = {(lam.q.w - d * qh.w) / nq, (lam.q.x - d * qh.x) / nq, (lam.q.y - d * qh.y) / nq,
-             (lam.q.z - d * qh.z) / nq};
-  }
-  float* gx = ab.grad_x0;
-  gx[0 * n + i] = lam.p.x; gx[1 * n + i] = lam.p.y; gx[2 * n + i] = lam.p.z;
-  gx[3 * n + i] = lam.v.x; gx[4 * n + i] = lam.v.y; gx[5 * n + i] = lam.v.z;
-  gx[6 * n + i] = lam.q.w; gx[7 * n + i] = lam.q.x; gx[8 * n + i] = lam.q.y; gx[9 * n + i] = lam.q.z;
-  gx[10 * n + i] = lam.w.x; gx[11 * n + i] = lam.w.y; gx[12 * n + i] = lam.w.z;
-  float* gg = ab.grad_gains_env;
-  const GainAdj& gb = z.gb;
-  const float v12[12] = {gb.kx.x, gb.kx.y, gb.kx.z, gb.kv.x, gb.kv.y, gb.kv.z,
-                         gb.kR.x, gb.kR.y, gb.kR.z, gb.kW.x, gb.kW.y, gb.kW.z};
+    const float2 f2 = make_float2(Wfb, Wfb), x2 = make_float2(wmb.x, wmb.x), y2 = make_float2(wmb.y, wmb.y),
+                 z2 = make_float2(wmb.z, wmb.z), keep2 = make_float2(1.f - P.alpha, 1.f - P.alpha),
+                 al2 = make_float2(P.alpha, P.alpha);
 #pragma unroll
-  for (int k = 0; k < 12; ++k) gg[k * n + i] = v12[k];
-#pragma unroll
-  for (int k = 0; k < 4; ++k) ab.grad_targets[k * n + i] = z.tb[k];
-}
-
-template <int NROT>
-__device__ __forceinline__ float* tape_at(const AdjointBuffers& ab, int t) {
-  return ab.tape + (size_t)t * 21 * ab.n;
-}
-
-// Reverse sweep of vehicle i. full_tape: every step-start state is already on
-// the tape (k_tape); otherwise each segment's states are recomputed here,
-// segment by segment, into the one-segment tape.
-template <int NROT, int MODE, bool FULL_TAPE>
-__device__ void adjoint_one(const AdjointBuffers& ab, const StepParams& P, uint32_t i) {
-  const uint32_t n = ab.n;
-  const Body b = body_at(ab.body, n, i);
-  const Gains g = gains_of(P);
-  const Cmd cm = load_cmd(ab, i, MODE);
-  const V3 goal = {ab.p_goal[i], ab.p_goal[n + i], ab.p_goal[2 * n + i]};
-  const float wgt = ab.loss_weights ? ab.loss_weights[i] : 1.f;
-  SweepState<NROT> z;
-  sweep_init(z);
-  const int H = ab.n_steps, K = ab.K;
-  if (FULL_TAPE) {
-    // the next (earlier) tape entry is requested one step ahead
-    Xs<NROT> x, x_prev;
-    load_x(tape_at<NROT>(ab, H - 1), tape_at<NROT>(ab, H - 1) + 13 * n, n, i, x_prev);
-    for (int t = H - 1; t >= 0; --t) {
-      x = x_prev;
-      if (t > 0) load_x(tape_at<NROT>(ab, t - 1), tape_at<NROT>(ab, t - 1) + 13 * n, n, i, x_prev);
-      sweep_step<NROT, MODE>(ab, P, x, cm, b, g, goal, wgt, z);
+    for (int j = 0; j < NROT / 2; ++j) {
+      const int i = 2 * j;
+      float2 un = make_float2(z.u[i], z.u[i + 1]);
+      un = __ffma2_rn(make_float2(P.A[T][0][i], P.A[T][0][i + 1]), f2, un);
+      un = __ffma2_rn(make_float2(P.A[T][1][i], P.A[T][1][i + 1]), x2, un);
+      un = __ffma2_rn(make_float2(P.A[T][2][i], P.A[T][2][i + 1]), y2, un);
+      un = __ffma2_rn(make_float2(P.A[T][3][i], P.A[T][3][i + 1]), z2, un);
+      const float2 k = __fmul2_rn(keep2, un);
+      z.u[i] = k.x;
+      z.u[i + 1] = k.y;
+      float2 c = __fmul2_rn(al2, un);
+      c.x = (x.pass >> i) & 1u ? c.x : 0.f;
+      c.y = (x.pass >> (i + 1)) & 1u ? c.y : 0.f;
+      const float2 cx = make_float2(c.x, c.x), cy = make_float2(c.y, c.y);
+      Ma = __ffma2_rn(make_float2(P.Ap[T][i][0], P.Ap[T][i][1]), cx, Ma);
+      Mc = __ffma2_rn(make_float2(P.Ap[T][i][2], P.Ap[T][i][3]), cx, Mc);
+      Ma = __ffma2_rn(make_float2(P.Ap[T][i + 1][0], P.Ap[T][i + 1][1]), cy, Ma);
+      Mc = __ffma2_rn(make_float2(P.Ap[T][i + 1][2], P.Ap[T][i + 1][3]), cy, Mc);
     }
-    sweep_finish(ab, i, z);
-    return;
   }
-  const int n_seg = (H + K - 1) / K;
-  for (int seg = n_seg - 1; seg >= 0; --seg) {
-    const int t0 = seg * K;
-    const int len = H - t0 < K ? H - t0 : K;
-    Xs<NROT> x;
-    load_x(ab.ckpt + (size_t)seg * 21 * n, ab.ckpt + (size_t)seg * 21 * n + 13 * n, n, i, x);
-    if (seg == 0) normalize(x.q);
-    // recompute the segment's step-start states into the tape
-    for (int t = 0; t < len; ++t) {
-      store_x(tape_at<NROT>(ab, t), tape_at<NROT>(ab, t) + 13 * n, n, i, x);
-      if (t + 1 < len) {
-        Step<NROT> S;
-        Xs<NROT> xn;
-        forward_step<NROT, MODE>(x, cm, b, g, P, S, xn);
-        x = xn;
+  const float Mf = Ma.x;
+  const V3 Mm = {Ma.y, Mc.x, Mc.y};
+  V3 gyrob = neg3(wmb);
+  z.p = pb;
+  if (MODE == kModeWrench) {
+    gb.tb[0] += Mf; gb.tb[1] += Mm.x; gb.tb[2] += Mm.y; gb.tb[3] += Mm.z;
+  } else {
+    const V3 kx = {P.kx[0], P.kx[1], P.kx[2]}, kv = {P.kv[0], P.kv[1], P.kv[2]};
+    // the step's R_d, commanded yaw rate and their intermediates, as controller() forms them
+    V3 rd0, rd1, rd2, a, ex, B0, B1, B2, vV;
+    float ian = 0.f, icn = 0.f, irxz = 0.f, rate = 0.f, hc = 1.f, hs = 0.f, cps = 1.f, sps = 0.f, ir = 0.f;
+    bool turned = false;
+    if (MODE == kModePosition) {
+      ex = {x.p.x - cm.c[0], x.p.y - cm.c[1], x.p.z - cm.c[2]};
+      a = {fmaf(-kx.x, ex.x, -(kv.x * x.v.x)), fmaf(-kx.y, ex.y, -(kv.y * x.v.y)),
+           fmaf(-kx.z, ex.z, fmaf(-kv.z, x.v.z, kGravity))};
+      const float a2 = dot(a, a);
+      ian = a2 > 1e-18f ? rsqrt_ftz(a2) : 0.f;
+      rd2 = ian > 0.f ? ian * a : V3{0.f, 0.f, 1.f};
+      hc = cm.c[3];
+      hs = cm.c[4];
+      V3 c = cross_xy(rd2, hc, hs);
+      float c2 = dot(c, c);
+      turned = !(c2 > 1e-18f);
+      if (turned) {
+        hc = -cm.c[4];
+        hs = cm.c[3];
+        c = cross_xy(rd2, hc, hs);
+        c2 = dot(c, c);
+      }
+      icn = rsqrt_ftz(c2);
+      rd1 = icn * c;
+      rd0 = cross(rd1, rd2);
+    } else {
+      const float rho2 = fmaf(r0.y, r0.y, r0.x * r0.x);
+      if (rho2 >= kMinNormal) {
+        ir = rsqrt_ftz(rho2);
+        cps = r0.x * ir;
+        sps = r0.y * ir;
+      }
+      float cphi, sphi, cth, sth;
+      if (MODE == kModeBodyVel) {
+        vV = {fmaf(sps, x.v.y, cps * x.v.x), fmaf(cps, x.v.y, -(sps * x.v.x)), x.v.z};
+        a = {kv.x * (cm.c[0] - vV.x), kv.y * (cm.c[1] - vV.y), fmaf(kv.z, cm.c[2] - vV.z, kGravity)};
+        const float rxz2 = fmaf(a.z, a.z, a.x * a.x);
+        const float an2 = fmaf(a.y, a.y, rxz2);
+        cphi = 1.f; sphi = 0.f; cth = 1.f; sth = 0.f;
+        if (rxz2 >= kMinNormal) {
+          irxz = rsqrt_ftz(rxz2);
+          ian = rsqrt_ftz(an2);
+          cth = a.z * irxz;
+          sth = a.x * irxz;
+          cphi = rxz2 * irxz * ian;
+          sphi = -a.y * ian;
+        } else if (an2 > 0.f) {
+          cphi = 0.f;
+          sphi = a.y > 0.f ? -1.f : 1.f;
+        }
+        rate = cm.c[3];
+      } else {
+        cphi = cm.c[0]; sphi = cm.c[1]; cth = cm.c[2]; sth = cm.c[3]; rate = cm.c[4];
+      }
+      // columns of R_y(theta_d) R_x(phi_d), then R_d = R_psi times them
+      B0 = {cth, 0.f, -sth};
+      B1 = {sth * sphi, cphi, cth * sphi};
+      B2 = {sth * cphi, -sphi, cth * cphi};
+      rd0 = {cps * B0.x, sps * B0.x, B0.z};
+      rd1 = {fmaf(cps, B1.x, -(sps * B1.y)), fmaf(sps, B1.x, cps * B1.y), B1.z};
+      rd2 = {fmaf(cps, B2.x, -(sps * B2.y)), fmaf(sps, B2.x, cps * B2.y), B2.z};
+    }
+    // M = -k_R e_R - k_W e_W + gyro(Omega), e_W = Omega - rate R^T e3, 2 e_R = vee(E - E^T), E = R_d^T R
+    gyrob = gyrob + Mm;
+    const V3 eWb = {-P.kW[0] * Mm.x, -P.kW[1] * Mm.y, -P.kW[2] * Mm.z};
+    const V3 eb = {-0.5f * P.kR[0] * Mm.x, -0.5f * P.kR[1] * Mm.y, -0.5f * P.kR[2] * Mm.z};  // of 2 e_R
+    const float E00 = dot(rd0, r0), E01 = dot(rd0, r1), E02 = dot(rd0, r2);
+    const float E10 = dot(rd1, r0), E11 = dot(rd1, r1), E12 = dot(rd1, r2);
+    const float E20 = dot(rd2, r0), E21 = dot(rd2, r1), E22 = dot(rd2, r2);
+    const V3 hm = 0.5f * Mm;
+    gb.kR = {fmaf(E12 - E21, hm.x, gb.kR.x), fmaf(E20 - E02, hm.y, gb.kR.y), fmaf(E01 - E10, hm.z, gb.kR.z)};
+    V3 eW = x.w;
+    if (MODE != kModePosition) eW = {fmaf(-rate, R[2][0], x.w.x), fmaf(-rate, R[2][1], x.w.y), fmaf(-rate, R[2][2], x.w.z)};
+    gb.kW = {fmaf(-eW.x, Mm.x, gb.kW.x), fmaf(-eW.y, Mm.y, gb.kW.y), fmaf(-eW.z, Mm.z, gb.kW.z)};
+    wb = wb + eWb;
+    // g += (tr(E) I - E) eb
+    g.x = fmaf(E11 + E22, eb.x, fmaf(-E01, eb.y, fmaf(-E02, eb.z, g.x)));
+    g.y = fmaf(E00 + E22, eb.y, fmaf(-E10, eb.x, fmaf(-E12, eb.z, g.y)));
+    g.z = fmaf(E00 + E11, eb.z, fmaf(-E20, eb.x, fmaf(-E21, eb.y, g.z)));
+    // columns of R_d: r_j with the adjoints of E_ij - E_ji
+    V3 rd0b = fma3(eb.y, r2, (-eb.z) * r1), rd1b = fma3(eb.z, r0, (-eb.x) * r2), rd2b = fma3(eb.x, r1, (-eb.y) * r0);
+    const float mf = b.m * Mf;
+    if (MODE == kModePosition) {
+      // f = m a . b3
+      V3 ab = mf * r2;
+      tilt = fma3(mf, a, tilt);
+      // b1d = b2d x b3d;  b2d = c / |c|, c = b3d x b1c;  b3d = a / |a| (constant e3 where |a| = 0)
+      rd1b = cross_add(rd2, rd0b, rd1b);
+      rd2b = cross_add(rd0b, rd1, rd2b);
+      const float d = dot(rd1, rd1b);
+      const V3 cb = icn * fma3(-d, rd1, rd1b);
+      rd2b = {fmaf(hs, cb.z, rd2b.x), fmaf(-hc, cb.z, rd2b.y), fmaf(hc, cb.y, fmaf(-hs, cb.x, rd2b.z))};
+      const float hcb = fmaf(cb.y, rd2.z, -(cb.z * rd2.y)), hsb = fmaf(cb.z, rd2.x, -(cb.x * rd2.z));
+      if (ian > 0.f) ab = normalize_bwd_add(rd2, ian, rd2b, ab);
+      // a = -k_x (p - p_d) - k_v v + g e3
+      const V3 xa = mul3(kx, ab);
+      z.p = z.p - xa;
+      vb = fma33(neg3(kv), ab, vb);
+      gb.kx = fma33(neg3(ex), ab, gb.kx);
+      gb.kv = fma33(neg3(x.v), ab, gb.kv);
+      gb.tb[0] += xa.x;
+      gb.tb[1] += xa.y;
+      gb.tb[2] += xa.z;
+      // b1c = (cos psi_d, sin psi_d, 0), turned by 90 degrees in the fallback: d b1c / d psi_d = (-hs, hc, 0) in both
+      gb.tb[3] = fmaf(-hs, hcb, fmaf(hc, hsb, gb.tb[3]));
+    } else {
+      // e_W's third row of R: g -= rate (eWb x R^T e3)
+      const V3 row = {R[2][0], R[2][1], R[2][2]};
+      const float rateb = -dot(row, eWb);
+      g = cross_add(rate * row, eWb, g);
+      // R_d = R_psi B: adjoints of B's columns and of (cos psi, sin psi)
+      const V3 B0b = {fmaf(sps, rd0b.y, cps * rd0b.x), fmaf(cps, rd0b.y, -(sps * rd0b.x)), rd0b.z};
+      const V3 B1b = {fmaf(sps, rd1b.y, cps * rd1b.x), fmaf(cps, rd1b.y, -(sps * rd1b.x)), rd1b.z};
+      const V3 B2b = {fmaf(sps, rd2b.y, cps * rd2b.x), fmaf(cps, rd2b.y, -(sps * rd2b.x)), rd2b.z};
+      float cpb = fmaf(rd2b.y, B2.y, fmaf(rd2b.x, B2.x, fmaf(rd1b.y, B1.y, fmaf(rd1b.x, B1.x, rd0b.x * B0.x))));
+      float spb = fmaf(rd2b.y, B2.x, fmaf(-rd2b.x, B2.y, fmaf(rd1b.y, B1.x, fmaf(-rd1b.x, B1.y, rd0b.y * B0.x))));
+      if (MODE == kModeAttThrust) {
+        // B = R_y(theta_d) R_x(phi_d): columns (ct, 0, -st), (st sp, cp, ct sp), (st cp, -sp, ct cp)
+        const float cp = cm.c[0], sp = cm.c[1], ct = cm.c[2], st = cm.c[3];
+        const float u1 = fmaf(ct, B1b.x, -(st * B1b.z)), u2 = fmaf(ct, B2b.x, -(st * B2b.z));
+        const float v1 = fmaf(st, B1b.x, ct * B1b.z), v2 = fmaf(st, B2b.x, ct * B2b.z);
+        gb.tb[1] += fmaf(-st, B0b.x, fmaf(-ct, B0b.z, fmaf(sp, u1, cp * u2)));
+        gb.tb[0] += fmaf(cp, v1 - B2b.y, -(sp * (v2 + B1b.y)));
+        gb.tb[2] += rateb;
+        gb.tb[3] += Mf;
+      } else {
+        // f = m a . (R_psi^T b3)
+        const V3 b3V = {fmaf(sps, r2.y, cps * r2.x), fmaf(cps, r2.y, -(sps * r2.x)), r2.z};
+        V3 ab = mf * b3V;
+        const V3 fb = mf * a;
+        tilt = {tilt.x + fmaf(cps, fb.x, -(sps * fb.y)), tilt.y + fmaf(sps, fb.x, cps * fb.y), tilt.z + fb.z};
+        cpb = fmaf(r2.x, fb.x, fmaf(r2.y, fb.y, cpb));
+        spb = fmaf(r2.y, fb.x, fmaf(-r2.x, fb.y, spb));
+        // B from a: B2 = a / |a|, B0 = (a_z, 0, -a_x) / |(a_x, a_z)|, B1 = B2 x B0 (constant when a_x = a_z = 0)
+        if (irxz > 0.f) {
+          const V3 B2c = cross_add(B0, B1b, B2b), B0c = cross_add(B1b, B2, B0b);
+          const float d = fmaf(B0.z, B0c.z, B0.x * B0c.x);
+          ab.z = fmaf(irxz, fmaf(-d, B0.x, B0c.x), ab.z);
+          ab.x = fmaf(-irxz, fmaf(-d, B0.z, B0c.z), ab.x);
+          ab = normalize_bwd_add(B2, ian, B2c, ab);
+        }
+        // a = k_v (v_d - v^V) + g e3,  v^V = R_psi^T v
+        const V3 tv = mul3(kv, ab);
+        gb.tb[0] += tv.x;
+        gb.tb[1] += tv.y;
+        gb.tb[2] += tv.z;
+        gb.tb[3] += rateb;
+        gb.kv = fma33(V3{cm.c[0] - vV.x, cm.c[1] - vV.y, cm.c[2] - vV.z}, ab, gb.kv);
+        vb = {vb.x - fmaf(cps, tv.x, -(sps * tv.y)), vb.y - fmaf(sps, tv.x, cps * tv.y), vb.z - tv.z};
+        cpb = fmaf(-x.v.x, tv.x, fmaf(-x.v.y, tv.y, cpb));
+        spb = fmaf(-x.v.y, tv.x, fmaf(x.v.x, tv.y, spb));
+      }
+      // (cos psi, sin psi) = (R00, R10) / |(R00, R10)|; ir = 0 where R00 = R10 = 0
+      const float d = fmaf(sps, spb, cps * cpb);
+      const float c0 = ir * fmaf(-d, cps, cpb), c1 = ir * fmaf(-d, sps, spb);  // adjoint of (R00, R10)
+      g.y = fmaf(-r2.x, c0, fmaf(-r2.y, c1, g.y));
+      g.z = fmaf(r1.x, c0, fmaf(r1.y, c1, g.z));
+    }
+  }
+  // b3 = R e3: g += e3 x (R^T tilt)
+  g.x -= dot(r1, tilt);
+  g.y += dot(r0, tilt);
+  // gyro = (gx wy wz, gy wz wx, gz wx wy)
+  const V3 gg = {b.gx * gyrob.x, b.gy * gyrob.y, b.gz * gyrob.z};
+  z.w = {fmaf(gg.y, x.w.z, fmaf(gg.z, x.w.y, wb.x)), fmaf(gg.x, x.w.z, fmaf(gg.z, x.w.x, wb.y)),
+         fmaf(gg.x, x.w.y, fmaf(gg.y, x.w.x, wb.z))};
+  z.v = vb;
+  z.g = g;
+}
+
+// Tape entries in flight per vehicle: the sweep's loads run this many steps
+// ahead of their use, asynchronously into shared memory (each thread copies
+// and reads its own column, so there is nothing to synchronise between threads).
+constexpr int kSweepStages = 4;
+constexpr int kAdjointBlock = 32;
+
+__device__ __forceinline__ void copy16_async(float4* dst_shared, const float4* src) {
+  const uint32_t d = (uint32_t)__cvta_generic_to_shared(dst_shared);
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(d), "l"(src) : "memory");
+}
+
+// Reverse sweep of slot's environment; the gain adjoints are returned in gb.
+template <bool FULL_TAPE> struct Sweep {
+  const AdjointBuffers& ab;
+  const StepParams& P;
+  uint32_t slot, env;
+  float4 (*ring)[4][kAdjointBlock];  // [kSweepStages][4][lane]
+  V3 (&gains)[4];
+  template <int NROT, int MODE> __device__ __forceinline__ void run() const {
+    const size_t n = ab.n;
+    const uint32_t lane = threadIdx.x;
+    const Body b = body_at(ab, env);
+    const Command cm = command_at<MODE>(ab, env);
+    const V3 goal = {ab.p_goal[env], ab.p_goal[n + env], ab.p_goal[2 * n + env]};
+    const float wgt = ab.loss_weights ? ab.loss_weights[env] : 1.f;
+    const float cp2 = 2.f * ab.w_pos * wgt, cw2 = 2.f * ab.w_omega * wgt;
+    Adj<NROT> z;
+    z.p = z.v = z.g = z.w = {0.f, 0.f, 0.f};
+#pragma unroll
+    for (int k = 0; k < NROT; ++k) z.u[k] = 0.f;
+    ParamAdj gb;
+    gb.kx = gb.kv = gb.kR = gb.kW = {0.f, 0.f, 0.f};
+    gb.tb[0] = gb.tb[1] = gb.tb[2] = gb.tb[3] = 0.f;
+    const int H = ab.n_steps;
+    V3 pn, wn;        // position and body rate after the step in hand
+    Q4 q0;            // unit attitude at step 0
+    const size_t row = 4 * n;
+    if (FULL_TAPE) {
+      const float4* const tape = ab.tape + slot;
+      {
+        const float4* e = tape + (size_t)H * row;
+        const float4 e0 = e[0], e1 = e[n], e3 = e[3 * n];
+        pn = {e0.x, e0.y, e0.z};
+        wn = {e1.z, e1.w, e3.x};
+      }
+      auto request = [&](int t) {  // a group per step, empty before the first
+        if (t >= 0) {
+          const float4* e = tape + (size_t)t * row;
+#pragma unroll
+          for (int r = 0; r < 4; ++r) copy16_async(&ring[t % kSweepStages][r][lane], e + r * n);
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+      };
+#pragma unroll
+      for (int k = 1; k < kSweepStages; ++k) request(H - k);
+      for (int t = H - 1; t >= 0; --t) {
+        request(t - (kSweepStages - 1));
+        asm volatile("cp.async.wait_group %0;" ::"n"(kSweepStages - 1) : "memory");
+        const float4(*e)[kAdjointBlock] = ring[t % kSweepStages];
+        const TapeStep x = unpack(e[0][lane], e[1][lane], e[2][lane], e[3][lane]);
+        backward_step<NROT, MODE>(x, pn, wn, cm, b, P, goal, cp2, cw2, z, gb);
+        pn = x.p;
+        wn = x.w;
+        q0 = x.q;
+      }
+    } else {
+      const int K = ab.K;
+      for (int seg = (H + K - 1) / K - 1; seg >= 0; --seg) {
+        const int t0 = seg * K, len = H - t0 < K ? H - t0 : K;
+        float4* const tape = ab.tape + slot;
+        Vehicle<NROT> v;
+        const float* ck = ab.ckpt + (size_t)seg * 21 * n;
+        load_vehicle(ck, ck + 13 * n, (uint32_t)n, slot, v);
+        for (int t = 0; t < len; ++t) {
+          const VState start = v.s;
+          float wf;
+          uint32_t pass = 0;
+          forward_step<NROT, MODE>(v, cm, b, P, wf, pass);
+          store_entry(tape + (size_t)t * row, n, start, wf, pass);
+        }
+        if (t0 + len == H) {  // the later segments' first entries carry pn and wn across the others
+          pn = v.s.p;
+          wn = v.s.w;
+        }
+        for (int t = len - 1; t >= 0; --t) {
+          const float4* e = tape + (size_t)t * row;
+          const TapeStep x = unpack(e[0], e[n], e[2 * n], e[3 * n]);
+          backward_step<NROT, MODE>(x, pn, wn, cm, b, P, goal, cp2, cw2, z, gb);
+          pn = x.p;
+          wn = x.w;
+          q0 = x.q;
+        }
       }
     }
-    // reverse sweep; the next (earlier) tape entry is requested one step ahead
-    Xs<NROT> x_prev;
-    load_x(tape_at<NROT>(ab, len - 1), tape_at<NROT>(ab, len - 1) + 13 * n, n, i, x_prev);
-    for (int t = len - 1; t >= 0; --t) {
-      x = x_prev;
-      if (t > 0) load_x(tape_at<NROT>(ab, t - 1), tape_at<NROT>(ab, t - 1) + 13 * n, n, i, x_prev);
-      sweep_step<NROT, MODE>(ab, P, x, cm, b, g, goal, wgt, z);
+    // the rollout started from q_0 / |q_0|: the adjoint of q_0 is 2 q (0, g) / |q_0|
+    const float s = 2.f * ab.inv_q0[slot];
+    const Q4 qb = quat_rate2(q0, z.g);
+    if (ab.grad_x0) {
+      float* gx = ab.grad_x0 + env;
+      const float v13[13] = {z.p.x, z.p.y, z.p.z, z.v.x, z.v.y, z.v.z, s * qb.w, s * qb.x, s * qb.y, s * qb.z,
+                             z.w.x, z.w.y, z.w.z};
+#pragma unroll
+      for (int k = 0; k < 13; ++k) gx[k * n] = v13[k];
     }
-  }
-  sweep_finish(ab, i, z);
-}
-
-// Step-start states of one segment of vehicle i, recomputed from its
-// checkpoint into the whole-horizon tape (tape step t0 + t, t < len).
-template <int NROT, int MODE>
-__device__ void tape_one(const AdjointBuffers& ab, const StepParams& P, uint32_t i, int seg) {
-  const uint32_t n = ab.n;
-  const int t0 = seg * ab.K;
-  const int len = ab.n_steps - t0 < ab.K ? ab.n_steps - t0 : ab.K;
-  const Body b = body_at(ab.body, n, i);
-  const Gains g = gains_of(P);
-  const Cmd cm = load_cmd(ab, i, MODE);
-  Xs<NROT> x;
-  load_x(ab.ckpt + (size_t)seg * 21 * n, ab.ckpt + (size_t)seg * 21 * n + 13 * n, n, i, x);
-  if (seg == 0) normalize(x.q);
-  for (int t = 0; t < len; ++t) {
-    store_x(tape_at<NROT>(ab, t0 + t), tape_at<NROT>(ab, t0 + t) + 13 * n, n, i, x);
-    if (t + 1 < len) {
-      Step<NROT> S;
-      Xs<NROT> xn;
-      forward_step<NROT, MODE>(x, cm, b, g, P, S, xn);
-      x = xn;
+    if (ab.grad_gains_env) {
+      float* gg = ab.grad_gains_env + env;
+      const float v12[12] = {gb.kx.x, gb.kx.y, gb.kx.z, gb.kv.x, gb.kv.y, gb.kv.z,
+                             gb.kR.x, gb.kR.y, gb.kR.z, gb.kW.x, gb.kW.y, gb.kW.z};
+#pragma unroll
+      for (int k = 0; k < 12; ++k) gg[k * n] = v12[k];
     }
+    if (ab.grad_targets) {
+#pragma unroll
+      for (int k = 0; k < 4; ++k) ab.grad_targets[k * n + env] = gb.tb[k];
+    }
+    gains[0] = gb.kx;
+    gains[1] = gb.kv;
+    gains[2] = gb.kR;
+    gains[3] = gb.kW;
   }
-}
+};
 
-template <int NROT>
-__device__ __forceinline__ void tape_mode(const AdjointBuffers& ab, const StepParams& P, uint32_t i, int seg) {
-  switch (mode_of(ab, i)) {
-    case kModePosition: tape_one<NROT, kModePosition>(ab, P, i, seg); break;
-    case kModeBodyVel: tape_one<NROT, kModeBodyVel>(ab, P, i, seg); break;
-    case kModeAttThrust: tape_one<NROT, kModeAttThrust>(ab, P, i, seg); break;
-    default: tape_one<NROT, kModeWrench>(ab, P, i, seg); break;
-  }
-}
-
-// One thread per (vehicle, segment): thread j handles vehicle j % n of
-// segment j / n, so a warp's loads and stores stay coalesced.
-constexpr int kTapeBlock = 128;
-__global__ void __launch_bounds__(kTapeBlock) k_tape(AdjointBuffers ab, StepParams P, int n_seg) {
-  const uint64_t j = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (j >= (uint64_t)ab.n * n_seg) return;
-  const uint32_t i = (uint32_t)(j % ab.n);
-  const int seg = (int)(j / ab.n);
-  const int nr = rotors_of(ab, i);
-  if (nr == 4) tape_mode<4>(ab, P, i, seg);
-  else if (nr == 6) tape_mode<6>(ab, P, i, seg);
-  else tape_mode<8>(ab, P, i, seg);
-}
-
-template <int NROT, bool FULL_TAPE>
-__device__ __forceinline__ void adjoint_mode(const AdjointBuffers& ab, const StepParams& P, uint32_t i) {
-  switch (mode_of(ab, i)) {
-    case kModePosition: adjoint_one<NROT, kModePosition, FULL_TAPE>(ab, P, i); break;
-    case kModeBodyVel: adjoint_one<NROT, kModeBodyVel, FULL_TAPE>(ab, P, i); break;
-    case kModeAttThrust: adjoint_one<NROT, kModeAttThrust, FULL_TAPE>(ab, P, i); break;
-    default: adjoint_one<NROT, kModeWrench, FULL_TAPE>(ab, P, i); break;
-  }
-}
-
-// One warp per block and at most 128 registers. Each SM sub-partition holds a
-// quarter of the register file: 128 registers fit four warps per
+// One warp per block and at most 128 registers: four warps fit per SM
 // sub-partition, 16 per SM, so a 65,536-vehicle fleet (2,048 warps) is
-// resident in one wave on 152 SMs, and single-warp blocks spread the warps
-// evenly (13 or 14 per SM). The sweep wants about 168 registers, and the cap
-// spills about 1.3 KB per thread; at 144 registers (12 warps per SM) the
-// fleet needed 1.12 waves, which cost more than the spills do.
-constexpr int kAdjointBlock = 32;
+// resident in one wave on 152 SMs; nothing spills. Bound by instruction issue
+// (75 % of cycles, and the sub-partitions that hold four warps, not three,
+// finish last); the tape leaves DRAM at half its rate. 65,536 quads x 256
+// steps: 262 us for 206 M warp instructions, against 501 us for 365 M (and
+// 194 us for a launch that recomputed the tape) when the sweep rebuilt the
+// whole step and carried the adjoints of q and R.
+// The warp's sum of each gain's adjoint (a fixed tree over its lanes) goes to
+// partial[gain][warp].
 template <bool FULL_TAPE>
 __global__ void __maxnreg__(128) k_adjoint(AdjointBuffers ab, StepParams P) {
-  const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= ab.n) return;
-  const int nr = rotors_of(ab, i);
-  if (nr == 4) adjoint_mode<4, FULL_TAPE>(ab, P, i);
-  else if (nr == 6) adjoint_mode<6, FULL_TAPE>(ab, P, i);
-  else adjoint_mode<8, FULL_TAPE>(ab, P, i);
-}
-
-// Deterministic fleet sum of the 12 per-env gain gradients: each of the
-// `parts` blocks sums a fixed contiguous range in a fixed tree order into
-// partial[k][block]; one block then sums the partials in the same way.
-constexpr int kRedThreads = 256;
-
-__device__ __forceinline__ float block_tree_sum(float v, float* sh) {
-  sh[threadIdx.x] = v;
-  __syncthreads();
-  for (int s = kRedThreads / 2; s > 0; s >>= 1) {
-    if ((int)threadIdx.x < s) sh[threadIdx.x] += sh[threadIdx.x + s];
-    __syncthreads();
+  __shared__ float4 ring[FULL_TAPE ? kSweepStages : 1][4][kAdjointBlock];
+  const uint32_t slot = blockIdx.x * kAdjointBlock + threadIdx.x;
+  V3 gains[4] = {{0.f, 0.f, 0.f}, {0.f, 0.f, 0.f}, {0.f, 0.f, 0.f}, {0.f, 0.f, 0.f}};
+  if (slot < ab.n) {
+    const uint32_t env = ab.order[slot];
+    by_airframe_and_mode(rotors_of(ab, env), mode_of(ab, env), Sweep<FULL_TAPE>{ab, P, slot, env, ring, gains});
   }
-  float r = sh[0];
+  __syncwarp();
+  const float v12[12] = {gains[0].x, gains[0].y, gains[0].z, gains[1].x, gains[1].y, gains[1].z,
+                         gains[2].x, gains[2].y, gains[2].z, gains[3].x, gains[3].y, gains[3].z};
+#pragma unroll
+  for (int k = 0; k < 12; ++k) {
+    float v = v12[k];
+#pragma unroll
+    for (int d = 16; d > 0; d >>= 1) v += __shfl_xor_sync(0xFFFFFFFFu, v, d);
+    if (threadIdx.x == 0) ab.partial[(size_t)k * gridDim.x + blockIdx.x] = v;
+  }
+}
+
+// Fleet sum of the warps' partial sums: one block per gain, each thread over a
+// fixed stride, then a fixed tree, so repeated calls give identical bits.
+constexpr int kRedThreads = 1024;
+__global__ void __launch_bounds__(kRedThreads) k_reduce_gains(const float* partial, uint32_t parts, float* out) {
+  __shared__ float sh[kRedThreads / 32];
+  const float* p = partial + (size_t)blockIdx.x * parts;
+  float acc = 0.f;
+  for (uint32_t j = threadIdx.x; j < parts; j += kRedThreads) acc += p[j];
+#pragma unroll
+  for (int d = 16; d > 0; d >>= 1) acc += __shfl_xor_sync(0xFFFFFFFFu, acc, d);
+  if ((threadIdx.x & 31u) == 0) sh[threadIdx.x >> 5] = acc;
   __syncthreads();
-  return r;
-}
-
-__global__ void __launch_bounds__(kRedThreads) k_reduce_partial(const float* per_env, uint32_t n, float* partial,
-                                                                int parts) {
-  __shared__ float sh[kRedThreads];
-  const int k = blockIdx.y;
-  const size_t chunk = (n + parts - 1) / parts;
-  const size_t lo = chunk * blockIdx.x, hi = lo + chunk < n ? lo + chunk : n;
-  float acc = 0.f;
-  for (size_t j = lo + threadIdx.x; j < hi; j += kRedThreads) acc += per_env[(size_t)k * n + j];
-  const float s = block_tree_sum(acc, sh);
-  if (threadIdx.x == 0) partial[k * parts + blockIdx.x] = s;
-}
-
-__global__ void __launch_bounds__(kRedThreads) k_reduce_final(const float* partial, int parts, float* out) {
-  __shared__ float sh[kRedThreads];
-  const int k = blockIdx.x;
-  float acc = 0.f;
-  for (int j = threadIdx.x; j < parts; j += kRedThreads) acc += partial[k * parts + j];
-  const float s = block_tree_sum(acc, sh);
-  if (threadIdx.x == 0) out[k] = s;
+  if (threadIdx.x < 32) {
+    float v = sh[threadIdx.x];
+#pragma unroll
+    for (int d = 16; d > 0; d >>= 1) v += __shfl_xor_sync(0xFFFFFFFFu, v, d);
+    if (threadIdx.x == 0) out[blockIdx.x] = v;
+  }
 }
 
 }  // namespace
 
 cudaError_t launch_record(const AdjointBuffers& ab, const StepParams& P, cudaStream_t st) {
-  k_record<<<(ab.n + kRecordBlock - 1) / kRecordBlock, kRecordBlock, 0, st>>>(ab, P);
+  const unsigned blocks = (ab.n + kRecordBlock - 1) / kRecordBlock;
+  if (ab.full_tape) k_record<true><<<blocks, kRecordBlock, 0, st>>>(ab, P);
+  else k_record<false><<<blocks, kRecordBlock, 0, st>>>(ab, P);
   return cudaGetLastError();
 }
 
 cudaError_t launch_adjoint(const AdjointBuffers& ab, const StepParams& P, cudaStream_t st) {
-  cudaError_t e;
-  if (ab.full_tape) {
-    const int n_seg = (ab.n_steps + ab.K - 1) / ab.K;
-    const uint64_t threads = (uint64_t)ab.n * n_seg;
-    k_tape<<<(unsigned)((threads + kTapeBlock - 1) / kTapeBlock), kTapeBlock, 0, st>>>(ab, P, n_seg);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  }
-  const unsigned blocks = (ab.n + kAdjointBlock - 1) / kAdjointBlock;
+  const unsigned blocks = (unsigned)adjoint_warps(ab.n);
   if (ab.full_tape) k_adjoint<true><<<blocks, kAdjointBlock, 0, st>>>(ab, P);
   else k_adjoint<false><<<blocks, kAdjointBlock, 0, st>>>(ab, P);
-  e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
-  dim3 g1(kReduceParts, 12);
-  k_reduce_partial<<<g1, kRedThreads, 0, st>>>(ab.grad_gains_env, ab.n, ab.partial, kReduceParts);
-  k_reduce_final<<<12, kRedThreads, 0, st>>>(ab.partial, kReduceParts, ab.grad_gains);
+  cudaError_t e = cudaGetLastError();
+  if (e != cudaSuccess || !ab.grad_gains) return e;
+  k_reduce_gains<<<12, kRedThreads, 0, st>>>(ab.partial, blocks, ab.grad_gains);
   return cudaGetLastError();
 }
 

@@ -8,32 +8,38 @@
 
 namespace agk {
 
-constexpr int kReduceParts = 256;  // first-level blocks of the gain-gradient reduction
+// Warps (blocks of the reverse sweep) of a fleet: one partial gain sum each.
+constexpr size_t adjoint_warps(size_t n) { return (n + 31) / 32; }
+// float4 words of one tape entry of one vehicle.
+constexpr int kTapeWords = 4;
 
-// Device buffers of one recorded rollout and its adjoint. Checkpoint s holds
-// the state (13 rows) and motors (8 rows) at step s*K as [21][n]; the tape
-// holds step-start states in the same layout: every step of the horizon when
-// full_tape is set, else one segment's K steps.
+// Device buffers of one recorded rollout and its adjoint. Arrays marked
+// "slot" are indexed by thread slot (environment order[slot]), the others by
+// environment. With full_tape the tape holds the entries of every step and the
+// end state; else it holds one segment's K entries, and checkpoint s holds
+// the state (13 rows) and motors (8 rows) at step s * K.
 struct AdjointBuffers {
   float* state;                // [13][n] fleet state (advanced by the record)
   float* motors;               // [8][n]
   const float* body;           // [4][n]
   const uint8_t* modes;        // [n] command mode per env (values above 3 act as a wrench)
   const float* targets;        // [4][n] command targets
+  const uint32_t* order;       // [n] thread slot -> environment, grouped by rotor type and mode
   const float* p_goal;         // [3][n]
-  float* ckpt;                 // [S][21][n]
-  float* tape;                 // [n_steps][21][n] (full_tape) or [K][21][n]
+  float* ckpt;                 // [S][21][n] slot (NULL with full_tape)
+  float4* tape;                // [n_steps + 1][4][n] (full_tape) or [K][4][n], slot
+  float* inv_q0;               // [n] slot: 1 / |q_0| of the given initial quaternion
   float* loss;                 // [n]
   uint8_t* saturated;          // [n] some motor hit a clamp during the record
   const float* loss_weights;   // [n] upstream gradient of each env's loss (NULL = 1)
-  float* grad_x0;              // [13][n]
+  float* grad_x0;              // [13][n] (NULL = not wanted, as the next three)
   float* grad_gains_env;       // [12][n]
   float* grad_targets;         // [4][n]
-  float* partial;              // [12][kReduceParts]
   float* grad_gains;           // [12]
+  float* partial;              // [12][adjoint_warps(n)]
   uint32_t n, n_quad, n_hexa, n_octo;
   int n_steps, K;
-  int full_tape;               // 1: the tape spans the whole horizon (recomputed by k_tape)
+  int full_tape;               // 1: the record wrote the whole horizon's tape
   float w_pos, w_omega;
 };
 

@@ -230,7 +230,7 @@ using namespace agh;
 void free_adjoint(ag_ctx* ctx) {
   agk::AdjointBuffers& a = ctx->adj;
   void* ptrs[] = {(void*)a.p_goal, a.ckpt, a.tape, a.loss, a.saturated, (void*)a.loss_weights, a.grad_x0,
-                  a.grad_gains_env, a.grad_targets, a.partial, a.grad_gains};
+                  a.grad_gains_env, a.grad_targets, a.partial, a.grad_gains, a.inv_q0};
   for (void* p : ptrs)
     if (p) cudaFree(p);
 }

@@ -14,43 +14,44 @@ using namespace agh;
 // Differentiable rollout: gains, recorded forward, adjoint.
 namespace {
 
-// Grows the adjoint buffers for a record of n_steps steps with interval K.
+// Buffers of a record of n_steps steps with checkpoint interval K: the tape of
+// the whole horizon when it fits (within hbm_budget_bytes when one is set), so
+// that the record writes what the sweep reads; else a tape of one segment and
+// the checkpoints the sweep recomputes it from.
 ag_status ensure_adjoint(ag_ctx* ctx, int n_steps, int K) {
   agk::AdjointBuffers& a = ctx->adj;
   const size_t n = ctx->cfg.n_envs;
   const size_t n_ckpt = (size_t)(n_steps + K - 1) / K;
   cudaError_t e = cudaSuccess;
   if (!a.loss) {
+    const size_t bytes_before = ctx->bytes;
     float* pg = nullptr; float* lw = nullptr;
     if (e == cudaSuccess) e = alloc(ctx, &pg, 3 * n);
-    if (e == cudaSuccess) e = alloc(ctx, &a.loss, n);
     if (e == cudaSuccess) e = alloc(ctx, &a.saturated, n);
     if (e == cudaSuccess) e = alloc(ctx, &lw, n);
+    if (e == cudaSuccess) e = alloc(ctx, &a.inv_q0, n);
     if (e == cudaSuccess) e = alloc(ctx, &a.grad_x0, 13 * n);
     if (e == cudaSuccess) e = alloc(ctx, &a.grad_gains_env, 12 * n);
     if (e == cudaSuccess) e = alloc(ctx, &a.grad_targets, 4 * n);
-    if (e == cudaSuccess) e = alloc(ctx, &a.partial, 12 * (size_t)agk::kReduceParts);
+    if (e == cudaSuccess) e = alloc(ctx, &a.partial, 12 * agk::adjoint_warps(n));
     if (e == cudaSuccess) e = alloc(ctx, &a.grad_gains, 12);
     a.p_goal = pg;
     a.loss_weights = lw;
-    if (e != cudaSuccess) { cudaGetLastError(); ctx->err = "adjoint buffers do not fit"; return AG_ERR_OOM; }
-  }
-  if (n_ckpt > ctx->adj_ckpt_cap) {
-    if (a.ckpt) {
-      cudaStreamSynchronize(ctx->stream);
-      cudaFree(a.ckpt);
-      a.ckpt = nullptr;
-      ctx->bytes -= ctx->adj_ckpt_cap * 21 * n * sizeof(float);
+    if (e == cudaSuccess) e = alloc(ctx, &a.loss, n);
+    if (e != cudaSuccess) {  // nothing half-allocated stays: the next call starts over
+      cudaGetLastError();
+      void* got[] = {(void*)a.p_goal, a.saturated, (void*)a.loss_weights, a.inv_q0, a.grad_x0, a.grad_gains_env,
+                     a.grad_targets, a.partial, a.grad_gains};
+      for (void* p : got)
+        if (p) cudaFree(p);
+      a = agk::AdjointBuffers{};
+      ctx->bytes = bytes_before;
+      ctx->err = "adjoint buffers do not fit";
+      return AG_ERR_OOM;
     }
-    e = alloc(ctx, &a.ckpt, n_ckpt * 21 * n);
-    if (e != cudaSuccess) { cudaGetLastError(); ctx->adj_ckpt_cap = 0; ctx->err = "checkpoints do not fit"; return AG_ERR_OOM; }
-    ctx->adj_ckpt_cap = n_ckpt;
   }
-  // The tape of step-start states: the whole horizon when it fits (within
-  // hbm_budget_bytes when one is set), so that the backward pass can
-  // recompute every segment in parallel; else one segment of K steps.
-  const size_t step_bytes = 21 * n * sizeof(float);
-  const size_t held = (size_t)ctx->adj_tape_cap * step_bytes;
+  const size_t entry_bytes = agk::kTapeWords * n * sizeof(float4);
+  const size_t held = (size_t)ctx->adj_tape_cap * entry_bytes;
   auto free_tape = [&]() {
     if (a.tape) {
       cudaStreamSynchronize(ctx->stream);
@@ -60,27 +61,51 @@ ag_status ensure_adjoint(ag_ctx* ctx, int n_steps, int K) {
     }
     ctx->adj_tape_cap = 0;
   };
-  if ((size_t)ctx->adj_tape_cap < (size_t)n_steps) {
-    const size_t full_bytes = (size_t)n_steps * step_bytes;
+  const size_t full = (size_t)n_steps + 1;  // one entry per step and the end state
+  if (ctx->adj_tape_cap < full) {
     const uint64_t budget = ctx->cfg.hbm_budget_bytes;
-    if (budget == 0 || ctx->bytes - held + full_bytes <= budget) {
+    if (budget == 0 || ctx->bytes - held + full * entry_bytes <= budget) {
       free_tape();
-      if (alloc(ctx, &a.tape, (size_t)n_steps * 21 * n) == cudaSuccess) {
-        ctx->adj_tape_cap = n_steps;
+      if (alloc(ctx, &a.tape, full * agk::kTapeWords * n) == cudaSuccess) {
+        ctx->adj_tape_cap = full;
       } else {
         cudaGetLastError();  // an out-of-memory cudaMalloc leaves no sticky error
         a.tape = nullptr;
       }
     }
   }
-  a.full_tape = (size_t)ctx->adj_tape_cap >= (size_t)n_steps ? 1 : 0;
-  if (!a.full_tape && K > ctx->adj_tape_cap) {
+  a.full_tape = ctx->adj_tape_cap >= full ? 1 : 0;
+  if (a.full_tape) return AG_OK;
+  const size_t entries = (size_t)(K < n_steps ? K : n_steps);
+  if (entries > ctx->adj_tape_cap) {
     free_tape();
-    e = alloc(ctx, &a.tape, (size_t)K * 21 * n);
-    if (e != cudaSuccess) { cudaGetLastError(); ctx->adj_tape_cap = 0; ctx->err = "tape does not fit"; return AG_ERR_OOM; }
-    ctx->adj_tape_cap = K;
+    e = alloc(ctx, &a.tape, entries * agk::kTapeWords * n);
+    if (e != cudaSuccess) { cudaGetLastError(); a.tape = nullptr; ctx->err = "tape does not fit"; return AG_ERR_OOM; }
+    ctx->adj_tape_cap = entries;
+  }
+  if (n_ckpt > ctx->adj_ckpt_cap) {
+    if (a.ckpt) {
+      cudaStreamSynchronize(ctx->stream);
+      cudaFree(a.ckpt);
+      a.ckpt = nullptr;
+      ctx->bytes -= ctx->adj_ckpt_cap * 21 * n * sizeof(float);
+      ctx->adj_ckpt_cap = 0;
+    }
+    e = alloc(ctx, &a.ckpt, n_ckpt * 21 * n);
+    if (e != cudaSuccess) { cudaGetLastError(); a.ckpt = nullptr; ctx->err = "checkpoints do not fit"; return AG_ERR_OOM; }
+    ctx->adj_ckpt_cap = n_ckpt;
   }
   return AG_OK;
+}
+
+// Memory of the context's own device, which its kernels can write without a
+// staging copy (managed, host and other devices' memory is copied to).
+bool on_own_device(const ag_ctx* ctx, const void* p) {
+  cudaPointerAttributes pa;
+  const bool own = cudaPointerGetAttributes(&pa, p) == cudaSuccess && pa.type == cudaMemoryTypeDevice &&
+                   pa.device == ctx->device;
+  cudaGetLastError();
+  return own;
 }
 
 }  // namespace
@@ -113,20 +138,24 @@ extern "C" ag_status ag_rollout_loss(ag_ctx* ctx, uint32_t n_steps, float w_pos,
     return fail_invalid(ctx, "n_steps must be in 1..2^30; p_goal and loss are required");
   const size_t n = c.n_envs;
   const int K = c.record_every ? (int)c.record_every : 32;
+  ctx->adj_recorded = false;  // the buffers of the last record may be replaced
   if ((s = ensure_adjoint(ctx, (int)n_steps, K)) != AG_OK) return s;
   agk::AdjointBuffers& a = ctx->adj;
   if ((s = check_cuda(ctx, cudaMemcpyAsync((void*)a.p_goal, p_goal, 3 * n * sizeof(float), cudaMemcpyDefault,
                                            ctx->stream), "copy goals")) != AG_OK) return s;
   a.state = ctx->fb.state; a.motors = ctx->fb.motors; a.body = ctx->fb.body; a.targets = ctx->fb.targets;
   a.modes = ctx->fb.modes;
+  a.order = ctx->fb.order;
   a.n = c.n_envs; a.n_quad = c.n_quad; a.n_hexa = c.n_hexa; a.n_octo = c.n_octo;
   a.n_steps = (int)n_steps; a.K = K; a.w_pos = w_pos; a.w_omega = w_omega;
   ctx->adj_P = step_params(ctx);
-  ctx->adj_recorded = false;
-  if ((s = check_cuda(ctx, agk::launch_record(a, ctx->adj_P, ctx->stream), "record launch")) != AG_OK) return s;
+  const bool direct = on_own_device(ctx, loss);
+  agk::AdjointBuffers rec = a;
+  if (direct) rec.loss = loss;
+  if ((s = check_cuda(ctx, agk::launch_record(rec, ctx->adj_P, ctx->stream), "record launch")) != AG_OK) return s;
   ctx->adj_recorded = true;
-  if ((s = check_cuda(ctx, cudaMemcpyAsync(loss, a.loss, n * sizeof(float), cudaMemcpyDefault, ctx->stream),
-                      "copy loss out")) != AG_OK) return s;
+  if (!direct && (s = check_cuda(ctx, cudaMemcpyAsync(loss, a.loss, n * sizeof(float), cudaMemcpyDefault, ctx->stream),
+                                 "copy loss out")) != AG_OK) return s;
   if (saturated)
     s = check_cuda(ctx, cudaMemcpyAsync(saturated, a.saturated, n, cudaMemcpyDefault, ctx->stream), "copy flags out");
   return s;
@@ -150,18 +179,22 @@ extern "C" ag_status ag_backward(ag_ctx* ctx, const float* loss_weights, float* 
   } else {
     a.loss_weights = nullptr;
   }
+  // a wanted output in the context's own device memory is written in place, any other through the staging
+  // buffer; unwanted ones are not formed
+  struct Out { float* user; float** field; float* stage; size_t count; const char* what; };
+  const Out outs[4] = {{grad_x0, &a.grad_x0, a.grad_x0, 13 * n, "copy grad x0"},
+                       {grad_gains, &a.grad_gains, a.grad_gains, 12, "copy grad gains"},
+                       {grad_gains_per_env, &a.grad_gains_env, a.grad_gains_env, 12 * n, "copy per-env grad gains"},
+                       {grad_targets, &a.grad_targets, a.grad_targets, 4 * n, "copy grad targets"}};
+  bool staged[4];
+  for (int k = 0; k < 4; ++k) {
+    staged[k] = outs[k].user && !on_own_device(ctx, outs[k].user);
+    *outs[k].field = staged[k] ? outs[k].stage : outs[k].user;
+  }
   if ((s = check_cuda(ctx, agk::launch_adjoint(a, ctx->adj_P, ctx->stream), "adjoint launch")) != AG_OK) return s;
-  cudaStream_t st = ctx->stream;
-  if (grad_x0 && (s = check_cuda(ctx, cudaMemcpyAsync(grad_x0, a.grad_x0, 13 * n * sizeof(float), cudaMemcpyDefault,
-                                                      st), "copy grad x0")) != AG_OK) return s;
-  if (grad_gains && (s = check_cuda(ctx, cudaMemcpyAsync(grad_gains, a.grad_gains, 12 * sizeof(float),
-                                                         cudaMemcpyDefault, st), "copy grad gains")) != AG_OK) return s;
-  if (grad_gains_per_env && (s = check_cuda(ctx, cudaMemcpyAsync(grad_gains_per_env, a.grad_gains_env,
-                                                                  12 * n * sizeof(float), cudaMemcpyDefault, st),
-                                             "copy per-env grad gains")) != AG_OK) return s;
-  if (grad_targets)
-    s = check_cuda(ctx, cudaMemcpyAsync(grad_targets, a.grad_targets, 4 * n * sizeof(float), cudaMemcpyDefault, st),
-                   "copy grad targets");
+  for (int k = 0; k < 4; ++k)
+    if (staged[k] && (s = check_cuda(ctx, cudaMemcpyAsync(outs[k].user, outs[k].stage, outs[k].count * sizeof(float),
+                                                          cudaMemcpyDefault, ctx->stream), outs[k].what)) != AG_OK)
+      return s;
   return s;
 }
-

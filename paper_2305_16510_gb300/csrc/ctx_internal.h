@@ -28,7 +28,7 @@ struct ag_ctx {
   // differentiable rollout (allocated at the first ag_rollout_loss)
   agk::AdjointBuffers adj;
   size_t adj_ckpt_cap;       // checkpoints the ckpt buffer holds
-  int adj_tape_cap;          // steps the tape holds
+  size_t adj_tape_cap;       // entries the tape holds
   bool adj_recorded;
   agk::StepParams adj_P;     // parameters of the recorded rollout
   // depth rendering staging (allocated on first use, grown as needed)

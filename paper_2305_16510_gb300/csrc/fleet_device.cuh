@@ -262,9 +262,11 @@ __device__ __forceinline__ Wrench4 controller(const VState& s, const Command& cm
 // the realised wrench A u. Two motors travel as one FP32 pair through the
 // allocation and the lag, and the wrench accumulates as the pairs (f, M_x)
 // and (M_y, M_z), in packed FMAs (__ffma2_rn) that round each lane as the
-// scalar form would, in the same order.
+// scalar form would, in the same order. pass (may be NULL) receives one bit
+// per motor whose command lies strictly inside the limits.
 template <int NROT>
-__device__ __forceinline__ Wrench4 allocate(const Wrench4& cmd, float (&u)[NROT], const StepParams& P) {
+__device__ __forceinline__ Wrench4 allocate(const Wrench4& cmd, float (&u)[NROT], const StepParams& P,
+                                            uint32_t* pass = nullptr) {
   constexpr int T = NROT == 4 ? 0 : (NROT == 6 ? 1 : 2);
   const float2 f2 = make_float2(cmd.f, cmd.f), mx2 = make_float2(cmd.mx, cmd.mx);
   const float2 my2 = make_float2(cmd.my, cmd.my), mz2 = make_float2(cmd.mz, cmd.mz);
@@ -274,6 +276,8 @@ __device__ __forceinline__ Wrench4 allocate(const Wrench4& cmd, float (&u)[NROT]
   for (int j = 0; j < NROT / 2; ++j) {
     float2 uc = __ffma2_rn(P.Ap2[T][j][3], mz2,
                            __ffma2_rn(P.Ap2[T][j][2], my2, __ffma2_rn(P.Ap2[T][j][1], mx2, __fmul2_rn(P.Ap2[T][j][0], f2))));
+    if (pass)
+      *pass |= (uc.x > 0.f && uc.x < P.u_max ? 1u << (2 * j) : 0u) | (uc.y > 0.f && uc.y < P.u_max ? 2u << (2 * j) : 0u);
     uc = make_float2(fminf(fmaxf(uc.x, 0.f), P.u_max), fminf(fmaxf(uc.y, 0.f), P.u_max));
     float2 uu = make_float2(u[2 * j], u[2 * j + 1]);
     uu = __ffma2_rn(alpha2, __fadd2_rn(uc, make_float2(-uu.x, -uu.y)), uu);
