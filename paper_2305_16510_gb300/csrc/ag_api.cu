@@ -156,8 +156,8 @@ namespace {
 size_t buffer_bytes(const ag_config* c) {
   size_t n = c->n_envs;
   size_t per = sizeof(float) * (13 + 8 + 4 + 4 + 4 + 4) + sizeof(uint32_t) * 4 + 3 /* modes, collided, hits */ + 1;
-  return n * per + (size_t)c->n_obstacles * 10 * n * sizeof(float) +
-         agk::box_pair_elems(n, c->n_obstacles) * sizeof(float2) + sizeof(uint32_t) + sizeof(unsigned long long);
+  return n * per + agk::box_record_bytes(n, c->n_obstacles) + (c->n_obstacles ? 10 * n * sizeof(float) : 0) +
+         sizeof(uint32_t) + sizeof(unsigned long long);
 }
 
 }  // namespace
@@ -221,6 +221,14 @@ bool on_device(const void* p) {
   return dev;
 }
 
+bool on_own_device(const ag_ctx* ctx, const void* p) {
+  cudaPointerAttributes pa;
+  const bool own = cudaPointerGetAttributes(&pa, p) == cudaSuccess && pa.type == cudaMemoryTypeDevice &&
+                   pa.device == ctx->device;
+  cudaGetLastError();
+  return own;
+}
+
 }  // namespace agh
 
 namespace {
@@ -245,9 +253,9 @@ void free_all(ag_ctx* ctx) {
   if (ctx->reach_goals) cudaFree(ctx->reach_goals);
   if (ctx->reach_steps) cudaFree(ctx->reach_steps);
   agk::FleetBuffers& f = ctx->fb;
-  void* ptrs[] = {f.state, f.motors, f.body, f.modes, f.targets, f.boxes, f.epoch, f.collided, f.reset_ids,
-                  f.n_reset, f.tests_run, f.cmd, f.wrench, f.resets, f.hits, f.order, f.boxes_slot, ctx->mask_dev,
-                  ctx->order_scratch, f.slot_of, (void*)f.box_rand};
+  void* ptrs[] = {f.state, f.motors, f.body, f.modes, f.targets, f.box_bound, f.box_rest, f.epoch, f.collided, f.reset_ids,
+                  f.n_reset, f.tests_run, f.cmd, f.wrench, f.resets, f.hits, f.order, ctx->mask_dev,
+                  ctx->box_stage, (void*)f.box_rand};
   for (void* p : ptrs)
     if (p) cudaFree(p);
 }
@@ -313,7 +321,7 @@ ag_status ag_create(const ag_config* cfg, void* cuda_stream, ag_ctx** out) {
   ctx->seed = cfg->seed;
   std::memset(&ctx->fb, 0, sizeof(ctx->fb));
   ctx->mask_dev = nullptr;
-  ctx->order_scratch = nullptr;
+  ctx->box_stage = nullptr;
   std::memset(&ctx->adj, 0, sizeof(ctx->adj));
   ctx->adj_ckpt_cap = 0;
   ctx->adj_tape_cap = 0;
@@ -342,8 +350,9 @@ ag_status ag_create(const ag_config* cfg, void* cuda_stream, ag_ctx** out) {
   if (e == cudaSuccess) e = alloc(ctx, &f.body, 4 * n);
   if (e == cudaSuccess) e = alloc(ctx, &f.modes, n);
   if (e == cudaSuccess) e = alloc(ctx, &f.targets, 4 * n);
-  if (e == cudaSuccess) e = alloc(ctx, &f.boxes, (size_t)cfg->n_obstacles * 10 * n);
-  if (e == cudaSuccess) e = alloc(ctx, &f.boxes_slot, agk::box_pair_elems(n, cfg->n_obstacles));
+  if (e == cudaSuccess) e = alloc(ctx, &f.box_bound, (size_t)cfg->n_obstacles * n);
+  if (e == cudaSuccess) e = alloc(ctx, &f.box_rest, (size_t)cfg->n_obstacles * n * 2);
+  if (e == cudaSuccess && cfg->n_obstacles) e = alloc(ctx, &ctx->box_stage, 10 * n);
   if (e == cudaSuccess) e = alloc(ctx, &f.epoch, n);
   if (e == cudaSuccess) e = alloc(ctx, &f.collided, n);
   if (e == cudaSuccess) e = alloc(ctx, &f.reset_ids, n);
@@ -356,8 +365,6 @@ ag_status ag_create(const ag_config* cfg, void* cuda_stream, ag_ctx** out) {
   if (e == cudaSuccess) e = alloc(ctx, &ctx->mask_dev, n);
   if (e == cudaSuccess) e = alloc(ctx, &ctx->check_dev, 1);
   if (e == cudaSuccess) e = alloc(ctx, &f.order, n);
-  if (e == cudaSuccess && cfg->n_obstacles) e = alloc(ctx, &f.slot_of, n);
-  if (e == cudaSuccess) e = alloc(ctx, &ctx->order_scratch, agk::order_scratch_words(cfg->n_envs));
   if (e != cudaSuccess) {
     g_create_error = std::string("device allocation failed: ") + cudaGetErrorString(e);
     cudaGetLastError();
@@ -376,14 +383,15 @@ ag_status ag_create(const ag_config* cfg, void* cuda_stream, ag_ctx** out) {
   }
   if (e == cudaSuccess) e = cudaMemsetAsync(f.modes, AG_MODE_WRENCH, n, st);
   if (e == cudaSuccess) e = cudaMemsetAsync(f.targets, 0, 4 * n * sizeof(float), st);
-  if (e == cudaSuccess && f.boxes) e = cudaMemsetAsync(f.boxes, 0, (size_t)cfg->n_obstacles * 10 * n * sizeof(float), st);
-  if (e == cudaSuccess && f.boxes_slot)
-    e = cudaMemsetAsync(f.boxes_slot, 0, agk::box_pair_elems(n, cfg->n_obstacles) * sizeof(float2), st);
+  if (e == cudaSuccess && f.box_bound)
+    e = cudaMemsetAsync(f.box_bound, 0, (size_t)cfg->n_obstacles * n * sizeof(float4), st);
+  if (e == cudaSuccess && f.box_rest)
+    e = cudaMemsetAsync(f.box_rest, 0, (size_t)cfg->n_obstacles * n * 2 * sizeof(float4), st);
   if (e == cudaSuccess) e = cudaMemsetAsync(f.epoch, 0, n * sizeof(uint32_t), st);
   if (e == cudaSuccess) e = cudaMemsetAsync(f.collided, 0, n, st);
   if (e == cudaSuccess) e = cudaMemsetAsync(f.n_reset, 0, sizeof(uint32_t), st);
   if (e == cudaSuccess) e = cudaMemsetAsync(f.tests_run, 0, sizeof(unsigned long long), st);
-  if (e == cudaSuccess) e = agk::launch_build_order(f, ctx->order_scratch, st);
+  if (e == cudaSuccess) e = agk::launch_build_order(f, st);
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);
   if (e != cudaSuccess) {
     g_create_error = std::string("initialisation failed: ") + cudaGetErrorString(e);
@@ -412,7 +420,7 @@ ag_status ag_set_commands(ag_ctx* ctx, const uint8_t* modes, const float* target
   if (modes) {
     s = check_cuda(ctx, cudaMemcpyAsync(ctx->fb.modes, modes, n, cudaMemcpyDefault, ctx->stream), "copy modes");
     if (s != AG_OK) return s;
-    s = check_cuda(ctx, agk::launch_build_order(ctx->fb, ctx->order_scratch, ctx->stream), "build order");
+    s = check_cuda(ctx, agk::launch_build_order(ctx->fb, ctx->stream), "build order");
     if (s != AG_OK) return s;
   }
   if (targets)
@@ -428,7 +436,6 @@ ag_status ag_set_obstacles(ag_ctx* ctx, const float* boxes) {
   if (!boxes) return fail_invalid(ctx, "boxes is NULL");
   if (ctx->cfg.n_obstacles == 0) return AG_OK;
   const uint32_t n = ctx->cfg.n_envs, n_obs = ctx->cfg.n_obstacles;
-  const size_t count = (size_t)n_obs * 10 * n;
   uint32_t bad = 0;
   if (on_device(boxes)) {
     s = count_bad_on_device(ctx, [&](cudaStream_t st) {
@@ -446,20 +453,34 @@ ag_status ag_set_obstacles(ag_ctx* ctx, const float* boxes) {
       }
   }
   if (bad) return fail_invalid(ctx, "boxes: finite centres, half-extents > 0 and unit quaternions required");
-  s = check_cuda(ctx, cudaMemcpyAsync(ctx->fb.boxes, boxes, count * sizeof(float), cudaMemcpyDefault, ctx->stream),
-                 "copy boxes");
-  if (s != AG_OK) return s;
-  return check_cuda(ctx, agk::launch_permute_boxes(ctx->fb, ctx->stream), "permute boxes");
+  cudaStream_t st = ctx->stream;
+  if (on_own_device(ctx, boxes))
+    return check_cuda(ctx, agk::launch_pack_boxes(ctx->fb, boxes, n, 0, n_obs, st), "pack boxes");
+  for (uint32_t k = 0; k < n_obs; ++k) {  // box by box through the staging rows
+    if ((s = check_cuda(ctx, cudaMemcpyAsync(ctx->box_stage, boxes + (size_t)k * 10 * n, 10 * (size_t)n * sizeof(float),
+                                             cudaMemcpyDefault, st), "copy boxes")) != AG_OK) return s;
+    if ((s = check_cuda(ctx, agk::launch_pack_boxes(ctx->fb, ctx->box_stage, n, k, 1, st), "pack boxes")) != AG_OK)
+      return s;
+  }
+  return AG_OK;
 }
 
 ag_status ag_get_obstacles(ag_ctx* ctx, float* boxes) {
   ag_status s = enter(ctx);
   if (s != AG_OK) return s;
   if (!boxes) return fail_invalid(ctx, "boxes is NULL");
-  const size_t count = (size_t)ctx->cfg.n_obstacles * 10 * ctx->cfg.n_envs;
-  if (count == 0) return AG_OK;
-  return check_cuda(ctx, cudaMemcpyAsync(boxes, ctx->fb.boxes, count * sizeof(float), cudaMemcpyDefault, ctx->stream),
-                    "copy boxes out");
+  const uint32_t n = ctx->cfg.n_envs, n_obs = ctx->cfg.n_obstacles;
+  if (n_obs == 0) return AG_OK;
+  cudaStream_t st = ctx->stream;
+  if (on_own_device(ctx, boxes))
+    return check_cuda(ctx, agk::launch_unpack_boxes(ctx->fb, boxes, 0, n_obs, st), "unpack boxes");
+  for (uint32_t k = 0; k < n_obs; ++k) {
+    if ((s = check_cuda(ctx, agk::launch_unpack_boxes(ctx->fb, ctx->box_stage, k, 1, st), "unpack boxes")) != AG_OK)
+      return s;
+    if ((s = check_cuda(ctx, cudaMemcpyAsync(boxes + (size_t)k * 10 * n, ctx->box_stage, 10 * (size_t)n * sizeof(float),
+                                             cudaMemcpyDefault, st), "copy boxes out")) != AG_OK) return s;
+  }
+  return AG_OK;
 }
 
 ag_status ag_set_obstacle_randomization(ag_ctx* ctx, const float env_min[3], const float env_max[3],

@@ -98,16 +98,6 @@ ag_status ensure_adjoint(ag_ctx* ctx, int n_steps, int K) {
   return AG_OK;
 }
 
-// Memory of the context's own device, which its kernels can write without a
-// staging copy (managed, host and other devices' memory is copied to).
-bool on_own_device(const ag_ctx* ctx, const void* p) {
-  cudaPointerAttributes pa;
-  const bool own = cudaPointerGetAttributes(&pa, p) == cudaSuccess && pa.type == cudaMemoryTypeDevice &&
-                   pa.device == ctx->device;
-  cudaGetLastError();
-  return own;
-}
-
 }  // namespace
 
 extern "C" ag_status ag_set_gains(ag_ctx* ctx, const float* gains12) {

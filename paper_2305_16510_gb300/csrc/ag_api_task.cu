@@ -58,7 +58,8 @@ ag_status render_depth_impl(ag_ctx* ctx, uint32_t width, uint32_t height, float 
   }
   agk::DepthArgs a;
   a.state = ctx->fb.state;
-  a.boxes = ctx->fb.boxes;
+  a.box_bound = ctx->fb.box_bound;
+  a.box_rest = ctx->fb.box_rest;
   a.env_ids = ids_dev;
   a.out = out;
   a.n = n;
@@ -158,7 +159,7 @@ ag_status ag_reach_begin(ag_ctx* ctx, const ag_reach_config* cfg, const float* g
       AG_OK) return s;
   if ((s = check_cuda(ctx, cudaMemsetAsync(ctx->fb.modes, (int)cfg->command_mode, n, st), "set modes")) != AG_OK)
     return s;
-  if ((s = check_cuda(ctx, agk::launch_build_order(ctx->fb, ctx->order_scratch, st), "build order")) != AG_OK)
+  if ((s = check_cuda(ctx, agk::launch_build_order(ctx->fb, st), "build order")) != AG_OK)
     return s;
   ctx->reach = *cfg;
   ctx->reach_active = true;

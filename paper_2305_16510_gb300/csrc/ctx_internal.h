@@ -19,7 +19,7 @@ struct ag_ctx {
   int device;
   agk::FleetBuffers fb;
   uint8_t* mask_dev;         // [n] staging for ag_reset masks
-  uint32_t* order_scratch;   // per-block key counts / offsets of the grouping permutation
+  float* box_stage;          // [10][n] one box's rows on their way to or from memory of another kind (NULL without boxes)
   uint64_t seed;             // Philox key of collision resets
   bool failed;
   std::string err;
@@ -59,6 +59,9 @@ ag_status enter(ag_ctx* ctx);
 agk::StepParams step_params(const ag_ctx* ctx);
 // true for device or managed memory (a kernel can read it), false for host memory.
 bool on_device(const void* p);
+// true for memory of the context's own device, which its kernels read and
+// write in place (managed, host and other devices' memory is copied).
+bool on_own_device(const ag_ctx* ctx, const void* p);
 // Rotor allocation matrix A and its pseudo-inverse A^+ in FP64, stored float32.
 void rotor_matrices(int n, double arm, double k_yaw, float A[4][8], float Ap[8][4]);
 // "" for a valid config, else a static message (no allocation).

@@ -81,11 +81,11 @@ __device__ __forceinline__ CamPose camera_pose(const DepthArgs& a, uint32_t env)
 
 // record of box k: (M00 M01 M02 M10) (M11 M12 M20 M21) (M22 lo.x lo.y lo.z) (hi.x hi.y hi.z 0)
 __device__ __forceinline__ void box_record(const DepthArgs& a, uint32_t env, const CamPose& c, int k, float4* rec) {
-  const uint32_t n = a.n;
-  const float* bx = a.boxes + (size_t)k * 10 * n + env;
+  const size_t at = (size_t)k * a.n + env;
+  const float4 b = a.box_bound[at], hq = a.box_rest[2 * at], q = a.box_rest[2 * at + 1];
   float Rb[3][3];
-  rotation(Q4{bx[6 * n], bx[7 * n], bx[8 * n], bx[9 * n]}, Rb);
-  const float v[3] = {c.o[0] - bx[0], c.o[1] - bx[n], c.o[2] - bx[2 * n]};
+  rotation(Q4{hq.w, q.x, q.y, q.z}, Rb);
+  const float v[3] = {c.o[0] - b.x, c.o[1] - b.y, c.o[2] - b.z};
   float M[3][3], ob[3];
 #pragma unroll
   for (int i = 0; i < 3; ++i) {
@@ -93,7 +93,7 @@ __device__ __forceinline__ void box_record(const DepthArgs& a, uint32_t env, con
 #pragma unroll
     for (int j = 0; j < 3; ++j) M[i][j] = fmaf(Rb[2][i], c.R[2][j], fmaf(Rb[1][i], c.R[1][j], Rb[0][i] * c.R[0][j]));
   }
-  const float h[3] = {bx[3 * n], bx[4 * n], bx[5 * n]};
+  const float h[3] = {hq.x, hq.y, hq.z};
   rec[0] = make_float4(M[0][0], M[0][1], M[0][2], M[1][0]);
   rec[1] = make_float4(M[1][1], M[1][2], M[2][0], M[2][1]);
   rec[2] = make_float4(M[2][2], -h[0] - ob[0], -h[1] - ob[1], -h[2] - ob[2]);
@@ -103,13 +103,13 @@ __device__ __forceinline__ void box_record(const DepthArgs& a, uint32_t env, con
 // Bounding sphere of box k in the camera frame: centre s, radius |h| with a
 // rounding margin.
 __device__ __forceinline__ float4 box_sphere(const DepthArgs& a, uint32_t env, const CamPose& c, int k) {
-  const uint32_t n = a.n;
-  const float* bx = a.boxes + (size_t)k * 10 * n + env;
-  const float v[3] = {bx[0] - c.o[0], bx[n] - c.o[1], bx[2 * n] - c.o[2]};
+  const size_t at = (size_t)k * a.n + env;
+  const float4 b = a.box_bound[at], hq = a.box_rest[2 * at];
+  const float v[3] = {b.x - c.o[0], b.y - c.o[1], b.z - c.o[2]};
   const float sx = fmaf(c.R[2][0], v[2], fmaf(c.R[1][0], v[1], c.R[0][0] * v[0]));
   const float sy = fmaf(c.R[2][1], v[2], fmaf(c.R[1][1], v[1], c.R[0][1] * v[0]));
   const float sz = fmaf(c.R[2][2], v[2], fmaf(c.R[1][2], v[1], c.R[0][2] * v[0]));
-  const float h0 = bx[3 * n], h1 = bx[4 * n], h2 = bx[5 * n];
+  const float h0 = hq.x, h1 = hq.y, h2 = hq.z;
   const float rho = 1.001f * sqrtf(h0 * h0 + h1 * h1 + h2 * h2) + 1e-4f * (fabsf(sx) + fabsf(sy) + fabsf(sz)) + 1e-6f;
   return make_float4(sx, sy, sz, rho);
 }

@@ -10,7 +10,8 @@ namespace agk {
 
 struct DepthArgs {
   const float* state;      // [13][n]
-  const float* boxes;      // [n_obs][10][n]
+  const float4* box_bound; // [n_obs][n]    (centre, circumscribed radius)
+  const float4* box_rest;  // [n_obs][n][2] (half-extents, q_w) (q_x, q_y, q_z, 0)
   const uint32_t* env_ids; // [n_cams] or NULL (camera j = env j)
   float* out;              // [n_cams][height][width]
   uint32_t n, n_obs, n_cams, width, height;

@@ -439,13 +439,11 @@ __device__ __forceinline__ void integrate(VState& s, V3 b3, const Wrench4& W, co
     step_sie<DRAG>(s, b3, W, b, P.drag, P.h);
 }
 
-// Sphere of squared radius r2 at p versus the box (centre c, half-extents
-// hx, hy, hz, unit quaternion qb): p is taken into the box frame by the
-// conjugate rotation v - w t + u x t with t = 2 u x v; the distance to the
-// box is the norm of max(|d| - h, 0) per axis (equal to |d - clamp(d, -h, h)|);
-// touching counts. The operations and their order are those of the fused
-// step's paired test (pair_dist2), so both take the same decisions.
-__device__ __forceinline__ bool sphere_hits_box(V3 p, float r2, V3 c, V3 hb, Q4 qb) {
+// Squared distance from p to the box (centre c, half-extents hb, unit
+// quaternion qb): p is taken into the box frame by the conjugate rotation
+// v - w t + u x t with t = 2 u x v; the distance to the box is the norm of
+// max(|d| - h, 0) per axis (equal to |d - clamp(d, -h, h)|).
+__device__ __forceinline__ float box_dist2(V3 p, V3 c, V3 hb, Q4 qb) {
   const V3 v = p - c;
   const V3 u2 = {2.f * qb.x, 2.f * qb.y, 2.f * qb.z};
   const V3 t = cross(u2, v);                  // 2 u x v
@@ -455,7 +453,11 @@ __device__ __forceinline__ bool sphere_hits_box(V3 p, float r2, V3 c, V3 hb, Q4 
   const float ex = fmaxf(fabsf(d.x) - hb.x, 0.f);
   const float ey = fmaxf(fabsf(d.y) - hb.y, 0.f);
   const float ez = fmaxf(fabsf(d.z) - hb.z, 0.f);
-  return !(r2 < fmaf(ez, ez, fmaf(ey, ey, ex * ex)));
+  return fmaf(ez, ez, fmaf(ey, ey, ex * ex));
 }
+
+// The sphere of squared radius r2 touches a box at squared distance e2
+// (touching counts, and so does a NaN distance).
+__device__ __forceinline__ bool touches(float r2, float e2) { return !(r2 < e2); }
 
 }  // namespace agk

@@ -27,7 +27,10 @@ struct FleetBuffers {
   float* body;         // [4][n]   m, Jxx, Jyy, Jzz
   uint8_t* modes;      // [n]
   float* targets;      // [4][n]
-  float* boxes;        // [n_obs][10][n]
+  float* boxes;        // [n_obs][10][n] centre, half-extents, quaternion: the caller's array of the
+                       // allocation-free step; a context keeps the box records below instead
+  float4* box_bound;   // [n_obs][n]    (centre, radius of the circumscribed sphere)
+  float4* box_rest;    // [n_obs][n][2] (half-extents, q_w) (q_x, q_y, q_z, 0)
   uint32_t* epoch;     // [n]
   uint8_t* collided;   // [n]     hit a box during the last call
   uint32_t* reset_ids; // [n]     compact list of envs reset during the last call
@@ -38,10 +41,6 @@ struct FleetBuffers {
   uint32_t* resets;    // [n]     resets of this call per env
   uint8_t* hits;       // [n]     collision of the current step
   uint32_t* order;     // [n]     thread slot -> env, grouped by rotor type and mode (NULL = identity)
-  float2* boxes_slot;  // [ceil(n_obs/2)][10][n] the boxes in slot order, in pairs: element
-                       // (j*10 + f)*n + i = (field f of box 2j, of box 2j+1) of env order[i],
-                       // in the staged form of staged_field (-c, -h, -w, 2u)
-  uint32_t* slot_of;   // [n]     inverse of order (NULL when no obstacle re-draw is needed)
   const BoxRandDev* box_rand;  // [n_obs] obstacle re-draw on reset (NULL = boxes keep their poses)
   unsigned long long* tests_run;  // [1] exact collision tests of the last fused call (NULL = not counted)
   uint32_t n, n_quad, n_hexa, n_octo, n_obs;
@@ -63,23 +62,16 @@ cudaError_t launch_controller(const FleetBuffers& fb, const StepParams& P, cudaS
 cudaError_t launch_plain_step(const FleetBuffers& fb, const StepParams& P, int integrator, int n_steps,
                               int substeps, cudaStream_t st);
 
-// Builds fb.order from the current modes and rotor types (one launch; scratch
-// holds order_scratch_words(n) words), then refreshes fb.boxes_slot.
-cudaError_t launch_build_order(const FleetBuffers& fb, uint32_t* scratch, cudaStream_t st);
-size_t order_scratch_words(uint32_t n);
-// Elements (float2) of fb.boxes_slot for n envs with n_obs boxes each.
-inline size_t box_pair_elems(size_t n, size_t n_obs) { return (n_obs + 1) / 2 * 10 * n; }
+// Builds fb.order from the current modes and rotor types (one launch).
+cudaError_t launch_build_order(const FleetBuffers& fb, cudaStream_t st);
 
-// Refreshes fb.boxes_slot from fb.boxes and fb.order (after the boxes change).
-// An odd box count is padded with a box at 1e30 that no sphere can touch.
-cudaError_t launch_permute_boxes(const FleetBuffers& fb, cudaStream_t st);
-
-// Dynamic shared memory of a fused-kernel block of B threads: box pairs 1..
-// of every thread (pair 0 stays in registers).
-inline size_t fused_smem_bytes(int n_obs, int B) {
-  const int pairs = (n_obs + 1) / 2;
-  return pairs > 1 ? (size_t)(pairs - 1) * 10 * B * 8 : 0;
-}
+// Box records of boxes k0 .. k0 + count - 1 from the layout of ag_set_obstacles
+// (row f of box k0 + j at src[(j * 10 + f) * pitch + env]), and back (pitch n).
+cudaError_t launch_pack_boxes(const FleetBuffers& fb, const float* src, size_t pitch, uint32_t k0, uint32_t count,
+                              cudaStream_t st);
+cudaError_t launch_unpack_boxes(const FleetBuffers& fb, float* dst, uint32_t k0, uint32_t count, cudaStream_t st);
+// Bytes of the box records of n envs with n_obs boxes each.
+inline size_t box_record_bytes(size_t n, size_t n_obs) { return n * n_obs * 3 * sizeof(float4); }
 
 // Launch choices of the fused kernel. Defaults: mode-grouped order, the
 // block size (from 64, 128, 96, 32) with the most resident warps per SM by
@@ -87,9 +79,9 @@ inline size_t fused_smem_bytes(int n_obs, int B) {
 // while a vehicle provably cannot reach a box. Tuning overrides (read at each
 // launch): AG_FUSED_ORDER=identity runs env i in slot i (the ungrouped
 // ablation), AG_FUSED_BLOCK=32..128 (multiple of 32) sets the block size,
-// AG_FUSED_SKIP=0 runs the exact test at every step (same results, the
-// reference the skip is checked against).
+// AG_FUSED_SKIP=0 tests every box at every step (same results, the reference
+// the skip and the bounding spheres are checked against).
 struct FusedTuning { bool sorted; int block; bool skip; };
-FusedTuning fused_tuning_from_env(int n_obs);
+FusedTuning fused_tuning_from_env();
 
 }  // namespace agk

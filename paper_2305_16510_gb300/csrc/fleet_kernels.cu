@@ -5,15 +5,15 @@
 // launch of n_steps steps. Its 13 state words, motor thrusts, body
 // parameters and command live in registers across every substep; its boxes
 // are read only when a collision test runs (the first step, then only while
-// the vehicle may be within reach of a box), as coalesced rows of the
-// slot-ordered pair copy; state and command are read at the start and
-// written at the end of the launch (coalesced structure-of-arrays rows).
+// the vehicle may be within reach of a box); state and command are read at
+// the start and written at the end of the launch (coalesced structure-of-arrays rows).
 // Collision resets happen in registers; the reset list is built with one
 // __ballot_sync + __popc prefix and one atomicAdd per warp.
-#include <atomic>
 #include <cstdint>
 #include <cstdlib>
 #include <cstring>
+#include <type_traits>
+
 #include <cuda_runtime.h>
 
 #include "fleet_internal.h"
@@ -23,121 +23,43 @@
 namespace agk {
 namespace {
 
-// Dynamic shared memory cap of the fused kernel (box staging).
-constexpr size_t kFusedSmemCap = 200 * 1024;
-
-// Tuning override (read at each launch): AG_FUSED_BOXES=smem stages every
-// thread's boxes on chip for the whole launch instead of reading them from
-// the global pair copy when a collision test runs (the ablation of that
-// choice; results are identical).
-bool fused_boxes_staged_from_env() {
-  const char* v = std::getenv("AG_FUSED_BOXES");
-  return v && std::strcmp(v, "smem") == 0;
-}
-
-// Where a launch's collision tests read the boxes from.
-enum : int {
-  kBoxesNone = 0,    // no obstacles
-  kBoxesStaged = 1,  // staged per thread: pair 0 in registers, the others in shared memory
-  kBoxesGlobal = 2,  // the slot-ordered pair copy in global memory, read when a test runs
-};
-
 // Thread slot i of the launch simulates environment order[i] (a permutation
 // that groups environments of equal rotor count and command mode, so the
 // mode branches of the controller are warp-uniform), or environment i when
 // order is NULL. A collision test that cannot hit is skipped (simulate_cmd),
-// so tests are rare after the first step; by default a test reads the
-// environment's box pairs from the slot-ordered copy in global memory, which
-// needs no shared memory. Threads of one command mode run the loop
-// compiled for that mode (simulate). The bound of 4 blocks of 128 threads
+// so tests are rare after the first step; a test reads the environment's box
+// records (EnvBoxes). Threads of one command mode run the loop compiled for
+// that mode (simulate). With boxes the bound of 4 blocks of 128 threads
 // per SM holds the kernel under 128 registers, 4 warps per SM sub-partition
 // (16 per SM); a bound of 3 (140 registers, 12 warps per SM) measured
-// slower. The staged form keeps each thread's boxes on chip for the launch
-// instead: boxes 0 and 1 in registers, the others in shared memory
-// as float4 [pair][field pair][thread], so a warp's 16-byte loads of two
-// fields are consecutive and conflict-free (a thread reads only what it
-// wrote, so no barrier is needed).
+// slower.
 // Without obstacles the kernel stays within 128 registers. A quad-only
 // semi-implicit-Euler fleet without obstacles needs about 70 (no spills),
 // and its bound of 7 blocks per SM lets a 131,072-vehicle fleet run in one
 // wave; fleets with hexa and octo rotors keep the looser bound, which
 // measured faster for them.
-template <int INTEG, bool QUAD_ONLY, bool DRAG, int BOXES>
-__global__ void __launch_bounds__(128, BOXES == kBoxesGlobal ? 4
-                                       : (BOXES == kBoxesStaged ? 3 : ((QUAD_ONLY && INTEG == kIntegSIE) ? 7 : 4)))
+template <int INTEG, bool QUAD_ONLY, bool DRAG, bool BOXES>
+__global__ void __launch_bounds__(128, !BOXES && QUAD_ONLY && INTEG == kIntegSIE ? 7 : 4)
     k_fused_step(FleetBuffers fb, StepParams P, int n_steps, int substeps) {
-  extern __shared__ float4 sm_pairs[];  // [ceil(n_obs / 2) - 1][5][blockDim.x] box pairs 1..
-  const int B = blockDim.x;
-  const uint32_t slot = blockIdx.x * B + threadIdx.x;
+  const uint32_t slot = blockIdx.x * blockDim.x + threadIdx.x;
   const bool active = slot < fb.n;
   const uint32_t env = active ? (fb.order ? fb.order[slot] : slot) : slot;
-  RegSmemBoxPairs bx;
-  bx.sm = sm_pairs + threadIdx.x;
-  bx.B = B;
-#pragma unroll
-  for (int f = 0; f < 10; ++f) bx.r[f] = make_float2(0.f, 0.f);
-  const int n_obs = (int)fb.n_obs;
-  if (BOXES == kBoxesStaged && active && n_obs > 0) {
-    const int pairs = (n_obs + 1) / 2;
-    if (fb.order) {
-      // the slot-ordered pair copy: coalesced 8-byte rows
-#pragma unroll
-      for (int f = 0; f < 10; ++f) bx.r[f] = fb.boxes_slot[(size_t)f * fb.n + slot];
-      for (int r = 10; r < pairs * 10; r += 2) {
-        const float2 lo = fb.boxes_slot[(size_t)r * fb.n + slot], hi = fb.boxes_slot[(size_t)(r + 1) * fb.n + slot];
-        bx.sm[(r - 10) / 2 * B] = make_float4(lo.x, lo.y, hi.x, hi.y);
-      }
-    } else {
-      // ungrouped (env == slot): pair up the env-ordered rows here
-      bx.reload(fb, slot);
-      for (int j = 1; j < pairs; ++j) {
-        const int k0 = 2 * j, k1 = 2 * j + 1;
-#pragma unroll
-        for (int f = 0; f < 10; f += 2) {
-          float v[4];
-#pragma unroll
-          for (int c = 0; c < 4; ++c) {  // a_f, b_f, a_f+1, b_f+1
-            const int k = (c & 1) ? k1 : k0, ff = f + (c >> 1);
-            const float raw = k < n_obs ? fb.boxes[((size_t)k * 10 + ff) * fb.n + slot] : box_pad_field(ff);
-            v[c] = staged_field(ff, raw);
-          }
-          bx.sm[((j - 1) * 5 + f / 2) * B] = make_float4(v[0], v[1], v[2], v[3]);
-        }
-      }
-    }
-  }
   uint32_t resets = 0, tests = 0;
   bool any_hit = false;
   if (active) {
     const int nrot = QUAD_ONLY ? 4 : rotor_count(fb, env);
-    if (BOXES == kBoxesGlobal) {
-      GlobalBoxPairs gx{fb.boxes_slot, fb.n, slot};
-      if (nrot == 4)
-        simulate<4, INTEG, DRAG, true>(fb, P, env, slot, n_steps, substeps, n_obs, gx, P.seed_lo, P.seed_hi, resets, any_hit, tests);
-      else if (nrot == 6)
-        simulate<6, INTEG, DRAG, true>(fb, P, env, slot, n_steps, substeps, n_obs, gx, P.seed_lo, P.seed_hi, resets, any_hit, tests);
-      else
-        simulate<8, INTEG, DRAG, true>(fb, P, env, slot, n_steps, substeps, n_obs, gx, P.seed_lo, P.seed_hi, resets, any_hit, tests);
-    } else if (BOXES == kBoxesStaged) {
-      if (nrot == 4)
-        simulate<4, INTEG, DRAG, true>(fb, P, env, slot, n_steps, substeps, n_obs, bx, P.seed_lo, P.seed_hi, resets, any_hit, tests);
-      else if (nrot == 6)
-        simulate<6, INTEG, DRAG, true>(fb, P, env, slot, n_steps, substeps, n_obs, bx, P.seed_lo, P.seed_hi, resets, any_hit, tests);
-      else
-        simulate<8, INTEG, DRAG, true>(fb, P, env, slot, n_steps, substeps, n_obs, bx, P.seed_lo, P.seed_hi, resets, any_hit, tests);
-    } else {
-      NoBoxSource none;
-      if (nrot == 4)
-        simulate<4, INTEG, DRAG, true>(fb, P, env, slot, n_steps, substeps, 0, none, P.seed_lo, P.seed_hi, resets, any_hit, tests);
-      else if (nrot == 6)
-        simulate<6, INTEG, DRAG, true>(fb, P, env, slot, n_steps, substeps, 0, none, P.seed_lo, P.seed_hi, resets, any_hit, tests);
-      else
-        simulate<8, INTEG, DRAG, true>(fb, P, env, slot, n_steps, substeps, 0, none, P.seed_lo, P.seed_hi, resets, any_hit, tests);
-    }
+    const std::conditional_t<BOXES, EnvBoxes, NoBoxSource> boxes(fb, env);
+    const int n_obs = BOXES ? (int)fb.n_obs : 0;
+    if (nrot == 4)
+      simulate<4, INTEG, DRAG, true>(fb, P, env, n_steps, substeps, n_obs, boxes, P.seed_lo, P.seed_hi, resets, any_hit, tests);
+    else if (nrot == 6)
+      simulate<6, INTEG, DRAG, true>(fb, P, env, n_steps, substeps, n_obs, boxes, P.seed_lo, P.seed_hi, resets, any_hit, tests);
+    else
+      simulate<8, INTEG, DRAG, true>(fb, P, env, n_steps, substeps, n_obs, boxes, P.seed_lo, P.seed_hi, resets, any_hit, tests);
     fb.collided[env] = any_hit ? 1 : 0;
   }
   append_compact(resets > 0u, env, fb.reset_ids, fb.n_reset);
-  if (BOXES != kBoxesNone && fb.tests_run) {  // one atomic per warp
+  if (BOXES && fb.tests_run) {  // one atomic per warp
     const unsigned t = __reduce_add_sync(0xFFFFFFFFu, tests);
     if ((threadIdx.x & 31u) == 0u && t) atomicAdd(fb.tests_run, (unsigned long long)t);
   }
@@ -199,7 +121,6 @@ __global__ void __launch_bounds__(kOrderThreads) k_order_window(FleetBuffers fb)
       uint32_t pos = key_next[key] + rank;
       for (int w = 0; w < warp; ++w) pos += warp_count[w][key];
       fb.order[base + pos] = i;
-      if (fb.slot_of) fb.slot_of[i] = base + pos;
     }
     __syncthreads();
     if (threadIdx.x < 12) {  // advance each key by its count in this sub-window
@@ -211,20 +132,28 @@ __global__ void __launch_bounds__(kOrderThreads) k_order_window(FleetBuffers fb)
   }
 }
 
-__global__ void __launch_bounds__(256) k_permute_boxes(FleetBuffers fb) {
-  const uint32_t slot = blockIdx.x * blockDim.x + threadIdx.x;
-  if (slot >= fb.n) return;
-  const uint32_t env = fb.order[slot];
-  const int n_obs = (int)fb.n_obs;
-  for (int j = 0; j < (n_obs + 1) / 2; ++j) {
-    const int k0 = 2 * j, k1 = 2 * j + 1;
+// Box records from the caller's rows and back: thread (env, box).
+__global__ void __launch_bounds__(256) k_pack_boxes(FleetBuffers fb, const float* __restrict__ src, size_t pitch,
+                                                    uint32_t k0) {
+  const uint32_t env = blockIdx.x * blockDim.x + threadIdx.x;
+  if (env >= fb.n) return;
+  float v[10];
 #pragma unroll
-    for (int f = 0; f < 10; ++f) {
-      const float a = fb.boxes[((size_t)k0 * 10 + f) * fb.n + env];
-      const float b = k1 < n_obs ? fb.boxes[((size_t)k1 * 10 + f) * fb.n + env] : box_pad_field(f);
-      fb.boxes_slot[(size_t)(j * 10 + f) * fb.n + slot] = make_float2(staged_field(f, a), staged_field(f, b));
-    }
-  }
+  for (int f = 0; f < 10; ++f) v[f] = src[((size_t)blockIdx.y * 10 + f) * pitch + env];
+  const size_t at = (size_t)(k0 + blockIdx.y) * fb.n + env;
+  fb.box_bound[at] = make_float4(v[0], v[1], v[2], sqrtf(fmaf(v[5], v[5], fmaf(v[4], v[4], v[3] * v[3]))));
+  fb.box_rest[2 * at] = make_float4(v[3], v[4], v[5], v[6]);
+  fb.box_rest[2 * at + 1] = make_float4(v[7], v[8], v[9], 0.f);
+}
+
+__global__ void __launch_bounds__(256) k_unpack_boxes(FleetBuffers fb, float* __restrict__ dst, uint32_t k0) {
+  const uint32_t env = blockIdx.x * blockDim.x + threadIdx.x;
+  if (env >= fb.n) return;
+  const size_t at = (size_t)(k0 + blockIdx.y) * fb.n + env;
+  const float4 b = fb.box_bound[at], h = fb.box_rest[2 * at], q = fb.box_rest[2 * at + 1];
+  const float v[10] = {b.x, b.y, b.z, h.x, h.y, h.z, h.w, q.x, q.y, q.z};
+#pragma unroll
+  for (int f = 0; f < 10; ++f) dst[((size_t)blockIdx.y * 10 + f) * fb.n + env] = v[f];
 }
 
 // ag_reset: resample masked environments, clear collided flags, list them.
@@ -284,18 +213,24 @@ __global__ void __launch_bounds__(256) k_plain_integrate(FleetBuffers fb, StepPa
   store_state(fb.state, n, i, s);
 }
 
-// Collision test of every environment against its boxes read from global
-// memory; the per-env hit byte goes to `collided_now`.
+// Collision test of every environment against all its boxes, from the
+// caller's rows (the allocation-free step) or the context's records; the
+// per-env hit byte goes to `collided_now`.
 __global__ void __launch_bounds__(256) k_plain_collide(FleetBuffers fb, StepParams P, uint8_t* collided_now) {
   const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= fb.n) return;
   const uint32_t n = fb.n;
   V3 p = {fb.state[0 * n + i], fb.state[1 * n + i], fb.state[2 * n + i]};
   bool hit = false;
-  for (uint32_t k = 0; k < fb.n_obs; ++k) {
-    const float* bx = fb.boxes + (size_t)k * 10 * n + i;
-    hit |= sphere_hits_box(p, P.r2, V3{bx[0], bx[n], bx[2 * n]}, V3{bx[3 * n], bx[4 * n], bx[5 * n]},
-                           Q4{bx[6 * n], bx[7 * n], bx[8 * n], bx[9 * n]});
+  if (fb.boxes) {
+    for (uint32_t k = 0; k < fb.n_obs; ++k) {
+      const float* bx = fb.boxes + (size_t)k * 10 * n + i;
+      hit |= touches(P.r2, box_dist2(p, V3{bx[0], bx[n], bx[2 * n]}, V3{bx[3 * n], bx[4 * n], bx[5 * n]},
+                                     Q4{bx[6 * n], bx[7 * n], bx[8 * n], bx[9 * n]}));
+    }
+  } else {
+    const EnvBoxes boxes(fb, i);
+    for (uint32_t k = 0; k < fb.n_obs; ++k) hit |= touches(P.r2, boxes.dist2(p, (int)k));
   }
   collided_now[i] = hit ? 1 : 0;
 }
@@ -317,7 +252,7 @@ __global__ void __launch_bounds__(256) k_plain_reset_hits(FleetBuffers fb, StepP
   const int nrot = rotor_count(fb, i);
   const float hv = hover_per_motor(fb.body[i], nrot);
   for (int k = 0; k < nrot; ++k) fb.motors[k * n + i] = hv;
-  if (fb.box_rand) redraw_boxes(fb, i, fb.slot_of ? fb.slot_of[i] : i, epoch, P.seed_lo, P.seed_hi, NoBoxes{});
+  if (fb.box_rand) redraw_boxes(fb, i, epoch, P.seed_lo, P.seed_hi);
 }
 
 __global__ void __launch_bounds__(256) k_plain_compact(FleetBuffers fb) {
@@ -326,47 +261,30 @@ __global__ void __launch_bounds__(256) k_plain_compact(FleetBuffers fb) {
   append_compact(pred, i, fb.reset_ids, fb.n_reset);
 }
 
-template <int INTEG, bool QUAD_ONLY, bool DRAG, int BOXES>
+template <int INTEG, bool QUAD_ONLY, bool DRAG, bool BOXES>
 cudaError_t launch_fused_b(const FleetBuffers& fb, const StepParams& P, int n_steps, int substeps, int B,
                            cudaStream_t st) {
   const auto kernel = k_fused_step<INTEG, QUAD_ONLY, DRAG, BOXES>;
-  // raise the dynamic shared-memory cap once per instantiation and device (the attribute is per device)
-  static std::atomic<uint64_t> attr_set{0};
-  int dev = 0;
-  cudaError_t e = cudaGetDevice(&dev);
-  if (e != cudaSuccess) return e;
-  const uint64_t bit = dev < 64 ? (1ull << dev) : 0;
-  if (!bit || !(attr_set.load(std::memory_order_acquire) & bit)) {
-    e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kFusedSmemCap);
-    if (e != cudaSuccess) return e;
-    attr_set.fetch_or(bit, std::memory_order_release);
-  }
   if (B == 0) {  // the block size with the most resident warps per SM (ties: the earlier candidate)
     int best = -1;
     for (int b : {64, 128, 96, 32}) {
-      const size_t sm = BOXES == kBoxesStaged ? fused_smem_bytes((int)fb.n_obs, b) : 0;
-      if (sm > kFusedSmemCap) continue;
       int blocks = 0;
-      e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks, kernel, b, sm);
+      const cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks, kernel, b, 0);
       if (e != cudaSuccess) return e;
       if (blocks * b > best) { best = blocks * b; B = b; }
     }
     if (best <= 0) return cudaErrorInvalidConfiguration;
   }
-  const size_t smem = BOXES == kBoxesStaged ? fused_smem_bytes((int)fb.n_obs, B) : 0;
   const unsigned grid = (fb.n + B - 1) / B;
-  kernel<<<grid, B, smem, st>>>(fb, P, n_steps, substeps);
+  kernel<<<grid, B, 0, st>>>(fb, P, n_steps, substeps);
   return cudaGetLastError();
 }
 
 template <int INTEG, bool QUAD_ONLY, bool DRAG>
 cudaError_t launch_fused_t(const FleetBuffers& fb, const StepParams& P, int n_steps, int substeps, int B,
                            cudaStream_t st) {
-  if (fb.n_obs == 0) return launch_fused_b<INTEG, QUAD_ONLY, DRAG, kBoxesNone>(fb, P, n_steps, substeps, B, st);
-  // the global pair copy is in slot order: it serves the grouped order only
-  if (fb.order && fb.boxes_slot && !fused_boxes_staged_from_env())
-    return launch_fused_b<INTEG, QUAD_ONLY, DRAG, kBoxesGlobal>(fb, P, n_steps, substeps, B, st);
-  return launch_fused_b<INTEG, QUAD_ONLY, DRAG, kBoxesStaged>(fb, P, n_steps, substeps, B, st);
+  return fb.n_obs == 0 ? launch_fused_b<INTEG, QUAD_ONLY, DRAG, false>(fb, P, n_steps, substeps, B, st)
+                       : launch_fused_b<INTEG, QUAD_ONLY, DRAG, true>(fb, P, n_steps, substeps, B, st);
 }
 
 template <int INTEG>
@@ -383,7 +301,7 @@ cudaError_t launch_fused_i(const FleetBuffers& fb, const StepParams& P, int n_st
 
 }  // namespace
 
-FusedTuning fused_tuning_from_env(int n_obs) {
+FusedTuning fused_tuning_from_env() {
   FusedTuning t;
   t.sorted = true;
   t.block = 0;
@@ -392,7 +310,7 @@ FusedTuning fused_tuning_from_env(int n_obs) {
   if (const char* v = std::getenv("AG_FUSED_SKIP")) t.skip = std::strcmp(v, "0") != 0;
   if (const char* v = std::getenv("AG_FUSED_BLOCK")) {
     int b = std::atoi(v);
-    if (b >= 32 && b <= 128 && b % 32 == 0 && fused_smem_bytes(n_obs, b) <= kFusedSmemCap) t.block = b;
+    if (b >= 32 && b <= 128 && b % 32 == 0) t.block = b;
   }
   return t;
 }
@@ -402,7 +320,7 @@ cudaError_t launch_fused_step(const FleetBuffers& fb_in, const StepParams& P, in
   cudaError_t e = cudaMemsetAsync(fb_in.n_reset, 0, sizeof(uint32_t), st);
   if (e == cudaSuccess && fb_in.tests_run) e = cudaMemsetAsync(fb_in.tests_run, 0, sizeof(unsigned long long), st);
   if (e != cudaSuccess) return e;
-  const FusedTuning t = fused_tuning_from_env((int)fb_in.n_obs);
+  const FusedTuning t = fused_tuning_from_env();
   FleetBuffers fb = fb_in;
   if (!t.sorted) fb.order = nullptr;
   StepParams Pl = P;
@@ -411,22 +329,19 @@ cudaError_t launch_fused_step(const FleetBuffers& fb_in, const StepParams& P, in
                                  : launch_fused_i<kIntegSIE>(fb, Pl, n_steps, substeps, t.block, st);
 }
 
-cudaError_t launch_build_order(const FleetBuffers& fb, uint32_t* scratch, cudaStream_t st) {
-  (void)scratch;
+cudaError_t launch_build_order(const FleetBuffers& fb, cudaStream_t st) {
   k_order_window<<<(fb.n + kOrderWindow - 1) / kOrderWindow, kOrderThreads, 0, st>>>(fb);
-  cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
-  return launch_permute_boxes(fb, st);
+  return cudaGetLastError();
 }
 
-size_t order_scratch_words(uint32_t n) {
-  (void)n;
-  return 1;
+cudaError_t launch_pack_boxes(const FleetBuffers& fb, const float* src, size_t pitch, uint32_t k0, uint32_t count,
+                              cudaStream_t st) {
+  k_pack_boxes<<<dim3((fb.n + 255) / 256, count), 256, 0, st>>>(fb, src, pitch, k0);
+  return cudaGetLastError();
 }
 
-cudaError_t launch_permute_boxes(const FleetBuffers& fb, cudaStream_t st) {
-  if (fb.n_obs == 0 || !fb.order || !fb.boxes_slot) return cudaSuccess;
-  k_permute_boxes<<<(fb.n + 255) / 256, 256, 0, st>>>(fb);
+cudaError_t launch_unpack_boxes(const FleetBuffers& fb, float* dst, uint32_t k0, uint32_t count, cudaStream_t st) {
+  k_unpack_boxes<<<dim3((fb.n + 255) / 256, count), 256, 0, st>>>(fb, dst, k0);
   return cudaGetLastError();
 }
 

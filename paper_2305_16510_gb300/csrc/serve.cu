@@ -44,7 +44,7 @@ namespace {
 
 // One active request as the kernel sees it.
 struct ServeDesc {
-  FleetBuffers fb;          // its own buffers (quadrotors, boxes in slot order)
+  FleetBuffers fb;          // its own buffers (quadrotors)
   uint32_t seed_lo, seed_hi;
   int steps;                // steps in this launch
   uint32_t block_begin;     // first block of this request in the launch
@@ -53,7 +53,7 @@ struct ServeDesc {
 constexpr int kServeBlock = 128;
 
 template <int INTEG, bool DRAG>
-__global__ void __launch_bounds__(kServeBlock) k_serve_step(const ServeDesc* __restrict__ table, int n_req,
+__global__ void __launch_bounds__(kServeBlock, 4) k_serve_step(const ServeDesc* __restrict__ table, int n_req,
                                                            StepParams P, int substeps) {
   __shared__ int s_req;
   if (threadIdx.x == 0) {  // last request whose first block is <= this block
@@ -69,10 +69,9 @@ __global__ void __launch_bounds__(kServeBlock) k_serve_step(const ServeDesc* __r
   const uint32_t slot = (blockIdx.x - d.block_begin) * blockDim.x + threadIdx.x;
   if (slot >= d.fb.n || d.steps <= 0) return;
   const uint32_t env = d.fb.order[slot];
-  GlobalBoxPairs bx{d.fb.boxes_slot, d.fb.n, slot};
   uint32_t resets = 0, tests = 0;
   bool hit = false;
-  simulate<4, INTEG, DRAG>(d.fb, P, env, slot, d.steps, substeps, (int)d.fb.n_obs, bx, d.seed_lo, d.seed_hi, resets,
+  simulate<4, INTEG, DRAG>(d.fb, P, env, d.steps, substeps, (int)d.fb.n_obs, EnvBoxes(d.fb, env), d.seed_lo, d.seed_hi, resets,
                            hit, tests);
 }
 
@@ -128,13 +127,13 @@ class SlabAllocator {
 size_t align256(size_t b) { return (b + 255) & ~size_t(255); }
 
 // Device bytes one request needs (state, motors, body, targets, modes, epoch,
-// collided, reset ids, order, boxes twice, order scratch).
+// collided, reset ids and count, order, box records and the staging of one
+// box's rows).
 size_t request_bytes(size_t n, size_t n_obs) {
   size_t b = 0;
   b += align256(13 * n * 4) + align256(8 * n * 4) + align256(4 * n * 4) + align256(4 * n * 4);
   b += align256(n) + align256(n * 4) + align256(n) + align256(n * 4) + align256(4) + align256(n * 4);
-  b += align256(n_obs * 10 * n * 4) + align256(box_pair_elems(n, n_obs) * 8) +
-       align256(order_scratch_words((uint32_t)n) * 4);
+  b += align256(n_obs * n * 16) + align256(n_obs * n * 32) + align256(n_obs ? 10 * n * 4 : 0);
   return b;
 }
 
@@ -147,7 +146,7 @@ struct ServeRequest {
   std::chrono::steady_clock::time_point t_submit, t_done;
   size_t offset = 0;
   agk::FleetBuffers fb{};
-  uint32_t* order_scratch = nullptr;
+  float* box_stage = nullptr;  // [10][n] one box's rows on their way from host memory
   uint32_t remaining = 0;
   bool started = false;
   bool done = false;
@@ -208,19 +207,28 @@ void carve(ag_server* s, ServeRequest* r) {
   f.reset_ids = (uint32_t*)take(n * 4);
   f.n_reset = (uint32_t*)take(4);
   f.order = (uint32_t*)take(n * 4);
-  f.boxes = (float*)take(n_obs * 10 * n * 4);
-  f.boxes_slot = (float2*)take(agk::box_pair_elems(n, n_obs) * 8);
-  r->order_scratch = (uint32_t*)take(agk::order_scratch_words((uint32_t)n) * 4);
+  f.box_bound = (float4*)take(n_obs * n * 16);
+  f.box_rest = (float4*)take(n_obs * n * 32);
+  r->box_stage = (float*)take(n_obs ? 10 * n * 4 : 0);
   f.n = (uint32_t)n;
   f.n_quad = (uint32_t)n;
   f.n_obs = (uint32_t)n_obs;
-  if (n_obs == 0) { f.boxes = nullptr; f.boxes_slot = nullptr; }
+  if (n_obs == 0) f.box_bound = f.box_rest = nullptr;
 }
 
 __global__ void k_fill_body(float* body, uint32_t n, float m, float jx, float jy, float jz) {
   uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
   body[i] = m; body[n + i] = jx; body[2 * n + i] = jy; body[3 * n + i] = jz;
+}
+
+// Device memory of the server's own device, which a kernel can read in place.
+bool on_device(const void* p, int device) {
+  cudaPointerAttributes pa;
+  const bool own = cudaPointerGetAttributes(&pa, p) == cudaSuccess && pa.type == cudaMemoryTypeDevice &&
+                   pa.device == device;
+  cudaGetLastError();
+  return own;
 }
 
 // Uploads a newly admitted request's inputs and draws its initial states.
@@ -243,12 +251,20 @@ cudaError_t start_request(ag_server* s, ServeRequest* r) {
       e = cudaGetLastError();
     }
   }
-  if (e == cudaSuccess && in.n_obstacles)
-    e = cudaMemcpy2DAsync(f.boxes, n * 4, in.boxes, pitch * 4, n * 4, (size_t)in.n_obstacles * 10, cudaMemcpyDefault,
-                          st);
+  if (e == cudaSuccess && in.n_obstacles) {
+    if (on_device(in.boxes, s->device)) {
+      e = agk::launch_pack_boxes(f, in.boxes, pitch, 0, in.n_obstacles, st);
+    } else {
+      for (uint32_t k = 0; k < in.n_obstacles && e == cudaSuccess; ++k) {
+        e = cudaMemcpy2DAsync(r->box_stage, n * 4, in.boxes + (size_t)k * 10 * pitch, pitch * 4, n * 4, 10,
+                              cudaMemcpyDefault, st);
+        if (e == cudaSuccess) e = agk::launch_pack_boxes(f, r->box_stage, n, k, 1, st);
+      }
+    }
+  }
   if (e == cudaSuccess) e = cudaMemsetAsync(f.epoch, 0, n * 4, st);
   if (e == cudaSuccess) e = agk::launch_reset(f, nullptr, (uint32_t)(in.seed & 0xFFFFFFFFu), (uint32_t)(in.seed >> 32), st);
-  if (e == cudaSuccess) e = agk::launch_build_order(f, r->order_scratch, st);
+  if (e == cudaSuccess) e = agk::launch_build_order(f, st);
   return e;
 }
 

@@ -12,6 +12,7 @@
 //   reward = -crash after a collision, else -|p - g| - w_v |v| - w_omega |Omega|
 //   done   = collided or |p - g| > max_dist or steps >= max_steps
 #include <cstdint>
+#include <type_traits>
 
 #include <cuda_runtime.h>
 
@@ -39,30 +40,6 @@ __device__ __forceinline__ void observe(const VState& s, V3 g, float* o) {
   o[6] = sgn * s.q.w; o[7] = sgn * s.q.x; o[8] = sgn * s.q.y; o[9] = sgn * s.q.z;
   o[10] = s.w.x; o[11] = s.w.y; o[12] = s.w.z;
 }
-
-// Boxes of environment env read two at a time from the env-ordered array
-// (plain loads: a re-draw in the same launch rewrites them).
-struct EnvBoxPairs {
-  const float* boxes;
-  uint32_t n, env;
-  __device__ __forceinline__ float2 at(int j, int f, int n_obs) const {
-    const int k0 = 2 * j, k1 = 2 * j + 1;
-    return make_float2(staged_field(f, boxes[((size_t)k0 * 10 + f) * n + env]),
-                       staged_field(f, k1 < n_obs ? boxes[((size_t)k1 * 10 + f) * n + env] : box_pad_field(f)));
-  }
-  __device__ __forceinline__ bool any_hit_min(V3 p, float r2, int n_obs, float& m) const {
-    const float2 px = dup2(p.x), py = dup2(p.y), pz = dup2(p.z);
-    bool hit = false;
-    m = __int_as_float(0x7f800000);
-    for (int j = 0; j < (n_obs + 1) >> 1; ++j)
-      hit |= pair_hits_min(px, py, pz, r2, at(j, 0, n_obs), at(j, 1, n_obs), at(j, 2, n_obs), at(j, 3, n_obs),
-                           at(j, 4, n_obs), at(j, 5, n_obs), at(j, 6, n_obs), at(j, 7, n_obs), at(j, 8, n_obs),
-                           at(j, 9, n_obs), m);
-    return hit;
-  }
-  __device__ __forceinline__ NoBoxes staged() const { return {}; }
-  __device__ __forceinline__ void reload(const FleetBuffers&, uint32_t) {}
-};
 
 // Reward, termination and in-place reset of environment i after its step
 // (s: its state after the step; hit: it collided, and the step already
@@ -105,9 +82,9 @@ __device__ __forceinline__ void write_obs(const ReachArgs& a, const float* stage
 // command mode, so warps are mode-uniform without a grouping permutation.
 // Without boxes the step is memory-latency bound: a bound of 14 blocks (28
 // warps) per SM measured best, against 16 blocks (64 registers, more spills)
-// and 20 (48 registers). With boxes it keeps 12 warps per SM (170 registers).
+// and 20 (48 registers). With boxes 8 blocks (16 warps, 128 registers).
 template <int INTEG, bool DRAG, bool BOXES>
-__global__ void __launch_bounds__(kTaskBlock, BOXES ? 384 / kTaskBlock : 896 / kTaskBlock)
+__global__ void __launch_bounds__(kTaskBlock, BOXES ? 512 / kTaskBlock : 896 / kTaskBlock)
     k_reach_step(ReachArgs a, StepParams P, int substeps) {
   __shared__ float stage[kTaskBlock * kObs];  // odd row length: conflict-free
   const FleetBuffers& fb = a.fb;
@@ -125,28 +102,16 @@ __global__ void __launch_bounds__(kTaskBlock, BOXES ? 384 / kTaskBlock : 896 / k
     for (int k = 0; k < 4; ++k) t[k] = fmaf(a.scale[k], fminf(fmaxf(v[k], -1.f), 1.f), a.offset[k]);
     const Command cm = prepare_command(fb.modes[i], t[0], t[1], t[2], t[3]);
     const int nrot = rotor_count(fb, i);
-    // environment i's place in the slot-ordered box copy (a re-draw updates it there)
-    const uint32_t slot = fb.slot_of ? fb.slot_of[i] : i;
-    const int n_obs = (int)fb.n_obs;
     bool hit = false;
     VState s;
-    if (BOXES) {
-      EnvBoxPairs bx{fb.boxes, n, i};
-      if (nrot == 4)
-        s = simulate_cmd<4, INTEG, DRAG>(fb, P, i, slot, cm, 1, substeps, n_obs, bx, a.seed_lo, a.seed_hi, resets, hit, tests);
-      else if (nrot == 6)
-        s = simulate_cmd<6, INTEG, DRAG>(fb, P, i, slot, cm, 1, substeps, n_obs, bx, a.seed_lo, a.seed_hi, resets, hit, tests);
-      else
-        s = simulate_cmd<8, INTEG, DRAG>(fb, P, i, slot, cm, 1, substeps, n_obs, bx, a.seed_lo, a.seed_hi, resets, hit, tests);
-    } else {
-      NoBoxSource none;
-      if (nrot == 4)
-        s = simulate_cmd<4, INTEG, DRAG>(fb, P, i, slot, cm, 1, substeps, 0, none, a.seed_lo, a.seed_hi, resets, hit, tests);
-      else if (nrot == 6)
-        s = simulate_cmd<6, INTEG, DRAG>(fb, P, i, slot, cm, 1, substeps, 0, none, a.seed_lo, a.seed_hi, resets, hit, tests);
-      else
-        s = simulate_cmd<8, INTEG, DRAG>(fb, P, i, slot, cm, 1, substeps, 0, none, a.seed_lo, a.seed_hi, resets, hit, tests);
-    }
+    const std::conditional_t<BOXES, EnvBoxes, NoBoxSource> boxes(fb, i);
+    const int n_obs = BOXES ? (int)fb.n_obs : 0;
+    if (nrot == 4)
+      s = simulate_cmd<4, INTEG, DRAG>(fb, P, i, cm, 1, substeps, n_obs, boxes, a.seed_lo, a.seed_hi, resets, hit, tests);
+    else if (nrot == 6)
+      s = simulate_cmd<6, INTEG, DRAG>(fb, P, i, cm, 1, substeps, n_obs, boxes, a.seed_lo, a.seed_hi, resets, hit, tests);
+    else
+      s = simulate_cmd<8, INTEG, DRAG>(fb, P, i, cm, 1, substeps, n_obs, boxes, a.seed_lo, a.seed_hi, resets, hit, tests);
     fb.collided[i] = hit ? 1 : 0;
 #pragma unroll
     for (int k = 0; k < 4; ++k) fb.targets[k * n + i] = t[k];  // the commands, as ag_set_commands keeps them

@@ -1,0 +1,67 @@
+"""Box records: the collision test reads every box's circumscribed sphere and
+runs the exact sphere-vs-box test only on those within reach. Its decisions
+must be those of the exact test on every box (AG_FUSED_SKIP=0), bit for bit,
+and the records must hold what ag_set_obstacles was given."""
+import numpy as np
+import pytest
+import torch
+
+from paper_2305_16510_gb300 import workloads as W
+
+from harness import gpu_fleet
+
+pytestmark = pytest.mark.gpu
+
+
+def _case(n_obs, seed):
+    """Long thin, flat and large boxes around the vehicles, quaternion norms off
+    by up to the admitted 1e-4 of the squared norm, some vehicles at positions
+    that are huge or not finite."""
+    n = 3001
+    w = W.Workload("records", n, 2, 1, n_obs, n, 0, 0, mode_mix=(0, 1, 2, 3))
+    inp = W.make_inputs(w, seed)
+    rng = np.random.default_rng(seed)
+    boxes = inp.boxes.copy()
+    boxes[:, 0:3] = rng.uniform(-3, 3, (n_obs, 3, n))
+    boxes[:, 3:6] = rng.choice([0.01, 0.1, 0.5, 2.5], (n_obs, 3, n)) / np.sqrt(n_obs)
+    boxes[:, 6:10] *= np.sqrt(1 + rng.uniform(-9e-5, 9e-5, (n_obs, 1, n)))
+    return w, W.Inputs(inp.modes, inp.targets, inp.body, np.ascontiguousarray(boxes, np.float32))
+
+
+@pytest.mark.parametrize("n_obs", [1, 2, 31, 32, 33, 64])
+def test_sphere_first_tests_decide_as_the_exact_test(n_obs, monkeypatch):
+    w, inp = _case(n_obs, 60 + n_obs)
+    outs = []
+    for skip in ("1", "0"):
+        monkeypatch.setenv("AG_FUSED_SKIP", skip)
+        fl = gpu_fleet(w, inp, 5)
+        fl.reset(None, 5)
+        st = fl.state()
+        st[0:3, 0:40:8] = torch.tensor([float("inf"), float("nan"), -float("inf"), 1e19, 3e38], device="cuda")
+        st[0, 3:43:8] = 1e20
+        st[1, 4:44:8] = -2e6
+        fl.set_state(st)
+        got = []
+        for steps in (1, 1, 1, 7, 60):   # single steps want only the decision, longer calls the clearance too
+            fl.step(steps)
+            col, ids = fl.events()
+            got += [fl.state(), fl.motors(), fl.epoch(), col, ids.sort().values]
+        outs.append([t.cpu().numpy() for t in got])
+        fl.close()
+    for a, b in zip(*outs):
+        np.testing.assert_array_equal(a, b)
+    assert (outs[0][-3] > 1).sum() > 50   # collisions happened
+
+
+@pytest.mark.parametrize("n_obs", [1, 3])
+def test_obstacles_round_trip_from_host_and_device(n_obs):
+    w, inp = _case(n_obs, 7)
+    fl = gpu_fleet(w, inp, 5)
+    np.testing.assert_array_equal(fl.obstacles().cpu().numpy(), inp.boxes)
+    from paper_2305_16510_gb300 import _abi
+    _abi.ag_set_obstacles(fl.ctx, inp.boxes[:, :, ::-1].copy())        # pageable host memory
+    host = np.empty_like(inp.boxes)
+    _abi.ag_get_obstacles(fl.ctx, host)
+    fl.synchronize()
+    np.testing.assert_array_equal(host, inp.boxes[:, :, ::-1])
+    fl.close()
