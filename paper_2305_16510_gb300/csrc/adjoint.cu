@@ -152,7 +152,7 @@ template <bool FULL_TAPE> struct Record {
   const StepParams& P;
   uint32_t slot, env;
   template <int NROT, int MODE> __device__ __forceinline__ void run() const {
-    const uint32_t n = ab.n;
+    const uint32_t n = ab.n, ns = ab.n_slots;
     Vehicle<NROT> x;
     load_vehicle(ab.state, ab.motors, n, env, x);
     ab.inv_q0[slot] = 1.f / sqrtf(dot4(x.s.q));
@@ -167,8 +167,8 @@ template <bool FULL_TAPE> struct Record {
     int to_ckpt = 0;
     for (int t = 0; t < ab.n_steps; ++t) {
       if (!FULL_TAPE && to_ckpt-- == 0) {
-        store_vehicle(ckpt, ckpt + 13 * (size_t)n, n, slot, x);
-        ckpt += 21 * (size_t)n;
+        store_vehicle(ckpt, ckpt + 13 * (size_t)ns, ns, slot, x);
+        ckpt += 21 * (size_t)ns;
         to_ckpt = ab.K - 1;
       }
       const VState start = x.s;
@@ -177,13 +177,13 @@ template <bool FULL_TAPE> struct Record {
       forward_step<NROT, MODE>(x, cm, b, P, wf, pass);
       all_pass &= pass;
       if (FULL_TAPE) {
-        store_entry(entry, n, start, wf, pass);
-        entry += 4 * (size_t)n;
+        store_entry(entry, ns, start, wf, pass);
+        entry += 4 * (size_t)ns;
       }
       const V3 e = x.s.p - goal;
       loss += fmaf(ab.w_omega, dot(x.s.w, x.s.w), ab.w_pos * dot(e, e));
     }
-    if (FULL_TAPE) store_entry(entry, n, x.s, 0.f, 0u);  // entry H: the end state
+    if (FULL_TAPE) store_entry(entry, ns, x.s, 0.f, 0u);  // entry H: the end state
     store_vehicle(ab.state, ab.motors, n, env, x);
     ab.loss[env] = loss;
     ab.saturated[env] = all_pass == (1u << NROT) - 1u ? 0 : 1;
@@ -199,8 +199,8 @@ constexpr int kRecordBlock = 32;
 template <bool FULL_TAPE>
 __global__ void __launch_bounds__(kRecordBlock) k_record(AdjointBuffers ab, StepParams P) {
   const uint32_t slot = blockIdx.x * blockDim.x + threadIdx.x;
-  if (slot >= ab.n) return;
-  const uint32_t env = ab.order[slot];
+  const uint32_t env = ab.order[slot];  // n_slots is a multiple of the block
+  if (env >= ab.n) return;
   by_airframe_and_mode(rotors_of(ab, env), mode_of(ab, env), Record<FULL_TAPE>{ab, P, slot, env});
 }
 
@@ -486,7 +486,7 @@ template <bool FULL_TAPE> struct Sweep {
   float4 (*ring)[4][kAdjointBlock];  // [kSweepStages][4][lane]
   V3 (&gains)[4];
   template <int NROT, int MODE> __device__ __forceinline__ void run() const {
-    const size_t n = ab.n;
+    const size_t n = ab.n, ns = ab.n_slots;
     const uint32_t lane = threadIdx.x;
     const Body b = body_at(ab, env);
     const Command cm = command_at<MODE>(ab, env);
@@ -503,12 +503,12 @@ template <bool FULL_TAPE> struct Sweep {
     const int H = ab.n_steps;
     V3 pn, wn;        // position and body rate after the step in hand
     Q4 q0;            // unit attitude at step 0
-    const size_t row = 4 * n;
+    const size_t row = 4 * ns;
     if (FULL_TAPE) {
       const float4* const tape = ab.tape + slot;
       {
         const float4* e = tape + (size_t)H * row;
-        const float4 e0 = e[0], e1 = e[n], e3 = e[3 * n];
+        const float4 e0 = e[0], e1 = e[ns], e3 = e[3 * ns];
         pn = {e0.x, e0.y, e0.z};
         wn = {e1.z, e1.w, e3.x};
       }
@@ -516,7 +516,7 @@ template <bool FULL_TAPE> struct Sweep {
         if (t >= 0) {
           const float4* e = tape + (size_t)t * row;
 #pragma unroll
-          for (int r = 0; r < 4; ++r) copy16_async(&ring[t % kSweepStages][r][lane], e + r * n);
+          for (int r = 0; r < 4; ++r) copy16_async(&ring[t % kSweepStages][r][lane], e + r * ns);
         }
         asm volatile("cp.async.commit_group;" ::: "memory");
       };
@@ -538,14 +538,14 @@ template <bool FULL_TAPE> struct Sweep {
         const int t0 = seg * K, len = H - t0 < K ? H - t0 : K;
         float4* const tape = ab.tape + slot;
         Vehicle<NROT> v;
-        const float* ck = ab.ckpt + (size_t)seg * 21 * n;
-        load_vehicle(ck, ck + 13 * n, (uint32_t)n, slot, v);
+        const float* ck = ab.ckpt + (size_t)seg * 21 * ns;
+        load_vehicle(ck, ck + 13 * ns, (uint32_t)ns, slot, v);
         for (int t = 0; t < len; ++t) {
           const VState start = v.s;
           float wf;
           uint32_t pass = 0;
           forward_step<NROT, MODE>(v, cm, b, P, wf, pass);
-          store_entry(tape + (size_t)t * row, n, start, wf, pass);
+          store_entry(tape + (size_t)t * row, ns, start, wf, pass);
         }
         if (t0 + len == H) {  // the later segments' first entries carry pn and wn across the others
           pn = v.s.p;
@@ -553,7 +553,7 @@ template <bool FULL_TAPE> struct Sweep {
         }
         for (int t = len - 1; t >= 0; --t) {
           const float4* e = tape + (size_t)t * row;
-          const TapeStep x = unpack(e[0], e[n], e[2 * n], e[3 * n]);
+          const TapeStep x = unpack(e[0], e[ns], e[2 * ns], e[3 * ns]);
           backward_step<NROT, MODE>(x, pn, wn, cm, b, P, goal, cp2, cw2, z, gb);
           pn = x.p;
           wn = x.w;
@@ -604,10 +604,9 @@ __global__ void __maxnreg__(128) k_adjoint(AdjointBuffers ab, StepParams P) {
   __shared__ float4 ring[FULL_TAPE ? kSweepStages : 1][4][kAdjointBlock];
   const uint32_t slot = blockIdx.x * kAdjointBlock + threadIdx.x;
   V3 gains[4] = {{0.f, 0.f, 0.f}, {0.f, 0.f, 0.f}, {0.f, 0.f, 0.f}, {0.f, 0.f, 0.f}};
-  if (slot < ab.n) {
-    const uint32_t env = ab.order[slot];
+  const uint32_t env = ab.order[slot];  // n_slots is a multiple of the block
+  if (env < ab.n)
     by_airframe_and_mode(rotors_of(ab, env), mode_of(ab, env), Sweep<FULL_TAPE>{ab, P, slot, env, ring, gains});
-  }
   __syncwarp();
   const float v12[12] = {gains[0].x, gains[0].y, gains[0].z, gains[1].x, gains[1].y, gains[1].z,
                          gains[2].x, gains[2].y, gains[2].z, gains[3].x, gains[3].y, gains[3].z};
@@ -643,14 +642,14 @@ __global__ void __launch_bounds__(kRedThreads) k_reduce_gains(const float* parti
 }  // namespace
 
 cudaError_t launch_record(const AdjointBuffers& ab, const StepParams& P, cudaStream_t st) {
-  const unsigned blocks = (ab.n + kRecordBlock - 1) / kRecordBlock;
+  const unsigned blocks = ab.n_slots / kRecordBlock;
   if (ab.full_tape) k_record<true><<<blocks, kRecordBlock, 0, st>>>(ab, P);
   else k_record<false><<<blocks, kRecordBlock, 0, st>>>(ab, P);
   return cudaGetLastError();
 }
 
 cudaError_t launch_adjoint(const AdjointBuffers& ab, const StepParams& P, cudaStream_t st) {
-  const unsigned blocks = (unsigned)adjoint_warps(ab.n);
+  const unsigned blocks = ab.n_slots / kAdjointBlock;
   if (ab.full_tape) k_adjoint<true><<<blocks, kAdjointBlock, 0, st>>>(ab, P);
   else k_adjoint<false><<<blocks, kAdjointBlock, 0, st>>>(ab, P);
   cudaError_t e = cudaGetLastError();

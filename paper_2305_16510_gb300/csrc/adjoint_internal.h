@@ -8,14 +8,12 @@
 
 namespace agk {
 
-// Warps (blocks of the reverse sweep) of a fleet: one partial gain sum each.
-constexpr size_t adjoint_warps(size_t n) { return (n + 31) / 32; }
 // float4 words of one tape entry of one vehicle.
 constexpr int kTapeWords = 4;
 
 // Device buffers of one recorded rollout and its adjoint. Arrays marked
-// "slot" are indexed by thread slot (environment order[slot]), the others by
-// environment. With full_tape the tape holds the entries of every step and the
+// "slot" have n_slots columns, one per thread slot (environment order[slot],
+// none in the padding); the others are indexed by environment. With full_tape the tape holds the entries of every step and the
 // end state; else it holds one segment's K entries, and checkpoint s holds
 // the state (13 rows) and motors (8 rows) at step s * K.
 struct AdjointBuffers {
@@ -24,11 +22,11 @@ struct AdjointBuffers {
   const float* body;           // [4][n]
   const uint8_t* modes;        // [n] command mode per env (values above 3 act as a wrench)
   const float* targets;        // [4][n] command targets
-  const uint32_t* order;       // [n] thread slot -> environment, grouped by rotor type and mode
+  const uint32_t* order;       // [n_slots] thread slot -> environment, grouped by rotor type and mode
   const float* p_goal;         // [3][n]
-  float* ckpt;                 // [S][21][n] slot (NULL with full_tape)
-  float4* tape;                // [n_steps + 1][4][n] (full_tape) or [K][4][n], slot
-  float* inv_q0;               // [n] slot: 1 / |q_0| of the given initial quaternion
+  float* ckpt;                 // [S][21] slot (NULL with full_tape)
+  float4* tape;                // [n_steps + 1][4] (full_tape) or [K][4], slot
+  float* inv_q0;               // slot: 1 / |q_0| of the given initial quaternion
   float* loss;                 // [n]
   uint8_t* saturated;          // [n] some motor hit a clamp during the record
   const float* loss_weights;   // [n] upstream gradient of each env's loss (NULL = 1)
@@ -36,8 +34,8 @@ struct AdjointBuffers {
   float* grad_gains_env;       // [12][n]
   float* grad_targets;         // [4][n]
   float* grad_gains;           // [12]
-  float* partial;              // [12][adjoint_warps(n)]
-  uint32_t n, n_quad, n_hexa, n_octo;
+  float* partial;              // [12][n_slots / 32]: one sum per warp
+  uint32_t n, n_slots, n_quad, n_hexa, n_octo;
   int n_steps, K;
   int full_tape;               // 1: the record wrote the whole horizon's tape
   float w_pos, w_omega;

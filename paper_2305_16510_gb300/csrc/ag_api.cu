@@ -155,8 +155,8 @@ namespace {
 
 size_t buffer_bytes(const ag_config* c) {
   size_t n = c->n_envs;
-  size_t per = sizeof(float) * (13 + 8 + 4 + 4 + 4 + 4) + sizeof(uint32_t) * 4 + 3 /* modes, collided, hits */ + 1;
-  return n * per + agk::box_record_bytes(n, c->n_obstacles) + (c->n_obstacles ? 10 * n * sizeof(float) : 0) +
+  size_t per = sizeof(float) * (13 + 8 + 4 + 4 + 4) + sizeof(uint32_t) * 3 + 3 /* modes, collided, hits */ + 1;
+  return n * per + agk::OrderLayout{c->n_envs, c->n_quad, c->n_hexa}.total() * sizeof(uint32_t) + agk::box_record_bytes(n, c->n_obstacles) + (c->n_obstacles ? 10 * n * sizeof(float) : 0) +
          sizeof(uint32_t) + sizeof(unsigned long long);
 }
 
@@ -254,7 +254,7 @@ void free_all(ag_ctx* ctx) {
   if (ctx->reach_steps) cudaFree(ctx->reach_steps);
   agk::FleetBuffers& f = ctx->fb;
   void* ptrs[] = {f.state, f.motors, f.body, f.modes, f.targets, f.box_bound, f.box_rest, f.epoch, f.collided, f.reset_ids,
-                  f.n_reset, f.tests_run, f.cmd, f.wrench, f.resets, f.hits, f.order, ctx->mask_dev,
+                  f.n_reset, f.tests_run, f.cmd, f.resets, f.hits, f.order, ctx->mask_dev,
                   ctx->box_stage, (void*)f.box_rand};
   for (void* p : ptrs)
     if (p) cudaFree(p);
@@ -359,12 +359,13 @@ ag_status ag_create(const ag_config* cfg, void* cuda_stream, ag_ctx** out) {
   if (e == cudaSuccess) e = alloc(ctx, &f.n_reset, 1);
   if (e == cudaSuccess) e = alloc(ctx, &f.tests_run, 1);
   if (e == cudaSuccess) e = alloc(ctx, &f.cmd, 4 * n);
-  if (e == cudaSuccess) e = alloc(ctx, &f.wrench, 4 * n);
+  f.wrench = f.cmd;  // the allocation stage reads an environment's command before it writes its wrench
   if (e == cudaSuccess) e = alloc(ctx, &f.resets, n);
   if (e == cudaSuccess) e = alloc(ctx, &f.hits, n);
   if (e == cudaSuccess) e = alloc(ctx, &ctx->mask_dev, n);
   if (e == cudaSuccess) e = alloc(ctx, &ctx->check_dev, 1);
-  if (e == cudaSuccess) e = alloc(ctx, &f.order, n);
+  f.n_slots = agk::OrderLayout{cfg->n_envs, cfg->n_quad, cfg->n_hexa}.total();
+  if (e == cudaSuccess) e = alloc(ctx, &f.order, f.n_slots);
   if (e != cudaSuccess) {
     g_create_error = std::string("device allocation failed: ") + cudaGetErrorString(e);
     cudaGetLastError();

@@ -20,7 +20,7 @@ namespace {
 // the checkpoints the sweep recomputes it from.
 ag_status ensure_adjoint(ag_ctx* ctx, int n_steps, int K) {
   agk::AdjointBuffers& a = ctx->adj;
-  const size_t n = ctx->cfg.n_envs;
+  const size_t n = ctx->cfg.n_envs, slots = ctx->fb.n_slots;
   const size_t n_ckpt = (size_t)(n_steps + K - 1) / K;
   cudaError_t e = cudaSuccess;
   if (!a.loss) {
@@ -29,11 +29,11 @@ ag_status ensure_adjoint(ag_ctx* ctx, int n_steps, int K) {
     if (e == cudaSuccess) e = alloc(ctx, &pg, 3 * n);
     if (e == cudaSuccess) e = alloc(ctx, &a.saturated, n);
     if (e == cudaSuccess) e = alloc(ctx, &lw, n);
-    if (e == cudaSuccess) e = alloc(ctx, &a.inv_q0, n);
+    if (e == cudaSuccess) e = alloc(ctx, &a.inv_q0, slots);
     if (e == cudaSuccess) e = alloc(ctx, &a.grad_x0, 13 * n);
     if (e == cudaSuccess) e = alloc(ctx, &a.grad_gains_env, 12 * n);
     if (e == cudaSuccess) e = alloc(ctx, &a.grad_targets, 4 * n);
-    if (e == cudaSuccess) e = alloc(ctx, &a.partial, 12 * agk::adjoint_warps(n));
+    if (e == cudaSuccess) e = alloc(ctx, &a.partial, 12 * (slots / 32));
     if (e == cudaSuccess) e = alloc(ctx, &a.grad_gains, 12);
     a.p_goal = pg;
     a.loss_weights = lw;
@@ -50,7 +50,7 @@ ag_status ensure_adjoint(ag_ctx* ctx, int n_steps, int K) {
       return AG_ERR_OOM;
     }
   }
-  const size_t entry_bytes = agk::kTapeWords * n * sizeof(float4);
+  const size_t entry_bytes = agk::kTapeWords * slots * sizeof(float4);
   const size_t held = (size_t)ctx->adj_tape_cap * entry_bytes;
   auto free_tape = [&]() {
     if (a.tape) {
@@ -66,7 +66,7 @@ ag_status ensure_adjoint(ag_ctx* ctx, int n_steps, int K) {
     const uint64_t budget = ctx->cfg.hbm_budget_bytes;
     if (budget == 0 || ctx->bytes - held + full * entry_bytes <= budget) {
       free_tape();
-      if (alloc(ctx, &a.tape, full * agk::kTapeWords * n) == cudaSuccess) {
+      if (alloc(ctx, &a.tape, full * agk::kTapeWords * slots) == cudaSuccess) {
         ctx->adj_tape_cap = full;
       } else {
         cudaGetLastError();  // an out-of-memory cudaMalloc leaves no sticky error
@@ -79,7 +79,7 @@ ag_status ensure_adjoint(ag_ctx* ctx, int n_steps, int K) {
   const size_t entries = (size_t)(K < n_steps ? K : n_steps);
   if (entries > ctx->adj_tape_cap) {
     free_tape();
-    e = alloc(ctx, &a.tape, entries * agk::kTapeWords * n);
+    e = alloc(ctx, &a.tape, entries * agk::kTapeWords * slots);
     if (e != cudaSuccess) { cudaGetLastError(); a.tape = nullptr; ctx->err = "tape does not fit"; return AG_ERR_OOM; }
     ctx->adj_tape_cap = entries;
   }
@@ -88,10 +88,10 @@ ag_status ensure_adjoint(ag_ctx* ctx, int n_steps, int K) {
       cudaStreamSynchronize(ctx->stream);
       cudaFree(a.ckpt);
       a.ckpt = nullptr;
-      ctx->bytes -= ctx->adj_ckpt_cap * 21 * n * sizeof(float);
+      ctx->bytes -= ctx->adj_ckpt_cap * 21 * slots * sizeof(float);
       ctx->adj_ckpt_cap = 0;
     }
-    e = alloc(ctx, &a.ckpt, n_ckpt * 21 * n);
+    e = alloc(ctx, &a.ckpt, n_ckpt * 21 * slots);
     if (e != cudaSuccess) { cudaGetLastError(); a.ckpt = nullptr; ctx->err = "checkpoints do not fit"; return AG_ERR_OOM; }
     ctx->adj_ckpt_cap = n_ckpt;
   }
@@ -136,6 +136,7 @@ extern "C" ag_status ag_rollout_loss(ag_ctx* ctx, uint32_t n_steps, float w_pos,
   a.state = ctx->fb.state; a.motors = ctx->fb.motors; a.body = ctx->fb.body; a.targets = ctx->fb.targets;
   a.modes = ctx->fb.modes;
   a.order = ctx->fb.order;
+  a.n_slots = ctx->fb.n_slots;
   a.n = c.n_envs; a.n_quad = c.n_quad; a.n_hexa = c.n_hexa; a.n_octo = c.n_octo;
   a.n_steps = (int)n_steps; a.K = K; a.w_pos = w_pos; a.w_omega = w_omega;
   ctx->adj_P = step_params(ctx);

@@ -20,6 +20,39 @@ struct NvtxRange {
   NvtxRange& operator=(const NvtxRange&) = delete;
 };
 
+// The grouping order. Windows of kOrderWindow consecutive environments are each
+// partitioned by key (rotor type, command mode); a key's run of slots starts at
+// a multiple of 32, so that no warp holds two keys, and the slots between runs
+// hold kNoEnv. A window has room for four keys per rotor type in it, each run
+// rounded up: under 1 % more slots than environments, but for the two windows
+// in which the type may change.
+constexpr uint32_t kOrderWindow = 16384;
+constexpr uint32_t kNoEnv = 0xFFFFFFFFu;
+struct OrderLayout {
+  uint32_t n, n_quad, n_hexa;
+  static constexpr __host__ __device__ uint32_t room(uint32_t count, uint32_t types) {
+    return (count + 31u * 4u * types) / 32u * 32u;
+  }
+  __host__ __device__ uint32_t count(uint32_t w) const {
+    const uint32_t lo = w * kOrderWindow;
+    return n - lo < kOrderWindow ? n - lo : kOrderWindow;
+  }
+  __host__ __device__ uint32_t types(uint32_t w) const {
+    const uint32_t lo = w * kOrderWindow, hi = lo + count(w), octo = n_quad + n_hexa;
+    return (lo < n_quad ? 1u : 0u) + ((lo > n_quad ? lo : n_quad) < (hi < octo ? hi : octo) ? 1u : 0u) +
+           ((lo > octo ? lo : octo) < hi ? 1u : 0u);
+  }
+  __host__ __device__ uint32_t slots(uint32_t w) const { return room(count(w), types(w)); }
+  __host__ __device__ uint32_t windows() const { return (n + kOrderWindow - 1) / kOrderWindow; }
+  // First slot of window w.
+  __host__ __device__ uint32_t base(uint32_t w) const {
+    const uint32_t v1 = n_quad / kOrderWindow, v2 = (n_quad + n_hexa) / kOrderWindow, one = room(kOrderWindow, 1);
+    return w * one + (v1 < w ? slots(v1) - one : 0u) + (v2 != v1 && v2 < w ? slots(v2) - one : 0u);
+  }
+  // Slots of the fleet (a multiple of 32).
+  __host__ __device__ uint32_t total() const { return base(windows() - 1) + slots(windows() - 1); }
+};
+
 // Device buffers of one fleet (all structure-of-arrays over n environments).
 struct FleetBuffers {
   float* state;        // [13][n]  p, v, q, Omega
@@ -40,10 +73,12 @@ struct FleetBuffers {
   float* wrench;       // [4][n]  realised wrench
   uint32_t* resets;    // [n]     resets of this call per env
   uint8_t* hits;       // [n]     collision of the current step
-  uint32_t* order;     // [n]     thread slot -> env, grouped by rotor type and mode (NULL = identity)
+  uint32_t* order;     // [n_slots] thread slot -> env, grouped by rotor type and mode, kNoEnv in the
+                       // padding (NULL = identity over n slots)
   const BoxRandDev* box_rand;  // [n_obs] obstacle re-draw on reset (NULL = boxes keep their poses)
   unsigned long long* tests_run;  // [1] exact collision tests of the last fused call (NULL = not counted)
   uint32_t n, n_quad, n_hexa, n_octo, n_obs;
+  uint32_t n_slots;    // thread slots of order (OrderLayout::total)
 };
 
 // Launch constants of a configuration: gains, FP64-computed allocation

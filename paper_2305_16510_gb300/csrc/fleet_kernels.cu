@@ -42,8 +42,8 @@ template <int INTEG, bool QUAD_ONLY, bool DRAG, bool BOXES>
 __global__ void __launch_bounds__(128, !BOXES && QUAD_ONLY && INTEG == kIntegSIE ? 7 : 4)
     k_fused_step(FleetBuffers fb, StepParams P, int n_steps, int substeps) {
   const uint32_t slot = blockIdx.x * blockDim.x + threadIdx.x;
-  const bool active = slot < fb.n;
-  const uint32_t env = active ? (fb.order ? fb.order[slot] : slot) : slot;
+  const uint32_t env = fb.order ? (slot < fb.n_slots ? fb.order[slot] : kNoEnv) : slot;
+  const bool active = env < fb.n;
   uint32_t resets = 0, tests = 0;
   bool any_hit = false;
   if (active) {
@@ -65,18 +65,24 @@ __global__ void __launch_bounds__(128, !BOXES && QUAD_ONLY && INTEG == kIntegSIE
   }
 }
 
-// Grouping permutation: key = rotor-type index * 4 + mode (12 keys). Slots
-// [w * W, (w + 1) * W), W = 4,096, hold the environments of the same window, stably
-// partitioned by key: inside a window the controller's mode branches become
-// warp-uniform (at most one mixed warp per key boundary), and since a window's
-// envs are loaded by blocks that run at the same time, the sectors their
-// gathers share are served from L2 instead of being fetched again from DRAM.
-// One block per window: the key totals give each key's start; then, 1,024
-// envs at a time, each env is ranked inside its warp with __match_any_sync and
-// offset by its key's running position and the preceding warps' counts.
-constexpr int kOrderThreads = 1024;
-constexpr int kOrderSub = 4;                                  // sub-windows per window
-constexpr int kOrderWindow = kOrderThreads * kOrderSub;       // 4,096 envs
+// Grouping order: key = rotor-type index * 4 + mode (12 keys). Each window of
+// 16,384 environments is stably partitioned by key, every key's run of slots
+// starting at a multiple of 32 (OrderLayout): a warp then holds one key and the
+// controller's mode branches are warp-uniform, and since a window's envs are
+// loaded by blocks that run at the same time, the sectors their gathers share
+// are served from L2 instead of being fetched again from DRAM. With runs that
+// were not padded, one warp per key boundary ran two modes' code in turn, and
+// launches of one wave waited for it (131,072 quads of two modes x 100 steps:
+// 127 us a pass against 121; 1,000 quads' gradient 491 us against 412). A
+// window of 4,096 needs four times the padding (8 % with three rotor types,
+// which cost a 4M mixed fleet 0.9 %).
+// One block per window. Each warp takes a contiguous share of the window's
+// environments, 32 at a time, and counts them by key (__match_any_sync, one
+// add per key and 32 environments); a scan over the warps gives every warp its
+// place in each key's run, and a second pass over the modes writes the slots.
+constexpr int kOrderThreads = 1024, kOrderWarps = kOrderThreads / 32;
+
+__host__ __device__ inline OrderLayout order_layout(const FleetBuffers& fb) { return {fb.n, fb.n_quad, fb.n_hexa}; }
 
 __device__ __forceinline__ uint32_t order_key(const FleetBuffers& fb, uint32_t i) {
   const int nrot = rotor_count(fb, i);
@@ -85,50 +91,55 @@ __device__ __forceinline__ uint32_t order_key(const FleetBuffers& fb, uint32_t i
 }
 
 __global__ void __launch_bounds__(kOrderThreads) k_order_window(FleetBuffers fb) {
-  __shared__ uint32_t warp_count[kOrderThreads / 32][12];
-  __shared__ uint32_t key_next[12];  // next free position of each key in the window
-  const uint32_t base = blockIdx.x * kOrderWindow;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  // pass 1: totals per key over the window -> start position of each key
-  if (threadIdx.x < 12) key_next[threadIdx.x] = 0;
+  __shared__ uint32_t place[kOrderWarps][12];  // counts, then the next place of the warp in each key's run
+  __shared__ uint32_t run[12];                 // length, then the first slot of each key's run
+  const OrderLayout layout = order_layout(fb);
+  const uint32_t first = blockIdx.x * kOrderWindow, count = layout.count(blockIdx.x), slots = layout.slots(blockIdx.x);
+  uint32_t* const order = fb.order + layout.base(blockIdx.x);
+  const uint32_t warp = threadIdx.x >> 5, lane = threadIdx.x & 31u;
+  const uint32_t share = (count + kOrderThreads - 1) / kOrderThreads * 32u;  // environments per warp
+  const uint32_t lo = warp * share, hi = min(lo + share, count);
+  for (uint32_t k = threadIdx.x; k < slots; k += kOrderThreads) order[k] = kNoEnv;
+  if (lane < 12) place[warp][lane] = 0;
+  __syncwarp();
+  for (uint32_t i = lo; i < hi; i += 32) {
+    const uint32_t key = i + lane < hi ? order_key(fb, first + i + lane) : 12u;
+    const unsigned same = __match_any_sync(0xFFFFFFFFu, key);
+    if (key < 12u && (int)lane == __ffs(same) - 1) place[warp][key] += __popc(same);
+    __syncwarp();
+  }
   __syncthreads();
-  for (int sub = 0; sub < kOrderSub; ++sub) {
-    const uint32_t i = base + sub * kOrderThreads + threadIdx.x;
-    if (i < fb.n) atomicAdd(&key_next[order_key(fb, i)], 1u);
+  if (warp < 12) {  // warp k: exclusive scan of key k's counts over the warps
+    const uint32_t own = place[lane][warp];
+    uint32_t sum = own;
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+      const uint32_t up = __shfl_up_sync(0xFFFFFFFFu, sum, d);
+      if ((int)lane >= d) sum += up;
+    }
+    place[lane][warp] = sum - own;
+    if (lane == 31) run[warp] = sum;
   }
   __syncthreads();
   if (threadIdx.x == 0) {
-    uint32_t run = 0;
+    uint32_t at = 0;
     for (int k = 0; k < 12; ++k) {
-      const uint32_t c = key_next[k];
-      key_next[k] = run;
-      run += c;
+      const uint32_t length = run[k];
+      run[k] = at;
+      at += (length + 31u) & ~31u;
     }
   }
   __syncthreads();
-  // pass 2: sub-window by sub-window, stable ranks inside each key
-  for (int sub = 0; sub < kOrderSub; ++sub) {
-    const uint32_t i = base + sub * kOrderThreads + threadIdx.x;
-    const bool active = i < fb.n;
-    const uint32_t key = active ? order_key(fb, i) : 12u;
+  for (uint32_t i = lo; i < hi; i += 32) {
+    const uint32_t key = i + lane < hi ? order_key(fb, first + i + lane) : 12u;
     const unsigned same = __match_any_sync(0xFFFFFFFFu, key);
-    const uint32_t rank = __popc(same & ((1u << lane) - 1u));
-    if (lane < 12) warp_count[warp][lane] = 0;
+    const uint32_t at = key < 12u ? place[warp][key] : 0u;
     __syncwarp();
-    if (active && rank == 0) warp_count[warp][key] = __popc(same);
-    __syncthreads();
-    if (active) {
-      uint32_t pos = key_next[key] + rank;
-      for (int w = 0; w < warp; ++w) pos += warp_count[w][key];
-      fb.order[base + pos] = i;
+    if (key < 12u) {
+      if ((int)lane == __ffs(same) - 1) place[warp][key] = at + __popc(same);
+      order[run[key] + at + __popc(same & ((1u << lane) - 1u))] = first + i + lane;
     }
-    __syncthreads();
-    if (threadIdx.x < 12) {  // advance each key by its count in this sub-window
-      uint32_t c = 0;
-      for (int w = 0; w < kOrderThreads / 32; ++w) c += warp_count[w][threadIdx.x];
-      key_next[threadIdx.x] += c;
-    }
-    __syncthreads();
+    __syncwarp();
   }
 }
 
@@ -275,7 +286,8 @@ cudaError_t launch_fused_b(const FleetBuffers& fb, const StepParams& P, int n_st
     }
     if (best <= 0) return cudaErrorInvalidConfiguration;
   }
-  const unsigned grid = (fb.n + B - 1) / B;
+  const uint32_t slots = fb.order ? fb.n_slots : fb.n;
+  const unsigned grid = (slots + B - 1) / B;
   kernel<<<grid, B, 0, st>>>(fb, P, n_steps, substeps);
   return cudaGetLastError();
 }
@@ -330,7 +342,7 @@ cudaError_t launch_fused_step(const FleetBuffers& fb_in, const StepParams& P, in
 }
 
 cudaError_t launch_build_order(const FleetBuffers& fb, cudaStream_t st) {
-  k_order_window<<<(fb.n + kOrderWindow - 1) / kOrderWindow, kOrderThreads, 0, st>>>(fb);
+  k_order_window<<<order_layout(fb).windows(), kOrderThreads, 0, st>>>(fb);
   return cudaGetLastError();
 }
 

@@ -67,8 +67,9 @@ __global__ void __launch_bounds__(kServeBlock, 4) k_serve_step(const ServeDesc* 
   __syncthreads();
   const ServeDesc& d = table[s_req];
   const uint32_t slot = (blockIdx.x - d.block_begin) * blockDim.x + threadIdx.x;
-  if (slot >= d.fb.n || d.steps <= 0) return;
+  if (slot >= d.fb.n_slots || d.steps <= 0) return;
   const uint32_t env = d.fb.order[slot];
+  if (env >= d.fb.n) return;
   uint32_t resets = 0, tests = 0;
   bool hit = false;
   simulate<4, INTEG, DRAG>(d.fb, P, env, d.steps, substeps, (int)d.fb.n_obs, EnvBoxes(d.fb, env), d.seed_lo, d.seed_hi, resets,
@@ -127,12 +128,12 @@ class SlabAllocator {
 size_t align256(size_t b) { return (b + 255) & ~size_t(255); }
 
 // Device bytes one request needs (state, motors, body, targets, modes, epoch,
-// collided, reset ids and count, order, box records and the staging of one
-// box's rows).
+// collided, reset count, order (its first use is as the initial reset's id
+// list), box records and the staging of one box's rows).
 size_t request_bytes(size_t n, size_t n_obs) {
   size_t b = 0;
   b += align256(13 * n * 4) + align256(8 * n * 4) + align256(4 * n * 4) + align256(4 * n * 4);
-  b += align256(n) + align256(n * 4) + align256(n) + align256(n * 4) + align256(4) + align256(n * 4);
+  b += align256(n) + align256(n * 4) + align256(n) + align256(4) + align256(OrderLayout{(uint32_t)n, (uint32_t)n, 0}.total() * sizeof(uint32_t));
   b += align256(n_obs * n * 16) + align256(n_obs * n * 32) + align256(n_obs ? 10 * n * 4 : 0);
   return b;
 }
@@ -204,9 +205,10 @@ void carve(ag_server* s, ServeRequest* r) {
   f.modes = (uint8_t*)take(n);
   f.epoch = (uint32_t*)take(n * 4);
   f.collided = (uint8_t*)take(n);
-  f.reset_ids = (uint32_t*)take(n * 4);
   f.n_reset = (uint32_t*)take(4);
-  f.order = (uint32_t*)take(n * 4);
+  f.n_slots = agk::OrderLayout{(uint32_t)n, (uint32_t)n, 0}.total();
+  f.order = (uint32_t*)take(f.n_slots * sizeof(uint32_t));
+  f.reset_ids = f.order;  // written by the initial reset, before the order is built
   f.box_bound = (float4*)take(n_obs * n * 16);
   f.box_rest = (float4*)take(n_obs * n * 32);
   r->box_stage = (float*)take(n_obs ? 10 * n * 4 : 0);
@@ -343,7 +345,7 @@ void serve_loop(ag_server* s) {
         d.seed_hi = (uint32_t)(r->in.seed >> 32);
         d.steps = (int)steps;
         d.block_begin = blocks;
-        blocks += (r->in.n_envs + agk::kServeBlock - 1) / agk::kServeBlock;
+        blocks += (r->fb.n_slots + agk::kServeBlock - 1) / agk::kServeBlock;
       }
       const int n_req = (int)sched.size();
       e = cudaMemcpyAsync(s->table_dev[b], s->table_host[b], sizeof(agk::ServeDesc) * n_req, cudaMemcpyHostToDevice,
