@@ -203,6 +203,14 @@ __device__ __forceinline__ float clearance_threshold2(V3 p, float min_e2, float 
   return t > 0.f ? t * t : -1.f;
 }
 
+// When one thread of a warp has to test, the others wait for it anyway: those
+// that have moved at least half their clearance (this share of its square)
+// test along with it instead of holding the warp up again soon after. Tests
+// run early decide what tests run in time would. 1,048,576 quads among 16
+// boxes x 1,000 steps: 52.7 -> 50.9 ms (48.5 ms without any test after the
+// first step); shares of 0.5, 0.1, 0.03 and 0 measured 51.1, 50.9, 51.0, 51.0.
+constexpr float kJoinTest = 0.25f;
+
 // The per-vehicle body of the fused kernels, specialised on the rotor count:
 // n_steps steps of `substeps` substeps, then the sphere-vs-box test against
 // n_obs boxes and, on a hit, the Philox reset keyed (seed_lo, seed_hi).
@@ -232,6 +240,7 @@ __device__ __forceinline__ VState simulate_cmd(const FleetBuffers& fb, const Ste
   V3 p_test = {0.f, 0.f, 0.f};
   float thr2 = -1.f;
   const float r = sqrtf(P.r2);
+  const unsigned group = __activemask();  // threads of one launch, so of one trip count
   for (int step = 0; step < n_steps; ++step) {
     for (int ss = 0; ss < substeps; ++ss) {
       V3 b3;
@@ -240,7 +249,8 @@ __device__ __forceinline__ VState simulate_cmd(const FleetBuffers& fb, const Ste
     }
     if (n_obs > 0) {
       const V3 dp = s.p - p_test;
-      if (!(dot(dp, dp) < thr2)) {
+      const float moved2 = dot(dp, dp);
+      if (n_steps == 1 || (__any_sync(group, !(moved2 < thr2)) && !(moved2 < kJoinTest * thr2))) {
         float min_e2;
         const bool hit = boxes.any_hit(s.p, r, P.r2, n_obs, step + 1 < n_steps, P.exact_tests != 0, min_e2);
         tests += 1;
