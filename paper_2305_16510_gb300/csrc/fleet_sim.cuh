@@ -47,6 +47,25 @@ __device__ __forceinline__ Command load_command(const FleetBuffers& fb, uint32_t
                          fb.targets[3 * n + i]);
 }
 
+// What a launch reads of one vehicle, as it is in memory. It is requested
+// before anything waits for the command (whose angles go through sincosf, a
+// branch that no load moves across): a single-step launch then waits for memory
+// once instead of twice.
+template <int NROT> struct VehicleRows {
+  VState s;
+  float u[NROT], body[4];
+};
+template <int NROT> __device__ __forceinline__ VehicleRows<NROT> load_vehicle(const FleetBuffers& fb, uint32_t env) {
+  const uint32_t n = fb.n;
+  VehicleRows<NROT> v;
+  v.s = load_state(fb.state, n, env);
+#pragma unroll
+  for (int k = 0; k < NROT; ++k) v.u[k] = fb.motors[k * n + env];
+#pragma unroll
+  for (int k = 0; k < 4; ++k) v.body[k] = fb.body[k * n + env];
+  return v;
+}
+
 // Overwrites one environment with its reset draw for `epoch`.
 template <int NROT>
 __device__ __forceinline__ void reset_in_registers(VState& s, float (&u)[NROT], float m, uint32_t env,
@@ -104,20 +123,45 @@ struct NoBoxSource {
 // A single step over 16 random boxes (centres U[-5, 5]^3, half-extents
 // U[0.1, 1]) tests about 0.13 boxes per vehicle exactly, so it reads 16 bytes
 // per box and little more instead of 40: a task step of 131,072 environments
-// (RK4 x 4) takes 37 us a pass instead of 60, and the bench fleet's 1,000-step
-// call from fresh states 53.8 ms instead of 57.9. kBoxNear hardly matters:
+// (RK4 x 4) took 37 us a pass instead of 60, and the bench fleet's 1,000-step
+// call from fresh states 53.8 ms instead of 57.9 (both less since). kBoxNear hardly matters:
 // 0.25 and 1 m measured 53.9 ms.
 constexpr float kBoxSlack = 1e-3f, kBoxNear = 0.5f;
 
-struct EnvBoxes {
+// GROUPED: the spheres are loaded in whole groups (8, or 16 while more than 8
+// are left) before any is looked at, so that a group waits for memory once. It
+// serves the single-step kernel, where every thread tests (131,072 quads with
+// 3 / 8 / 16 / 32 boxes: 23.3 / 27.6 / 34.7 / 52.5 us a pass); in the launches
+// of many steps, where few do, the plain loop leaves more registers to the
+// step (1M x 1,000 steps: 50.5 ms against 51.6).
+template <bool GROUPED> struct EnvBoxesT {
   const float4* bound;  // this environment's column of box_bound
   const float4* rest;   // and of box_rest
   uint32_t n;
-  __device__ __forceinline__ EnvBoxes(const FleetBuffers& fb, uint32_t env)
+  __device__ __forceinline__ EnvBoxesT(const FleetBuffers& fb, uint32_t env)
       : bound(fb.box_bound + env), rest(fb.box_rest + 2 * (size_t)env), n(fb.n) {}
   __device__ __forceinline__ float dist2(V3 p, int k) const {
     const float4 b = bound[(size_t)k * n], h = rest[2 * (size_t)k * n], q = rest[2 * (size_t)k * n + 1];
     return box_dist2(p, V3{b.x, b.y, b.z}, V3{h.x, h.y, h.z}, Q4{h.w, q.x, q.y, q.z});
+  }
+  // The distance from p to the sphere b, low by the margin above.
+  static __device__ __forceinline__ float low_distance(V3 p, float4 b) {
+    const V3 v = p - V3{b.x, b.y, b.z};
+    const float d2 = dot(v, v);
+    return fmaf(d2 * rsqrt_ftz(d2), 1.f - 3e-4f, -b.w);
+  }
+  // Spheres k0 .. k0 + G - 1 (the last box again beyond n_obs), bits from bit.
+  template <int G>
+  __device__ __forceinline__ void scan(V3 p, int k0, int n_obs, int bit, float reach, float& far, uint32_t& exact) const {
+    float4 b[G];
+#pragma unroll
+    for (int j = 0; j < G; ++j) b[j] = bound[(size_t)min(k0 + j, n_obs - 1) * n];
+#pragma unroll
+    for (int j = 0; j < G; ++j) {
+      const float low = low_distance(p, b[j]);
+      if (low > reach) far = fminf(far, low);
+      else if (k0 + j < n_obs) exact |= 1u << (bit + j);
+    }
   }
   __device__ __forceinline__ bool any_hit(V3 p, float r, float r2, int n_obs, bool want_min, bool all, float& m) const {
     const float inf = __int_as_float(0x7f800000);
@@ -127,14 +171,23 @@ struct EnvBoxes {
     for (int k0 = 0; k0 < n_obs; k0 += 32) {
       const int count = min(32, n_obs - k0);
       uint32_t exact = 0;
-#pragma unroll 4
-      for (int j = 0; j < count; ++j) {
-        const float4 b = bound[(size_t)(k0 + j) * n];
-        const V3 v = p - V3{b.x, b.y, b.z};
-        const float d2 = dot(v, v);
-        const float low = fmaf(d2 * rsqrt_ftz(d2), 1.f - 3e-4f, -b.w);
-        if (low > reach) far = fminf(far, low);
-        else exact |= 1u << j;
+      if (GROUPED) {
+        for (int j = 0; j < count;) {
+          if (count - j <= 8) {
+            scan<8>(p, k0 + j, n_obs, j, reach, far, exact);
+            j += 8;
+          } else {
+            scan<16>(p, k0 + j, n_obs, j, reach, far, exact);
+            j += 16;
+          }
+        }
+      } else {
+#pragma unroll 8
+        for (int j = 0; j < count; ++j) {
+          const float low = low_distance(p, bound[(size_t)(k0 + j) * n]);
+          if (low > reach) far = fminf(far, low);
+          else exact |= 1u << j;
+        }
       }
       while (exact) {
         const int j = __ffs(exact) - 1;
@@ -148,6 +201,7 @@ struct EnvBoxes {
     return hit;
   }
 };
+using EnvBoxes = EnvBoxesT<false>;
 
 // New poses for every box of environment env, written to its records (the
 // half-extents and the sphere radius stay).
@@ -220,19 +274,18 @@ constexpr float kJoinTest = 0.25f;
 // and the controller's branches on it fold away.
 template <int NROT, int INTEG, bool DRAG, class Boxes, int MODE = -1>
 __device__ __forceinline__ VState simulate_cmd(const FleetBuffers& fb, const StepParams& P, uint32_t env,
-                                               const Command& cm_in, int n_steps, int substeps, int n_obs,
-                                               const Boxes& boxes, uint32_t seed_lo, uint32_t seed_hi, uint32_t& resets,
-                                               bool& any_hit, uint32_t& tests) {
+                                               const VehicleRows<NROT>& rows, const Command& cm_in, int n_steps,
+                                               int substeps, int n_obs, const Boxes& boxes, uint32_t seed_lo,
+                                               uint32_t seed_hi, uint32_t& resets, bool& any_hit, uint32_t& tests) {
   Command cm = cm_in;
   if (MODE >= 0) cm.mode = MODE;
   const uint32_t n = fb.n;
-  VState s = load_state(fb.state, n, env);
+  VState s = rows.s;
   normalize(s.q);
   float u[NROT];
 #pragma unroll
-  for (int k = 0; k < NROT; ++k) u[k] = fb.motors[k * n + env];
-  const Body b = load_body(fb.body, n, env);
-  uint32_t epoch = fb.epoch[env];
+  for (int k = 0; k < NROT; ++k) u[k] = rows.u[k];
+  const Body b = make_body(rows.body[0], rows.body[1], rows.body[2], rows.body[3]);
   // Collision tests that cannot hit are skipped (see clearance_threshold2):
   // p_test is the position of the last test, thr2 the squared distance
   // the vehicle may move from there before it could touch a box (-1: test
@@ -259,7 +312,8 @@ __device__ __forceinline__ VState simulate_cmd(const FleetBuffers& fb, const Ste
         if (hit) {
           any_hit = true;
           resets += 1;
-          epoch += 1;
+          const uint32_t epoch = fb.epoch[env] + 1u;  // read and written only where a reset needs it
+          fb.epoch[env] = epoch;
           reset_in_registers<NROT>(s, u, b.m, env, epoch, seed_lo, seed_hi);
           thr2 = -1.f;
           if (fb.box_rand) redraw_boxes(fb, env, epoch, seed_lo, seed_hi);
@@ -270,7 +324,6 @@ __device__ __forceinline__ VState simulate_cmd(const FleetBuffers& fb, const Ste
   store_state(fb.state, n, env, s);
 #pragma unroll
   for (int k = 0; k < NROT; ++k) fb.motors[k * n + env] = u[k];
-  fb.epoch[env] = epoch;
   return s;
 }
 
@@ -286,6 +339,7 @@ template <int NROT, int INTEG, bool DRAG, bool BY_MODE = false, class Boxes>
 __device__ __forceinline__ void simulate(const FleetBuffers& fb, const StepParams& P, uint32_t env,
                                          int n_steps, int substeps, int n_obs, const Boxes& boxes, uint32_t seed_lo,
                                          uint32_t seed_hi, uint32_t& resets, bool& any_hit, uint32_t& tests) {
+  const VehicleRows<NROT> rows = load_vehicle<NROT>(fb, env);
   const Command cm = load_command(fb, env);
   bool uniform = false;
   if (BY_MODE && fb.order) {
@@ -294,22 +348,22 @@ __device__ __forceinline__ void simulate(const FleetBuffers& fb, const StepParam
   }
   if (uniform) {
     if (cm.mode == kModePosition) {
-      simulate_cmd<NROT, INTEG, DRAG, Boxes, kModePosition>(fb, P, env, cm, n_steps, substeps, n_obs, boxes,
+      simulate_cmd<NROT, INTEG, DRAG, Boxes, kModePosition>(fb, P, env, rows, cm, n_steps, substeps, n_obs, boxes,
                                                            seed_lo, seed_hi, resets, any_hit, tests);
       return;
     }
     if (cm.mode == kModeBodyVel) {
-      simulate_cmd<NROT, INTEG, DRAG, Boxes, kModeBodyVel>(fb, P, env, cm, n_steps, substeps, n_obs, boxes,
+      simulate_cmd<NROT, INTEG, DRAG, Boxes, kModeBodyVel>(fb, P, env, rows, cm, n_steps, substeps, n_obs, boxes,
                                                           seed_lo, seed_hi, resets, any_hit, tests);
       return;
     }
     if (cm.mode == kModeAttThrust) {
-      simulate_cmd<NROT, INTEG, DRAG, Boxes, kModeAttThrust>(fb, P, env, cm, n_steps, substeps, n_obs, boxes,
+      simulate_cmd<NROT, INTEG, DRAG, Boxes, kModeAttThrust>(fb, P, env, rows, cm, n_steps, substeps, n_obs, boxes,
                                                             seed_lo, seed_hi, resets, any_hit, tests);
       return;
     }
   }
-  simulate_cmd<NROT, INTEG, DRAG>(fb, P, env, cm, n_steps, substeps, n_obs, boxes, seed_lo, seed_hi, resets,
+  simulate_cmd<NROT, INTEG, DRAG>(fb, P, env, rows, cm, n_steps, substeps, n_obs, boxes, seed_lo, seed_hi, resets,
                                   any_hit, tests);
 }
 

@@ -72,8 +72,9 @@ __global__ void __launch_bounds__(kServeBlock, 4) k_serve_step(const ServeDesc* 
   if (env >= d.fb.n) return;
   uint32_t resets = 0, tests = 0;
   bool hit = false;
-  simulate<4, INTEG, DRAG>(d.fb, P, env, d.steps, substeps, (int)d.fb.n_obs, EnvBoxes(d.fb, env), d.seed_lo, d.seed_hi, resets,
-                           hit, tests);
+  const EnvBoxes boxes(d.fb, env);
+  simulate<4, INTEG, DRAG>(d.fb, P, env, d.steps, substeps, (int)d.fb.n_obs, boxes, d.seed_lo, d.seed_hi, resets, hit,
+                           tests);
 }
 
 // First-fit allocator over [0, size) with coalescing frees (host bookkeeping

@@ -76,42 +76,55 @@ __device__ __forceinline__ void write_obs(const ReachArgs& a, const float* stage
     if (base + t < total) a.obs[base + t] = ws[t];
 }
 
+// The step itself for one airframe: action -> command t, one fleet step of
+// `substeps` substeps from the vehicle's rows.
+template <int NROT, int INTEG, bool DRAG, class Boxes>
+__device__ __forceinline__ VState reach_fly(const ReachArgs& a, const StepParams& P, uint32_t i, float4 act, int mode,
+                                            int substeps, int n_obs, const Boxes& boxes, float (&t)[4], bool& hit) {
+  const VehicleRows<NROT> rows = load_vehicle<NROT>(a.fb, i);
+  const float v[4] = {act.x, act.y, act.z, act.w};
+#pragma unroll
+  for (int k = 0; k < 4; ++k) t[k] = fmaf(a.scale[k], fminf(fmaxf(v[k], -1.f), 1.f), a.offset[k]);
+  const Command cm = prepare_command(mode, t[0], t[1], t[2], t[3]);
+  uint32_t resets = 0, tests = 0;
+  return simulate_cmd<NROT, INTEG, DRAG>(a.fb, P, i, rows, cm, 1, substeps, n_obs, boxes, a.seed_lo, a.seed_hi, resets,
+                                         hit, tests);
+}
+
 // One task step of environment i = thread: actions -> commands, one fleet
 // step (controller, allocation, integration, collision test and reset, as in
 // the fused fleet step), then reach_tail. Every environment shares the task's
 // command mode, so warps are mode-uniform without a grouping permutation.
-// Without boxes the step is memory-latency bound: a bound of 14 blocks (28
-// warps) per SM measured best, against 16 blocks (64 registers, more spills)
-// and 20 (48 registers). With boxes 8 blocks (16 warps, 128 registers).
-template <int INTEG, bool DRAG, bool BOXES>
-__global__ void __launch_bounds__(kTaskBlock, BOXES ? 512 / kTaskBlock : 896 / kTaskBlock)
+// Without boxes the step is memory-latency bound: a bound of 12 blocks (24
+// warps) per SM measured best (50.8 us a pass over 1,048,576 quads), against
+// 10 (53.2), 14 (51.3), 16 (52.2, 64 registers) and 18 (53.3); with the state
+// requested after the command's angles it took 57.4. With boxes 8 blocks (16
+// warps, 128 registers).
+template <int INTEG, bool QUAD_ONLY, bool DRAG, bool BOXES>
+__global__ void __launch_bounds__(kTaskBlock, BOXES ? 8 : 12)
     k_reach_step(ReachArgs a, StepParams P, int substeps) {
   __shared__ float stage[kTaskBlock * kObs];  // odd row length: conflict-free
   const FleetBuffers& fb = a.fb;
   const uint32_t i = blockIdx.x * kTaskBlock + threadIdx.x;
   const uint32_t n = fb.n;
-  uint32_t resets = 0, tests = 0;
   if (i < n) {
     // everything the step reads from memory, requested up front
     const float4 act = reinterpret_cast<const float4*>(a.actions)[i];
     const V3 g = load_goal(a, i);
     const uint32_t steps_before = a.steps[i];
-    const float v[4] = {act.x, act.y, act.z, act.w};
-    float t[4];
-#pragma unroll
-    for (int k = 0; k < 4; ++k) t[k] = fmaf(a.scale[k], fminf(fmaxf(v[k], -1.f), 1.f), a.offset[k]);
-    const Command cm = prepare_command(fb.modes[i], t[0], t[1], t[2], t[3]);
-    const int nrot = rotor_count(fb, i);
+    const int mode = fb.modes[i];
+    const int nrot = QUAD_ONLY ? 4 : rotor_count(fb, i);
     bool hit = false;
     VState s;
-    const std::conditional_t<BOXES, EnvBoxes, NoBoxSource> boxes(fb, i);
+    float t[4];
+    const std::conditional_t<BOXES, EnvBoxesT<true>, NoBoxSource> boxes(fb, i);
     const int n_obs = BOXES ? (int)fb.n_obs : 0;
     if (nrot == 4)
-      s = simulate_cmd<4, INTEG, DRAG>(fb, P, i, cm, 1, substeps, n_obs, boxes, a.seed_lo, a.seed_hi, resets, hit, tests);
+      s = reach_fly<4, INTEG, DRAG>(a, P, i, act, mode, substeps, n_obs, boxes, t, hit);
     else if (nrot == 6)
-      s = simulate_cmd<6, INTEG, DRAG>(fb, P, i, cm, 1, substeps, n_obs, boxes, a.seed_lo, a.seed_hi, resets, hit, tests);
+      s = reach_fly<6, INTEG, DRAG>(a, P, i, act, mode, substeps, n_obs, boxes, t, hit);
     else
-      s = simulate_cmd<8, INTEG, DRAG>(fb, P, i, cm, 1, substeps, n_obs, boxes, a.seed_lo, a.seed_hi, resets, hit, tests);
+      s = reach_fly<8, INTEG, DRAG>(a, P, i, act, mode, substeps, n_obs, boxes, t, hit);
     fb.collided[i] = hit ? 1 : 0;
 #pragma unroll
     for (int k = 0; k < 4; ++k) fb.targets[k * n + i] = t[k];  // the commands, as ag_set_commands keeps them
@@ -130,10 +143,11 @@ __global__ void __launch_bounds__(kTaskBlock) k_reach_observe(ReachArgs a) {
 template <int INTEG, bool DRAG>
 cudaError_t launch_step_t(const ReachArgs& a, const StepParams& P, int substeps, cudaStream_t st) {
   const unsigned grid = (a.fb.n + kTaskBlock - 1) / kTaskBlock;
-  if (a.fb.n_obs > 0)
-    k_reach_step<INTEG, DRAG, true><<<grid, kTaskBlock, 0, st>>>(a, P, substeps);
-  else
-    k_reach_step<INTEG, DRAG, false><<<grid, kTaskBlock, 0, st>>>(a, P, substeps);
+  // with boxes a kernel for quads alone measured slower (36.9 us a pass against 35.6, 131,072 quads, 16 boxes)
+  const auto kernel = a.fb.n_obs > 0           ? k_reach_step<INTEG, false, DRAG, true>
+                      : a.fb.n_quad == a.fb.n ? k_reach_step<INTEG, true, DRAG, false>
+                                              : k_reach_step<INTEG, false, DRAG, false>;
+  kernel<<<grid, kTaskBlock, 0, st>>>(a, P, substeps);
   return cudaGetLastError();
 }
 
