@@ -157,7 +157,7 @@ size_t buffer_bytes(const ag_config* c) {
   size_t n = c->n_envs;
   size_t per = sizeof(float) * (13 + 8 + 4 + 4 + 4) + sizeof(uint32_t) * 3 + 3 /* modes, collided, hits */ + 1;
   return n * per + agk::OrderLayout{c->n_envs, c->n_quad, c->n_hexa}.total() * sizeof(uint32_t) + agk::box_record_bytes(n, c->n_obstacles) + (c->n_obstacles ? 10 * n * sizeof(float) : 0) +
-         sizeof(uint32_t) + sizeof(unsigned long long);
+         sizeof(agk::CallCounts);
 }
 
 }  // namespace
@@ -224,7 +224,7 @@ bool on_device(const void* p) {
 bool on_own_device(const ag_ctx* ctx, const void* p) {
   cudaPointerAttributes pa;
   const bool own = cudaPointerGetAttributes(&pa, p) == cudaSuccess && pa.type == cudaMemoryTypeDevice &&
-                   pa.device == ctx->device;
+                   pa.device == ctx->device && reinterpret_cast<uintptr_t>(p) % 4 == 0;
   cudaGetLastError();
   return own;
 }
@@ -254,7 +254,7 @@ void free_all(ag_ctx* ctx) {
   if (ctx->reach_steps) cudaFree(ctx->reach_steps);
   agk::FleetBuffers& f = ctx->fb;
   void* ptrs[] = {f.state, f.motors, f.body, f.modes, f.targets, f.box_bound, f.box_rest, f.epoch, f.collided, f.reset_ids,
-                  f.n_reset, f.tests_run, f.cmd, f.resets, f.hits, f.order, ctx->mask_dev,
+                  f.counts, f.cmd, f.resets, f.hits, f.order, ctx->mask_dev,
                   ctx->box_stage, (void*)f.box_rand};
   for (void* p : ptrs)
     if (p) cudaFree(p);
@@ -356,8 +356,8 @@ ag_status ag_create(const ag_config* cfg, void* cuda_stream, ag_ctx** out) {
   if (e == cudaSuccess) e = alloc(ctx, &f.epoch, n);
   if (e == cudaSuccess) e = alloc(ctx, &f.collided, n);
   if (e == cudaSuccess) e = alloc(ctx, &f.reset_ids, n);
-  if (e == cudaSuccess) e = alloc(ctx, &f.n_reset, 1);
-  if (e == cudaSuccess) e = alloc(ctx, &f.tests_run, 1);
+  if (e == cudaSuccess) e = alloc(ctx, &f.counts, 1);
+  f.n_reset = f.counts ? &f.counts->resets : nullptr;
   if (e == cudaSuccess) e = alloc(ctx, &f.cmd, 4 * n);
   f.wrench = f.cmd;  // the allocation stage reads an environment's command before it writes its wrench
   if (e == cudaSuccess) e = alloc(ctx, &f.resets, n);
@@ -390,8 +390,7 @@ ag_status ag_create(const ag_config* cfg, void* cuda_stream, ag_ctx** out) {
     e = cudaMemsetAsync(f.box_rest, 0, (size_t)cfg->n_obstacles * n * 2 * sizeof(float4), st);
   if (e == cudaSuccess) e = cudaMemsetAsync(f.epoch, 0, n * sizeof(uint32_t), st);
   if (e == cudaSuccess) e = cudaMemsetAsync(f.collided, 0, n, st);
-  if (e == cudaSuccess) e = cudaMemsetAsync(f.n_reset, 0, sizeof(uint32_t), st);
-  if (e == cudaSuccess) e = cudaMemsetAsync(f.tests_run, 0, sizeof(unsigned long long), st);
+  if (e == cudaSuccess) e = cudaMemsetAsync(f.counts, 0, sizeof(agk::CallCounts), st);
   if (e == cudaSuccess) e = agk::launch_build_order(f, st);
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);
   if (e != cudaSuccess) {

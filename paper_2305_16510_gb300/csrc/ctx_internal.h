@@ -59,8 +59,8 @@ ag_status enter(ag_ctx* ctx);
 agk::StepParams step_params(const ag_ctx* ctx);
 // true for device or managed memory (a kernel can read it), false for host memory.
 bool on_device(const void* p);
-// true for memory of the context's own device, which its kernels read and
-// write in place (managed, host and other devices' memory is copied).
+// true for memory of the context's own device, aligned to 4 bytes, which its
+// kernels read and write in place (anything else is copied).
 bool on_own_device(const ag_ctx* ctx, const void* p);
 // Rotor allocation matrix A and its pseudo-inverse A^+ in FP64, stored float32.
 void rotor_matrices(int n, double arm, double k_yaw, float A[4][8], float Ap[8][4]);

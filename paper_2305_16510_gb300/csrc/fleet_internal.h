@@ -53,6 +53,12 @@ struct OrderLayout {
   __host__ __device__ uint32_t total() const { return base(windows() - 1) + slots(windows() - 1); }
 };
 
+// What a call counts, side by side so that one memset clears it.
+struct CallCounts {
+  unsigned long long tests;  // collision tests of the last fused call
+  uint32_t resets;           // length of the reset list
+};
+
 // Device buffers of one fleet (all structure-of-arrays over n environments).
 struct FleetBuffers {
   float* state;        // [13][n]  p, v, q, Omega
@@ -76,7 +82,7 @@ struct FleetBuffers {
   uint32_t* order;     // [n_slots] thread slot -> env, grouped by rotor type and mode, kNoEnv in the
                        // padding (NULL = identity over n slots)
   const BoxRandDev* box_rand;  // [n_obs] obstacle re-draw on reset (NULL = boxes keep their poses)
-  unsigned long long* tests_run;  // [1] exact collision tests of the last fused call (NULL = not counted)
+  CallCounts* counts;  // [1] a context's counts; n_reset points into it (NULL for the other users)
   uint32_t n, n_quad, n_hexa, n_octo, n_obs;
   uint32_t n_slots;    // thread slots of order (OrderLayout::total)
 };

@@ -58,11 +58,13 @@ __global__ void __launch_bounds__(128, !BOXES && QUAD_ONLY && INTEG == kIntegSIE
       simulate<8, INTEG, DRAG, true>(fb, P, env, n_steps, substeps, n_obs, boxes, P.seed_lo, P.seed_hi, resets, any_hit, tests);
     fb.collided[env] = any_hit ? 1 : 0;
   }
-  append_compact(resets > 0u, env, fb.reset_ids, fb.n_reset);
-  if (BOXES && fb.tests_run) {  // one atomic per warp
-    const unsigned t = __reduce_add_sync(0xFFFFFFFFu, tests);
-    if ((threadIdx.x & 31u) == 0u && t) atomicAdd(fb.tests_run, (unsigned long long)t);
+  if (!BOXES) {  // nothing can be reset: the counts are cleared here, not by a memset before the launch
+    if (slot == 0) *fb.counts = CallCounts{0, 0};
+    return;
   }
+  append_compact(resets > 0u, env, fb.reset_ids, &fb.counts->resets);
+  const unsigned t = __reduce_add_sync(0xFFFFFFFFu, tests);  // one atomic per warp
+  if ((threadIdx.x & 31u) == 0u && t) atomicAdd(&fb.counts->tests, (unsigned long long)t);
 }
 
 // Grouping order: key = rotor-type index * 4 + mode (12 keys). Each window of
@@ -288,6 +290,10 @@ cudaError_t launch_fused_b(const FleetBuffers& fb, const StepParams& P, int n_st
   }
   const uint32_t slots = fb.order ? fb.n_slots : fb.n;
   const unsigned grid = (slots + B - 1) / B;
+  if (BOXES) {
+    const cudaError_t e = cudaMemsetAsync(fb.counts, 0, sizeof(CallCounts), st);
+    if (e != cudaSuccess) return e;
+  }
   kernel<<<grid, B, 0, st>>>(fb, P, n_steps, substeps);
   return cudaGetLastError();
 }
@@ -329,9 +335,6 @@ FusedTuning fused_tuning_from_env() {
 
 cudaError_t launch_fused_step(const FleetBuffers& fb_in, const StepParams& P, int integrator, int n_steps,
                               int substeps, cudaStream_t st) {
-  cudaError_t e = cudaMemsetAsync(fb_in.n_reset, 0, sizeof(uint32_t), st);
-  if (e == cudaSuccess && fb_in.tests_run) e = cudaMemsetAsync(fb_in.tests_run, 0, sizeof(unsigned long long), st);
-  if (e != cudaSuccess) return e;
   const FusedTuning t = fused_tuning_from_env();
   FleetBuffers fb = fb_in;
   if (!t.sorted) fb.order = nullptr;

@@ -126,7 +126,7 @@ extern "C" ag_status ag_collision_tests_run(ag_ctx* ctx, uint64_t* tests) {
   if (s != AG_OK) return s;
   if (!tests) return agh::fail_invalid(ctx, "ag_collision_tests_run: tests is NULL");
   unsigned long long v = 0;
-  s = agh::check_cuda(ctx, cudaMemcpyAsync(&v, ctx->fb.tests_run, sizeof(v), cudaMemcpyDeviceToHost, ctx->stream),
+  s = agh::check_cuda(ctx, cudaMemcpyAsync(&v, &ctx->fb.counts->tests, sizeof(v), cudaMemcpyDeviceToHost, ctx->stream),
                       "copy test count");
   if (s == AG_OK) s = agh::check_cuda(ctx, cudaStreamSynchronize(ctx->stream), "synchronize");
   if (s == AG_OK) *tests = (uint64_t)v;

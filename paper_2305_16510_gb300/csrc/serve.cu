@@ -225,11 +225,11 @@ __global__ void k_fill_body(float* body, uint32_t n, float m, float jx, float jy
   body[i] = m; body[n + i] = jx; body[2 * n + i] = jy; body[3 * n + i] = jz;
 }
 
-// Device memory of the server's own device, which a kernel can read in place.
+// Device memory of the server's own device, aligned to 4 bytes, which a kernel can read in place.
 bool on_device(const void* p, int device) {
   cudaPointerAttributes pa;
   const bool own = cudaPointerGetAttributes(&pa, p) == cudaSuccess && pa.type == cudaMemoryTypeDevice &&
-                   pa.device == device;
+                   pa.device == device && reinterpret_cast<uintptr_t>(p) % 4 == 0;
   cudaGetLastError();
   return own;
 }
