@@ -408,6 +408,12 @@ ag_status ag_reach_begin(ag_ctx* ctx, const ag_reach_config* cfg, const float* g
  * for a NULL or misaligned pointer. */
 ag_status ag_reach_step(ag_ctx* ctx, const float* actions, float* obs, float* reward, uint8_t* done);
 
+/* ag_reach_step that also writes the step's collision flags uint8[n_envs]
+ * (those ag_get_state returns) to `collided`, device memory of the context's
+ * device; NULL is ag_reach_step. */
+ag_status ag_reach_step_flags(ag_ctx* ctx, const float* actions, float* obs, float* reward, uint8_t* done,
+                              uint8_t* collided);
+
 /* Observations float[n_envs][13] (device) of the current states, as written
  * by ag_reach_step; nothing else changes. AG_ERR_STATE before ag_reach_begin. */
 ag_status ag_reach_observe(ag_ctx* ctx, float* obs);

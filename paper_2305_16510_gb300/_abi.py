@@ -127,6 +127,7 @@ SIGNATURES = {
     "ag_reach_config_default": (None, [ctypes.POINTER(ag_reach_config)]),
     "ag_reach_begin": (ctypes.c_int, [_vp, ctypes.POINTER(ag_reach_config), _vp]),
     "ag_reach_step": (ctypes.c_int, [_vp, _vp, _vp, _vp, _vp]),
+    "ag_reach_step_flags": (ctypes.c_int, [_vp, _vp, _vp, _vp, _vp, _vp]),
     "ag_reach_observe": (ctypes.c_int, [_vp, _vp]),
     "ag_server_config_default": (None, [ctypes.POINTER(ag_server_config)]),
     "ag_server_create": (ctypes.c_int, [ctypes.POINTER(ag_server_config), ctypes.POINTER(_vp)]),
@@ -375,6 +376,12 @@ def ag_reach_begin(ctx: int, cfg: ag_reach_config, goals) -> None:
 
 def ag_reach_step(ctx: int, actions, obs, reward, done) -> None:
     _check(lib().ag_reach_step(ctx, ptr(actions), ptr(obs), ptr(reward), ptr(done)), "ag_reach_step", ctx)
+
+
+def ag_reach_step_flags(ctx: int, actions, obs, reward, done, collided) -> None:
+    """ag_reach_step that also writes the collision flags uint8 [n] (a device array)."""
+    _check(lib().ag_reach_step_flags(ctx, ptr(actions), ptr(obs), ptr(reward), ptr(done), ptr(collided)),
+           "ag_reach_step_flags", ctx)
 
 
 def ag_reach_observe(ctx: int, obs) -> None:

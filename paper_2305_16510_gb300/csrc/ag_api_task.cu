@@ -166,7 +166,8 @@ ag_status ag_reach_begin(ag_ctx* ctx, const ag_reach_config* cfg, const float* g
   return AG_OK;
 }
 
-static agk::ReachArgs reach_args(ag_ctx* ctx, const float* actions, float* obs, float* reward, uint8_t* done) {
+static agk::ReachArgs reach_args(ag_ctx* ctx, const float* actions, float* obs, float* reward, uint8_t* done,
+                                 uint8_t* collided) {
   agk::ReachArgs a;
   a.fb = ctx->fb;
   a.actions = actions;
@@ -175,6 +176,7 @@ static agk::ReachArgs reach_args(ag_ctx* ctx, const float* actions, float* obs, 
   a.obs = obs;
   a.reward = reward;
   a.done = done;
+  a.collided = collided;
   const ag_reach_config& c = ctx->reach;
   for (int k = 0; k < 4; ++k) {
     a.scale[k] = c.action_scale[k];
@@ -191,13 +193,18 @@ static agk::ReachArgs reach_args(ag_ctx* ctx, const float* actions, float* obs, 
 }
 
 ag_status ag_reach_step(ag_ctx* ctx, const float* actions, float* obs, float* reward, uint8_t* done) {
+  return ag_reach_step_flags(ctx, actions, obs, reward, done, nullptr);
+}
+
+ag_status ag_reach_step_flags(ag_ctx* ctx, const float* actions, float* obs, float* reward, uint8_t* done,
+                              uint8_t* collided) {
   agk::NvtxRange range("ag_reach_step");
   ag_status s = enter(ctx);
   if (s != AG_OK) return s;
   if (!ctx->reach_active) return AG_ERR_STATE;
   if (!actions || !obs || !reward || !done) return fail_invalid(ctx, "actions, obs, reward and done must be non-NULL");
   if (reinterpret_cast<uintptr_t>(actions) % 16 != 0) return fail_invalid(ctx, "actions must be 16-byte aligned");
-  const agk::ReachArgs a = reach_args(ctx, actions, obs, reward, done);
+  const agk::ReachArgs a = reach_args(ctx, actions, obs, reward, done, collided);
   return check_cuda(ctx, agk::launch_reach_step(a, step_params(ctx), (int)ctx->cfg.integrator,
                                                 (int)ctx->cfg.substeps_per_step, ctx->stream), "task step launch");
 }
@@ -208,7 +215,7 @@ ag_status ag_reach_observe(ag_ctx* ctx, float* obs) {
   if (s != AG_OK) return s;
   if (!ctx->reach_active) return AG_ERR_STATE;
   if (!obs) return fail_invalid(ctx, "obs must be non-NULL");
-  return check_cuda(ctx, agk::launch_reach_observe(reach_args(ctx, nullptr, obs, nullptr, nullptr), ctx->stream),
+  return check_cuda(ctx, agk::launch_reach_observe(reach_args(ctx, nullptr, obs, nullptr, nullptr, nullptr), ctx->stream),
                     "task observe launch");
 }
 

@@ -126,6 +126,7 @@ __global__ void __launch_bounds__(kTaskBlock, BOXES ? 8 : 12)
     else
       s = reach_fly<8, INTEG, DRAG>(a, P, i, act, mode, substeps, n_obs, boxes, t, hit);
     fb.collided[i] = hit ? 1 : 0;
+    if (a.collided) a.collided[i] = hit ? 1 : 0;
 #pragma unroll
     for (int k = 0; k < 4; ++k) fb.targets[k * n + i] = t[k];  // the commands, as ag_set_commands keeps them
     reach_tail(a, i, s, hit, steps_before, g, stage + threadIdx.x * kObs);

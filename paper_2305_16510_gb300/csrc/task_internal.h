@@ -16,6 +16,7 @@ struct ReachArgs {
   float* obs;            // [n][13]
   float* reward;         // [n]
   uint8_t* done;         // [n]
+  uint8_t* collided;     // [n] a copy of the flags for the caller (NULL = none)
   float scale[4], offset[4];
   float w_v, w_omega, crash, max_dist;
   uint32_t max_steps;

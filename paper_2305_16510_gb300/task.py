@@ -66,8 +66,7 @@ class ReachEnv:
             a = a.to(device=self.device, dtype=torch.float32).contiguous().clone()
         if tuple(a.shape) != (self.n, ACTION_DIM):
             raise ValueError(f"actions must have shape ({self.n}, {ACTION_DIM})")
-        _abi.ag_reach_step(self.fleet.ctx, a, self.obs, self.reward, self.done)
-        _abi.ag_get_state(self.fleet.ctx, collided=self._col)
+        _abi.ag_reach_step_flags(self.fleet.ctx, a, self.obs, self.reward, self.done, self._col)
         self._keep_actions = a
         return self.obs, self.reward, self.done, {"collided": self._col}
 
