@@ -36,10 +36,14 @@ ag_status render_depth_impl(ag_ctx* ctx, uint32_t width, uint32_t height, float 
     if (!on_device(env_ids))
       for (uint32_t j = 0; j < n_cams; ++j)
         if (env_ids[j] >= n) return fail_invalid(ctx, "environment id out of range");
-    if (!ctx->cam_ids && (s = alloc_or_oom(ctx, &ctx->cam_ids, n, "the camera ids")) != AG_OK) return s;
-    if ((s = check_cuda(ctx, cudaMemcpyAsync(ctx->cam_ids, env_ids, n_cams * sizeof(uint32_t), cudaMemcpyDefault, st),
-                        "copy camera ids")) != AG_OK) return s;
-    ids_dev = ctx->cam_ids;
+    if (on_own_device(ctx, env_ids)) {
+      ids_dev = env_ids;  // read in place: a copy first made a launch of few cameras a quarter longer
+    } else {
+      if (!ctx->cam_ids && (s = alloc_or_oom(ctx, &ctx->cam_ids, n, "the camera ids")) != AG_OK) return s;
+      if ((s = check_cuda(ctx, cudaMemcpyAsync(ctx->cam_ids, env_ids, n_cams * sizeof(uint32_t), cudaMemcpyDefault,
+                                               st), "copy camera ids")) != AG_OK) return s;
+      ids_dev = ctx->cam_ids;
+    }
   }
   const size_t count = (size_t)n_cams * width * height;
   const bool out_on_device = live_pairs ? true : on_device(depth);
