@@ -73,7 +73,7 @@ __global__ void __launch_bounds__(kServeBlock, 4) k_serve_step(const ServeDesc* 
   uint32_t resets = 0, tests = 0;
   bool hit = false;
   const EnvBoxes boxes(d.fb, env);
-  simulate<4, INTEG, DRAG>(d.fb, P, env, d.steps, substeps, (int)d.fb.n_obs, boxes, d.seed_lo, d.seed_hi, resets, hit,
+  simulate<4, INTEG, DRAG, true>(d.fb, P, env, d.steps, substeps, (int)d.fb.n_obs, boxes, d.seed_lo, d.seed_hi, resets, hit,
                            tests);
 }
 
