@@ -221,6 +221,13 @@ bool on_device(const void* p) {
   return dev;
 }
 
+bool on_host(const void* p) {
+  cudaPointerAttributes pa;
+  const bool host = cudaPointerGetAttributes(&pa, p) == cudaSuccess && pa.type == cudaMemoryTypeUnregistered;
+  cudaGetLastError();
+  return host;
+}
+
 bool on_own_device(const ag_ctx* ctx, const void* p) {
   cudaPointerAttributes pa;
   const bool own = cudaPointerGetAttributes(&pa, p) == cudaSuccess && pa.type == cudaMemoryTypeDevice &&

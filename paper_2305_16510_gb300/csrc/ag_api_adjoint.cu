@@ -2,6 +2,7 @@
 // (ag_set_gains, ag_rollout_loss, ag_backward).
 #include <cmath>
 #include <cstdint>
+#include <cstring>
 #include <string>
 
 #include <cuda_runtime.h>
@@ -105,7 +106,11 @@ extern "C" ag_status ag_set_gains(ag_ctx* ctx, const float* gains12) {
   if (s != AG_OK) return s;
   if (!gains12) return fail_invalid(ctx, "gains is NULL");
   float g[12];
-  if ((s = check_cuda(ctx, cudaMemcpy(g, gains12, sizeof(g), cudaMemcpyDefault), "copy gains")) != AG_OK) return s;
+  if (on_host(gains12)) {
+    std::memcpy(g, gains12, sizeof(g));  // no CUDA call: a synchronous cudaMemcpy waits for the device's queued work
+  } else if ((s = check_cuda(ctx, cudaMemcpy(g, gains12, sizeof(g), cudaMemcpyDefault), "copy gains")) != AG_OK) {
+    return s;
+  }
   for (int i = 0; i < 12; ++i)
     if (!std::isfinite(g[i])) return fail_invalid(ctx, "gains must be finite");
   for (int i = 0; i < 3; ++i) {

@@ -59,6 +59,8 @@ ag_status enter(ag_ctx* ctx);
 agk::StepParams step_params(const ag_ctx* ctx);
 // true for device or managed memory (a kernel can read it), false for host memory.
 bool on_device(const void* p);
+// true for pageable host memory (no copy in flight can be writing it).
+bool on_host(const void* p);
 // true for memory of the context's own device, aligned to 4 bytes, which its
 // kernels read and write in place (anything else is copied).
 bool on_own_device(const ag_ctx* ctx, const void* p);
