@@ -35,8 +35,11 @@
 // frame, radius |h| with a rounding margin) lies beyond max_range along the
 // axis, behind the camera, or outside one of the four planes through the
 // camera origin that bound the tile's rays (y = dy x and z = dz x at the
-// tile's extreme pixel centres). A culled box can change no pixel of the
-// tile, so the image is the same as without culling. When each component of
+// tile's extreme pixel centres), and then when the box itself does
+// (box_culled: 1,024 cameras x 270 x 480 among 16 boxes take 108.8 us with it
+// and 128.1 us without, of which storing the images takes 76). A culled box
+// can change no pixel of the tile, so the image is the same as without
+// culling. When each component of
 // a live box's ray direction keeps one sign over the tile, the near and far
 // slab bound of every axis is known for the whole tile: the tile's copy of
 // the record then holds them in place of lo and hi, and the per-pixel min /
@@ -58,7 +61,8 @@ constexpr int kDepthCols = 4;                                       // consecuti
 constexpr int kDepthColThreads = kDepthTile / kDepthCols;           // threads across a tile row: 8
 constexpr int kDepthRowStep = kDepthThreads / kDepthColThreads;     // rows between a thread's rows: 16
 constexpr int kDepthRowsPer = kDepthTile / kDepthRowStep;           // rows per thread: 2
-constexpr int kDepthTilesPerBlock = 8;                              // tiles of one camera per block
+constexpr int kDepthTilesPerBlock = 8;                              // at most: tiles of one camera per block
+constexpr int kDepthFill = 4;                                       // blocks per SM worth having
 static_assert(kDepthCols == 4 && kDepthRowsPer * kDepthRowStep == kDepthTile, "4 x 2 pixels per thread");
 
 struct CamPose {
@@ -136,6 +140,37 @@ __device__ __forceinline__ bool sphere_culled(float4 s, const TileRays& t, float
   if (t.zhi * s.x - s.z < -rho * t.nzhi) return true;
   if (s.z - t.zlo * s.x < -rho * t.nzlo) return true;
   return false;
+}
+
+// The box itself cannot meet any ray of the tile at depth below max_range,
+// where its sphere might: every corner of the box lies outside one of the four
+// planes (its extent along a plane's normal is sum_i h_i |n . a_i|, a_i = row i
+// of M, the box's axes in the camera frame), or no ray comes within one of the
+// box's slabs up to max_range (a ray's box-frame direction is linear in y and
+// z, so the tile's corner rays bound it). The margins cover float32 rounding
+// and a quaternion norm off by the 1e-4 that ag_set_obstacles admits.
+__device__ __forceinline__ bool box_culled(const float4* rec, float4 s, const TileRays& t, float max_range) {
+  const float4 r0 = rec[0], r1 = rec[1], r2 = rec[2], r3 = rec[3];
+  const float m[3][3] = {{r0.x, r0.y, r0.z}, {r0.w, r1.x, r1.y}, {r1.z, r1.w, r2.x}};
+  const float lo[3] = {r2.y, r2.z, r2.w}, hi[3] = {r3.x, r3.y, r3.z};
+  const float far = 5e-4f * (fabsf(s.x) + fabsf(s.y) + fabsf(s.z));
+  float ey0 = 0.f, ey1 = 0.f, ez0 = 0.f, ez1 = 0.f;  // extents along the four normals
+  bool out = false;
+#pragma unroll
+  for (int i = 0; i < 3; ++i) {
+    const float h = 0.5005f * (hi[i] - lo[i]);
+    ey1 = fmaf(h, fabsf(fmaf(t.yhi, m[i][0], -m[i][1])), ey1);
+    ey0 = fmaf(h, fabsf(fmaf(t.ylo, m[i][0], -m[i][1])), ey0);
+    ez1 = fmaf(h, fabsf(fmaf(t.zhi, m[i][0], -m[i][2])), ez1);
+    ez0 = fmaf(h, fabsf(fmaf(t.zlo, m[i][0], -m[i][2])), ez0);
+    const float y0 = t.ylo * m[i][1], y1 = t.yhi * m[i][1], z0 = t.zlo * m[i][2], z1 = t.zhi * m[i][2];
+    const float dmin = m[i][0] + fminf(y0, y1) + fminf(z0, z1), dmax = m[i][0] + fmaxf(y0, y1) + fmaxf(z0, z1);
+    const float eps = 1e-4f * (fabsf(lo[i]) + fabsf(hi[i]) + max_range) + 1e-6f;
+    out |= lo[i] > fmaf(max_range, fmaxf(dmax, 0.f), eps) || hi[i] < fmaf(max_range, fminf(dmin, 0.f), -eps);
+  }
+  out |= fmaf(t.yhi, s.x, -s.y) + ey1 < -far * t.nyhi || fmaf(-t.ylo, s.x, s.y) + ey0 < -far * t.nylo;
+  out |= fmaf(t.zhi, s.x, -s.z) + ez1 < -far * t.nzhi || fmaf(-t.zlo, s.x, s.z) + ez0 < -far * t.nzlo;
+  return out;
 }
 
 // Flags of a live (tile, box) pair: kLive, and kFixedSigns when each
@@ -231,13 +266,13 @@ __global__ void __launch_bounds__(kDepthThreads) k_render_depth(DepthArgs a) {
   extern __shared__ float4 tile_recs[];
   __shared__ int n_live[kDepthTilesPerBlock];
   __shared__ uint32_t tile_x0[kDepthTilesPerBlock], tile_y0[kDepthTilesPerBlock];  // pixel origin of each tile
-  // block -> (camera, group of kDepthTilesPerBlock consecutive tiles); cameras cam0, cam0 + 1, ...
+  // block -> (camera, group of tiles_per_block consecutive tiles); cameras cam0, cam0 + 1, ...
   const uint32_t tiles_x = (a.width + kDepthTile - 1) / kDepthTile;
   const uint32_t tiles = tiles_x * ((a.height + kDepthTile - 1) / kDepthTile);
-  const uint32_t groups = (tiles + kDepthTilesPerBlock - 1) / kDepthTilesPerBlock;
+  const uint32_t per_block = a.tiles_per_block, groups = (tiles + per_block - 1) / per_block;
   const uint32_t j = a.cam0 + blockIdx.x / groups;
-  const uint32_t t_begin = (blockIdx.x % groups) * kDepthTilesPerBlock;
-  const uint32_t t_end = min(t_begin + kDepthTilesPerBlock, tiles);
+  const uint32_t t_begin = (blockIdx.x % groups) * per_block;
+  const uint32_t t_end = min(t_begin + per_block, tiles);
   const uint32_t env = a.env_ids ? a.env_ids[j] : j;
   // a camera id outside the fleet reads nothing and yields a NaN image
   const bool bad_env = env >= a.n;
@@ -263,7 +298,7 @@ __global__ void __launch_bounds__(kDepthThreads) k_render_depth(DepthArgs a) {
   const uint32_t L = n_obs <= 16 ? 16u : 32u;  // the same for the whole block
   const uint32_t lane = threadIdx.x % 32, g = lane / L, gl = lane % L;
   const unsigned gmask = L == 32u ? 0xFFFFFFFFu : (0xFFFFu << (16u * g));  // the ballot bits of this group
-  for (uint32_t w0 = threadIdx.x / 32; w0 < (uint32_t)kDepthTilesPerBlock; w0 += kWarps * (32u / L)) {
+  for (uint32_t w0 = threadIdx.x / 32; w0 < per_block; w0 += kWarps * (32u / L)) {
     const uint32_t w = w0 + kWarps * g, t = t_begin + w;  // this group's tile
     const bool valid = t < t_end;
     const uint32_t tv = valid ? t : t_begin;               // an idle group computes on a real tile
@@ -284,7 +319,9 @@ __global__ void __launch_bounds__(kDepthThreads) k_render_depth(DepthArgs a) {
     for (int k0 = 0; k0 < n_obs; k0 += (int)L) {  // the same trip count for the whole warp
       const int k = k0 + (int)gl;
       uint8_t f = 0;
-      if (valid && k < n_obs && !sphere_culled(spheres[k], r, a.max_range)) f = slab_signs(recs + 4 * k, r);
+      if (valid && k < n_obs && !sphere_culled(spheres[k], r, a.max_range) &&
+          !box_culled(recs + 4 * k, spheres[k], r, a.max_range))
+        f = slab_signs(recs + 4 * k, r);
       const unsigned m = __ballot_sync(0xFFFFFFFFu, f != 0) & gmask;
       if (f && MODE != kCountLive) {
         const int at = count + __popc(m & ((1u << lane) - 1u));
@@ -403,12 +440,23 @@ __global__ void __launch_bounds__(kDepthThreads) k_render_depth(DepthArgs a) {
 cudaError_t launch_render_depth(const DepthArgs& a_in, cudaStream_t st) {
   const uint64_t tiles = (uint64_t)((a_in.width + kDepthTile - 1) / kDepthTile) *
                          ((a_in.height + kDepthTile - 1) / kDepthTile);
-  const uint64_t groups = (tiles + kDepthTilesPerBlock - 1) / kDepthTilesPerBlock;
+  // eight tiles per block share its camera's records; a launch too small to give every SM kDepthFill
+  // blocks takes fewer, down to one per block (61 cameras x 213 x 117: 8.4 us a pass against 10.9; filling
+  // to 2 or 8 blocks per SM measures the same)
+  DepthArgs a = a_in;
+  int sms = 0, dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  if (e != cudaSuccess) return e;
+  a.tiles_per_block = kDepthTilesPerBlock;
+  while (a.tiles_per_block > 1 &&
+         a_in.n_cams * ((tiles + a.tiles_per_block - 1) / a.tiles_per_block) < (uint64_t)kDepthFill * sms)
+    a.tiles_per_block /= 2;
+  const uint64_t groups = (tiles + a.tiles_per_block - 1) / a.tiles_per_block;
   // at most 2^31 - 1 blocks per launch
   const uint64_t cams_per_launch = ((1ull << 31) - 1) / groups;
   // the tiles' live-box records: at most 8 x 64 x 64 B = 32 KB, within the default 48 KB per block
-  const size_t smem = (size_t)kDepthTilesPerBlock * a_in.n_obs * 4 * sizeof(float4);
-  DepthArgs a = a_in;
+  const size_t smem = (size_t)a.tiles_per_block * a_in.n_obs * 4 * sizeof(float4);
   a.vec_store = a.width % 4 == 0 && (reinterpret_cast<uintptr_t>(a.out) & 15u) == 0;
   for (uint64_t c0 = 0; c0 < a_in.n_cams; c0 += cams_per_launch) {
     const uint64_t nc = a_in.n_cams - c0 < cams_per_launch ? a_in.n_cams - c0 : cams_per_launch;
@@ -416,7 +464,7 @@ cudaError_t launch_render_depth(const DepthArgs& a_in, cudaStream_t st) {
     if (a.live_pairs) k_render_depth<kCountLive><<<(unsigned)(nc * groups), kDepthThreads, 0, st>>>(a);
     else if (a.ieee_div) k_render_depth<kRenderIeee><<<(unsigned)(nc * groups), kDepthThreads, smem, st>>>(a);
     else k_render_depth<kRenderFast><<<(unsigned)(nc * groups), kDepthThreads, smem, st>>>(a);
-    const cudaError_t e = cudaGetLastError();
+    e = cudaGetLastError();
     if (e != cudaSuccess) return e;
   }
   return cudaSuccess;

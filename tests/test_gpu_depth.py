@@ -227,3 +227,20 @@ def test_live_pair_count_bounds_and_monotone_in_range():
     empty.reset(None, 3)
     assert _abi.ag_depth_live_pairs(empty.ctx, 64, 48, hfov, 10.0, None, None, 16) == 0
     empty.close()
+
+
+@pytest.mark.parametrize("width,height", [(32, 32), (33, 31), (213, 117), (480, 270)])
+def test_image_does_not_depend_on_how_many_cameras_a_launch_has(width, height):
+    """A launch of few cameras renders fewer tiles per block (8, 4, 2 or 1): the
+    same camera's image is the same bits in every launch."""
+    w = W.scaled(W.WORKLOADS["obstacles"], 640)
+    inp = W.make_inputs(w, 12)
+    fl = gpu_fleet(w, inp, 12)
+    fl.reset(None, 12)
+    hfov = 1.3
+    whole = fl.render_depth(width, height, hfov, 8.0)
+    assert (whole < 8.0).any() and (whole == 8.0).any()
+    for count in (1, 3, 17, 40, 75, 150, 300):
+        ids = torch.arange(639, 639 - count, -1, dtype=torch.int32, device="cuda")
+        assert torch.equal(fl.render_depth(width, height, hfov, 8.0, env_ids=ids), whole[ids.long()])
+    fl.close()
