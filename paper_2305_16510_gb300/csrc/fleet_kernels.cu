@@ -153,10 +153,7 @@ __global__ void __launch_bounds__(256) k_pack_boxes(FleetBuffers fb, const float
   float v[10];
 #pragma unroll
   for (int f = 0; f < 10; ++f) v[f] = src[((size_t)blockIdx.y * 10 + f) * pitch + env];
-  const size_t at = (size_t)(k0 + blockIdx.y) * fb.n + env;
-  fb.box_bound[at] = make_float4(v[0], v[1], v[2], sqrtf(fmaf(v[5], v[5], fmaf(v[4], v[4], v[3] * v[3]))));
-  fb.box_rest[2 * at] = make_float4(v[3], v[4], v[5], v[6]);
-  fb.box_rest[2 * at + 1] = make_float4(v[7], v[8], v[9], 0.f);
+  pack_box(fb, k0 + blockIdx.y, env, v);
 }
 
 __global__ void __launch_bounds__(256) k_unpack_boxes(FleetBuffers fb, float* __restrict__ dst, uint32_t k0) {

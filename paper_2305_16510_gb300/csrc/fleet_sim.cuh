@@ -203,6 +203,14 @@ template <bool GROUPED> struct EnvBoxesT {
 };
 using EnvBoxes = EnvBoxesT<false>;
 
+// The records of box k of environment env from its ten fields (ag_set_obstacles).
+__device__ __forceinline__ void pack_box(const FleetBuffers& fb, uint32_t k, uint32_t env, const float (&v)[10]) {
+  const size_t at = (size_t)k * fb.n + env;
+  fb.box_bound[at] = make_float4(v[0], v[1], v[2], sqrtf(fmaf(v[5], v[5], fmaf(v[4], v[4], v[3] * v[3]))));
+  fb.box_rest[2 * at] = make_float4(v[3], v[4], v[5], v[6]);
+  fb.box_rest[2 * at + 1] = make_float4(v[7], v[8], v[9], 0.f);
+}
+
 // New poses for every box of environment env, written to its records (the
 // half-extents and the sphere radius stay).
 static __device__ __noinline__ void redraw_boxes(float4* box_bound, float4* box_rest, const BoxRandDev* box_rand,

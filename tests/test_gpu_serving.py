@@ -177,3 +177,27 @@ def test_bounded_wait_and_invalid_requests(pool):
         with pytest.raises(_abi.AgError) as e:
             s.submit(rp.request(N_POOL, 10, 32, seed=1))
         assert e.value.status == _abi.AG_ERR_OOM
+
+
+@pytest.mark.parametrize("n,n_obs,with_body", [(1, 0, False), (33, 1, True), (257, 33, False), (4097, 3, True)])
+def test_request_inputs_in_host_memory_give_the_same_results(n, n_obs, with_body):
+    """Inputs in device memory are read by the admission kernel, host inputs are
+    copied first: the same request gives the same bits either way, at odd
+    offsets into the pool."""
+    from paper_2305_16510_gb300.serving import RequestPool
+    w = W.Workload("host", n + 7, 4, 1, max(n_obs, 1), n + 7, 0, 0, mass_rand=0.2, mode_mix=(0, 1, 2, 3))
+    inp = W.make_inputs(w, 15)
+    boxes = np.ascontiguousarray(inp.boxes.reshape(-1, n + 7))
+    pool = RequestPool(inp.modes, inp.targets, boxes, inp.body if with_body else None)
+    host = _abi.ag_request()
+    host.n_envs, host.n_steps, host.n_obstacles, host.seed, host.pitch = n, 60, n_obs, 9, n + 7
+    host.modes = inp.modes.ctypes.data + 5
+    host.targets = inp.targets.ctypes.data + 20
+    host.body = inp.body.ctypes.data + 20 if with_body else None
+    host.boxes = boxes.ctypes.data + 20 if n_obs else None
+    with _server(max_active=4, chunk_steps=25, hbm_budget_bytes=64 << 20) as s:
+        a = s.wait(s.submit(pool.request(n_envs=n, n_steps=60, n_obstacles=n_obs, seed=9, offset=5)))
+        b = s.wait(s.submit(host))
+    np.testing.assert_array_equal(a[0], b[0])
+    np.testing.assert_array_equal(a[1], b[1])
+    assert np.isfinite(a[0]).all() and (a[1] >= 1).all()
