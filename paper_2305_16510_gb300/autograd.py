@@ -53,6 +53,7 @@ class RolloutLoss(torch.autograd.Function):
         gt = torch.empty((4, fleet.n), dtype=torch.float32, device=fleet.device) if ctx.has_targets else None
         w = grad_loss.to(device=fleet.device, dtype=torch.float32).contiguous()
         _abi.ag_backward(fleet.ctx, w, gx, gg, None, gt)
+        fleet._keep_weights = w  # read by the queued sweep
         return gx, gg.to(ctx.gains_device), gt, None, None, None, None, None, None
 
 

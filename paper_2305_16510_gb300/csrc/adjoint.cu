@@ -159,7 +159,10 @@ template <bool FULL_TAPE> struct Record {
     normalize(x.s.q);
     const Body b = body_at(ab, env);
     const Command cm = command_at<MODE>(ab, env);
-    const V3 goal = {ab.p_goal[env], ab.p_goal[n + env], ab.p_goal[2 * n + env]};
+    const V3 goal = {ab.goal_in[env], ab.goal_in[n + env], ab.goal_in[2 * n + env]};
+    ab.p_goal[env] = goal.x;
+    ab.p_goal[n + env] = goal.y;
+    ab.p_goal[2 * n + env] = goal.z;
     float loss = 0.f;
     uint32_t all_pass = (1u << NROT) - 1u;
     float4* entry = ab.tape + slot;

@@ -23,7 +23,8 @@ struct AdjointBuffers {
   const uint8_t* modes;        // [n] command mode per env (values above 3 act as a wrench)
   const float* targets;        // [4][n] command targets
   const uint32_t* order;       // [n_slots] thread slot -> environment, grouped by rotor type and mode
-  const float* p_goal;         // [3][n]
+  const float* goal_in;        // [3][n] the record's goals (the caller's array, or p_goal)
+  float* p_goal;               // [3][n] kept for the sweep, written by the record
   float* ckpt;                 // [S][21] slot (NULL with full_tape)
   float4* tape;                // [n_steps + 1][4] (full_tape) or [K][4], slot
   float* inv_q0;               // slot: 1 / |q_0| of the given initial quaternion

@@ -99,6 +99,8 @@ ag_status ensure_adjoint(ag_ctx* ctx, int n_steps, int K) {
   return AG_OK;
 }
 
+bool overlap(const float* a, size_t na, const float* b, size_t nb) { return a < b + nb && b < a + na; }
+
 }  // namespace
 
 extern "C" ag_status ag_set_gains(ag_ctx* ctx, const float* gains12) {
@@ -136,8 +138,14 @@ extern "C" ag_status ag_rollout_loss(ag_ctx* ctx, uint32_t n_steps, float w_pos,
   ctx->adj_recorded = false;  // the buffers of the last record may be replaced
   if ((s = ensure_adjoint(ctx, (int)n_steps, K)) != AG_OK) return s;
   agk::AdjointBuffers& a = ctx->adj;
-  if ((s = check_cuda(ctx, cudaMemcpyAsync((void*)a.p_goal, p_goal, 3 * n * sizeof(float), cudaMemcpyDefault,
-                                           ctx->stream), "copy goals")) != AG_OK) return s;
+  // goals and loss in the context's own device memory are read and written in place
+  const bool loss_here = on_own_device(ctx, loss);
+  a.goal_in = p_goal;
+  if (!on_own_device(ctx, p_goal) || (loss_here && overlap(loss, n, p_goal, 3 * n))) {
+    if ((s = check_cuda(ctx, cudaMemcpyAsync(a.p_goal, p_goal, 3 * n * sizeof(float), cudaMemcpyDefault, ctx->stream),
+                        "copy goals")) != AG_OK) return s;
+    a.goal_in = a.p_goal;
+  }
   a.state = ctx->fb.state; a.motors = ctx->fb.motors; a.body = ctx->fb.body; a.targets = ctx->fb.targets;
   a.modes = ctx->fb.modes;
   a.order = ctx->fb.order;
@@ -145,12 +153,12 @@ extern "C" ag_status ag_rollout_loss(ag_ctx* ctx, uint32_t n_steps, float w_pos,
   a.n = c.n_envs; a.n_quad = c.n_quad; a.n_hexa = c.n_hexa; a.n_octo = c.n_octo;
   a.n_steps = (int)n_steps; a.K = K; a.w_pos = w_pos; a.w_omega = w_omega;
   ctx->adj_P = step_params(ctx);
-  const bool direct = on_own_device(ctx, loss);
   agk::AdjointBuffers rec = a;
-  if (direct) rec.loss = loss;
+  if (loss_here) rec.loss = loss;
+  a.goal_in = nullptr;  // the caller's array is not read after this launch
   if ((s = check_cuda(ctx, agk::launch_record(rec, ctx->adj_P, ctx->stream), "record launch")) != AG_OK) return s;
   ctx->adj_recorded = true;
-  if (!direct && (s = check_cuda(ctx, cudaMemcpyAsync(loss, a.loss, n * sizeof(float), cudaMemcpyDefault, ctx->stream),
+  if (!loss_here && (s = check_cuda(ctx, cudaMemcpyAsync(loss, a.loss, n * sizeof(float), cudaMemcpyDefault, ctx->stream),
                                  "copy loss out")) != AG_OK) return s;
   if (saturated)
     s = check_cuda(ctx, cudaMemcpyAsync(saturated, a.saturated, n, cudaMemcpyDefault, ctx->stream), "copy flags out");
@@ -169,12 +177,6 @@ extern "C" ag_status ag_backward(ag_ctx* ctx, const float* loss_weights, float* 
   if (!grad_x0 && !grad_gains && !grad_gains_per_env && !grad_targets) return AG_OK;
   agk::AdjointBuffers a = ctx->adj;
   const size_t n = ctx->cfg.n_envs;
-  if (loss_weights) {
-    if ((s = check_cuda(ctx, cudaMemcpyAsync((void*)a.loss_weights, loss_weights, n * sizeof(float),
-                                             cudaMemcpyDefault, ctx->stream), "copy weights")) != AG_OK) return s;
-  } else {
-    a.loss_weights = nullptr;
-  }
   // a wanted output in the context's own device memory is written in place, any other through the staging
   // buffer; unwanted ones are not formed
   struct Out { float* user; float** field; float* stage; size_t count; const char* what; };
@@ -187,6 +189,15 @@ extern "C" ag_status ag_backward(ag_ctx* ctx, const float* loss_weights, float* 
     staged[k] = outs[k].user && !on_own_device(ctx, outs[k].user);
     *outs[k].field = staged[k] ? outs[k].stage : outs[k].user;
   }
+  // the weights are read in place where a copy is not needed
+  bool weights_here = loss_weights && on_own_device(ctx, loss_weights);
+  for (int k = 0; k < 4; ++k)
+    if (weights_here && outs[k].user && overlap(outs[k].user, outs[k].count, loss_weights, n)) weights_here = false;
+  if (loss_weights && !weights_here &&
+      (s = check_cuda(ctx, cudaMemcpyAsync((void*)a.loss_weights, loss_weights, n * sizeof(float), cudaMemcpyDefault,
+                                           ctx->stream), "copy weights")) != AG_OK)
+    return s;
+  if (!loss_weights || weights_here) a.loss_weights = loss_weights;
   if ((s = check_cuda(ctx, agk::launch_adjoint(a, ctx->adj_P, ctx->stream), "adjoint launch")) != AG_OK) return s;
   for (int k = 0; k < 4; ++k)
     if (staged[k] && (s = check_cuda(ctx, cudaMemcpyAsync(outs[k].user, outs[k].stage, outs[k].count * sizeof(float),
