@@ -94,15 +94,15 @@ __device__ __forceinline__ void append_compact(bool pred, uint32_t env, uint32_t
   if (pred) ids[base + __popc(mask & ((1u << lane) - 1u))] = env;
 }
 
-// Box sources of the per-vehicle loop. any_hit(p, r, r2, n_obs, want_min,
-// all, m) says whether the sphere of radius r at p touches a box; with
-// want_min, m receives a squared distance that no box is nearer than (see
-// EnvBoxes). all: every box gets the exact test.
+// Box sources of the per-vehicle loop. any_hit(p, r, r2, n_obs, near,
+// all, m) says whether the sphere of radius r at p touches a box; m receives a
+// squared distance that no box is nearer than (see EnvBoxes). all: every box
+// gets the exact test.
 
 // No boxes at all (a fleet without obstacles).
 struct NoBoxSource {
   __device__ __forceinline__ NoBoxSource(const FleetBuffers&, uint32_t) {}
-  __device__ __forceinline__ bool any_hit(V3, float, float, int, bool, bool, float& m) const {
+  __device__ __forceinline__ bool any_hit(V3, float, float, int, float, bool, float& m) const {
     m = __int_as_float(0x7f800000);
     return false;
   }
@@ -110,10 +110,13 @@ struct NoBoxSource {
 
 // The box records of environment env. A test first reads every box's
 // circumscribed sphere, one 16-byte load each, and runs the exact test only on
-// the boxes whose sphere comes within reach:
-//   * r + kBoxSlack when only the decision is wanted (a launch's last step);
-//   * r + kBoxNear when the clearance is wanted too, so that the clearance is
-//     exact up to kBoxNear and at least the distance to the other spheres.
+// the boxes whose sphere comes within r + near. A launch's last test needs the
+// decision only and takes near = kBoxSlack; the others take kBoxNear, or
+// kBoxNearShort in calls of up to kShortCall steps, where a vehicle gets no
+// further, so that the clearance is exact up to near and at least the distance
+// to the other spheres (674,653 quads, 10 boxes, 2 / 6 / 20 steps: 195.9 ->
+// 192.1, 223.5 -> 218.9 and 299.2 -> 294.9 us a pass with the shorter reach;
+// 0.1 m 191.6 / 218.1 / 296.1, 0.05 m 191.4 / 218.5 / 298.2).
 // The sphere's distance is taken low by 3e-4 of the centre distance, which
 // covers the hardware square root and a quaternion whose norm is off by the
 // 1e-4 that ag_set_obstacles admits, and kBoxSlack covers the rest of the
@@ -124,9 +127,10 @@ struct NoBoxSource {
 // U[0.1, 1]) tests about 0.13 boxes per vehicle exactly, so it reads 16 bytes
 // per box and little more instead of 40: a task step of 131,072 environments
 // (RK4 x 4) took 37 us a pass instead of 60, and the bench fleet's 1,000-step
-// call from fresh states 53.8 ms instead of 57.9 (both less since). kBoxNear hardly matters:
-// 0.25 and 1 m measured 53.9 ms.
-constexpr float kBoxSlack = 1e-3f, kBoxNear = 0.5f;
+// call from fresh states 53.8 ms instead of 57.9 (both less since). There
+// kBoxNear hardly matters: 0.25 and 1 m measured 53.9 ms.
+constexpr float kBoxSlack = 1e-3f, kBoxNearShort = 0.2f, kBoxNear = 0.5f;  // m
+constexpr int kShortCall = 32;
 
 // GROUPED: the spheres are loaded in whole groups (8, or 16 while more than 8
 // are left) before any is looked at, so that a group waits for memory once. It
@@ -163,9 +167,9 @@ template <bool GROUPED> struct EnvBoxesT {
       else if (k0 + j < n_obs) exact |= 1u << (bit + j);
     }
   }
-  __device__ __forceinline__ bool any_hit(V3 p, float r, float r2, int n_obs, bool want_min, bool all, float& m) const {
+  __device__ __forceinline__ bool any_hit(V3 p, float r, float r2, int n_obs, float near, bool all, float& m) const {
     const float inf = __int_as_float(0x7f800000);
-    const float reach = all ? inf : r + (want_min ? kBoxNear : kBoxSlack);
+    const float reach = all ? inf : r + near;
     float far = inf, near2 = inf;  // over the spheres out of reach; over the exact tests (squared)
     bool hit = false;
     for (int k0 = 0; k0 < n_obs; k0 += 32) {
@@ -313,7 +317,8 @@ __device__ __forceinline__ VState simulate_cmd(const FleetBuffers& fb, const Ste
       const float moved2 = dot(dp, dp);
       if (n_steps == 1 || (__any_sync(group, !(moved2 < thr2)) && !(moved2 < kJoinTest * thr2))) {
         float min_e2;
-        const bool hit = boxes.any_hit(s.p, r, P.r2, n_obs, step + 1 < n_steps, P.exact_tests != 0, min_e2);
+        const bool hit = boxes.any_hit(s.p, r, P.r2, n_obs, step + 1 == n_steps ? kBoxSlack : n_steps <= kShortCall ? kBoxNearShort : kBoxNear,
+                                       P.exact_tests != 0, min_e2);
         tests += 1;
         p_test = s.p;
         thr2 = P.exact_tests ? -1.f : clearance_threshold2(s.p, min_e2, r);
