@@ -90,10 +90,10 @@ def alu_peak_tflops(info: dict) -> float:
 BYTES_PER_VEHICLE_LAUNCH = 4 * (26 + 8 + 4 + 4) + 1 + 8 + 4 * 160 + 1 + 4
 # DRAM traffic of one full-size fused launch (1,048,576 envs, 1,000 steps):
 # dram__bytes_read.sum + dram__bytes_write.sum from a one-pass ncu capture of
-# exactly this launch (797.11 MB + 68.19 MB). It scales with the fleet size
-# (each env is loaded and stored once per launch; the rare collision tests
-# after the first re-read a few boxes), not with the step count.
-TRAFFIC_BYTES_FULL_LAUNCH = 797.112064e6 + 68.190976e6
+# exactly this launch (413.52 MB + 60.44 MB). It scales with the fleet size
+# (each env is loaded and stored once per launch, of each box its 16-byte
+# sphere and of the few near ones the record), not with the step count.
+TRAFFIC_BYTES_FULL_LAUNCH = 413.523200e6 + 60.444928e6
 # Algorithmic bytes of one reach-task step per quad: read action 16, goal 12,
 # step counter 4, state 52, motors 16, body 16, epoch 4, mode 1 (121 B);
 # written state 52, motors 16, epoch 4, collided flag 1, command 16,
@@ -113,8 +113,8 @@ DEPTH_FLOP_PER_PIXEL, DEPTH_FLOP_PER_CAMERA_BOX, DEPTH_FLOP_PER_PIXEL_BOX = 21.0
 # mode, quadrotor, SIE, one substep, the step's loss term): the forward step
 # and its reverse-mode adjoint (the oracle run with the reverse-counting
 # scalar, every elementary operation's adjoint rule counted). The backward
-# launch's algorithmic work per vehicle-step is one forward recomputation
-# from the checkpoints plus the adjoint.
+# launch's algorithmic work per vehicle-step is the adjoint: the record keeps
+# what it needs of every step.
 FLOP_PER_VEHICLE_STEP_ADJ_FWD = 460.0
 FLOP_PER_VEHICLE_STEP_ADJ_REV = 1217.0
 
@@ -588,10 +588,9 @@ def adjoint_part(seed: int, world: int, alu_peak: float) -> dict:
             "ms_per_rollout": secs * 1e3 / k, **rate_stats(units, [a + b for a, b in zip(fwd_ms, bwd_ms)]),
             "record_ms": fwd_s * 1e3, "backward_ms": bwd_s * 1e3,
             "flop_per_vehicle_step": {"forward": FLOP_PER_VEHICLE_STEP_ADJ_FWD,
-                                      "reverse": FLOP_PER_VEHICLE_STEP_ADJ_FWD + FLOP_PER_VEHICLE_STEP_ADJ_REV},
+                                      "reverse": FLOP_PER_VEHICLE_STEP_ADJ_REV},
             "alu_frac_record": units * FLOP_PER_VEHICLE_STEP_ADJ_FWD / fwd_s / 1e12 / alu_peak,
-            "alu_frac_backward": units * (FLOP_PER_VEHICLE_STEP_ADJ_FWD + FLOP_PER_VEHICLE_STEP_ADJ_REV)
-            / bwd_s / 1e12 / alu_peak,
+            "alu_frac_backward": units * FLOP_PER_VEHICLE_STEP_ADJ_REV / bwd_s / 1e12 / alu_peak,
             "workload": "65,536 quads, position mode, SIE, horizon 256, checkpoint every 32 steps, "
                         "gradients w.r.t. x0 (13/vehicle) and 12 gains"}
 
