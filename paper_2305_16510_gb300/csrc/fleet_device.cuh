@@ -106,9 +106,9 @@ __device__ __forceinline__ float dot(V3 a, V3 b) { return fmaf(a.z, b.z, fmaf(a.
 // 1/x and 1/sqrt(x) by the hardware approximations with subnormal inputs
 // and results flushed to zero (PTX rcp.approx.ftz.f32, rsqrt.approx.ftz.f32).
 // Used only where x is a squared norm in the normal range: that of a
-// unit-scale quaternion, or one checked against 1e-18 or against the
-// smallest normal float (kMinNormal) first; a squared norm below kMinNormal
-// counts as 0.
+// unit-scale quaternion, one summed onto a normal number, or one checked
+// against 1e-18 or against the smallest normal float (kMinNormal) first; a
+// squared norm below kMinNormal counts as 0.
 constexpr float kMinNormal = 1.17549435e-38f;  // 2^-126
 __device__ __forceinline__ float rcp_ftz(float x) {
   float r;

@@ -148,10 +148,14 @@ template <bool GROUPED> struct EnvBoxesT {
     const float4 b = bound[(size_t)k * n], h = rest[2 * (size_t)k * n], q = rest[2 * (size_t)k * n + 1];
     return box_dist2(p, V3{b.x, b.y, b.z}, V3{h.x, h.y, h.z}, Q4{h.w, q.x, q.y, q.z});
   }
-  // The distance from p to the sphere b, low by the margin above.
+  // The distance from p to the sphere b, low by the margin above. The squared
+  // centre distance starts from kTiny, far below what the margins see, so the
+  // hardware root never gets a zero or a subnormal, which it takes for zero
+  // (its infinity would leave out a box around whose centre the vehicle is).
   static __device__ __forceinline__ float low_distance(V3 p, float4 b) {
+    constexpr float kTiny = 1e-37f;
     const V3 v = p - V3{b.x, b.y, b.z};
-    const float d2 = dot(v, v);
+    const float d2 = fmaf(v.z, v.z, fmaf(v.y, v.y, fmaf(v.x, v.x, kTiny)));
     return fmaf(d2 * rsqrt_ftz(d2), 1.f - 3e-4f, -b.w);
   }
   // Spheres k0 .. k0 + G - 1 (the last box again beyond n_obs), bits from bit.

@@ -7,6 +7,8 @@ import pytest
 import torch
 
 from paper_2305_16510_gb300 import workloads as W
+from paper_2305_16510_gb300.fleet import Fleet
+from paper_2305_16510_gb300.task import ReachEnv
 
 from harness import gpu_fleet
 
@@ -65,3 +67,36 @@ def test_obstacles_round_trip_from_host_and_device(n_obs):
     fl.synchronize()
     np.testing.assert_array_equal(host, inp.boxes[:, :, ::-1])
     fl.close()
+
+
+@pytest.mark.parametrize("steps", [1, 3])
+@pytest.mark.parametrize("n_obs", [1, 9])
+def test_vehicle_at_a_box_centre_collides(n_obs, steps, monkeypatch):
+    """Vehicles from 1e-24 to 1e-16 m off a box's centre, where the squared
+    distance is zero, subnormal or the smallest normal numbers: every one is
+    inside the box, in the fused step and in the task step."""
+    offs = np.concatenate([[0.0], np.geomspace(1e-24, 1e-16, 200)]).astype(np.float32)
+    dirs = np.array([[1, 0, 0], [0, -1, 0], [0, 0, 1], [1, 1, 1]], np.float32)
+    p = (dirs[:, :, None] * offs).transpose(1, 0, 2).reshape(3, -1)
+    n = p.shape[1]
+    boxes = np.zeros((n_obs, 10, n), np.float32)
+    boxes[:, 3:6], boxes[:, 6] = 0.1, 1.0
+    boxes[1:, 0] = 30.0                    # only the first box is near
+    st = np.zeros((13, n), np.float32)
+    st[0:3], st[6] = p, 1.0
+    for skip in ("1", "0"):
+        monkeypatch.setenv("AG_FUSED_SKIP", skip)
+        fl = Fleet(n, n_obstacles=n_obs, dt=1e-30, seed=4)   # so short a step that nothing moves
+        fl.set_obstacles(boxes)
+        fl.set_state(st)
+        fl.step(steps)
+        col, ids = fl.events()
+        assert bool(col.all()) and ids.numel() == n
+        fl.close()
+    env = ReachEnv(n, n_obstacles=n_obs, dt=1e-30, seed=4)
+    env.fleet.set_obstacles(boxes)
+    env.reset()
+    env.fleet.set_state(st)
+    *_, info = env.step(torch.zeros((n, 4), device="cuda"))
+    assert bool(info["collided"].all())
+    env.close()
