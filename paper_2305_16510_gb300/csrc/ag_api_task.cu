@@ -31,12 +31,16 @@ ag_status render_depth_impl(ag_ctx* ctx, uint32_t width, uint32_t height, float 
   if (!env_ids && n_cams > n) return fail_invalid(ctx, "n_cams exceeds n_envs");
   if (env_ids && n_cams > n) return fail_invalid(ctx, "at most n_envs cameras per call");
   cudaStream_t st = ctx->stream;
+  const size_t count = (size_t)n_cams * width * height;
   const uint32_t* ids_dev = nullptr;
   if (env_ids) {
     if (!on_device(env_ids))
       for (uint32_t j = 0; j < n_cams; ++j)
         if (env_ids[j] >= n) return fail_invalid(ctx, "environment id out of range");
-    if (on_own_device(ctx, env_ids)) {
+    const uintptr_t ids_at = reinterpret_cast<uintptr_t>(env_ids), image_at = reinterpret_cast<uintptr_t>(depth);
+    const bool overwritten = !live_pairs && ids_at < image_at + count * sizeof(float) &&
+                             image_at < ids_at + n_cams * sizeof(uint32_t);
+    if (on_own_device(ctx, env_ids) && !overwritten) {
       ids_dev = env_ids;  // read in place: a copy first made a launch of few cameras a quarter longer
     } else {
       if (!ctx->cam_ids && (s = alloc_or_oom(ctx, &ctx->cam_ids, n, "the camera ids")) != AG_OK) return s;
@@ -45,7 +49,6 @@ ag_status render_depth_impl(ag_ctx* ctx, uint32_t width, uint32_t height, float 
       ids_dev = ctx->cam_ids;
     }
   }
-  const size_t count = (size_t)n_cams * width * height;
   const bool out_on_device = live_pairs ? true : on_device(depth);
   float* out = depth;
   if (live_pairs && !ctx->live_dev &&

@@ -244,3 +244,24 @@ def test_image_does_not_depend_on_how_many_cameras_a_launch_has(width, height):
         ids = torch.arange(639, 639 - count, -1, dtype=torch.int32, device="cuda")
         assert torch.equal(fl.render_depth(width, height, hfov, 8.0, env_ids=ids), whole[ids.long()])
     fl.close()
+
+
+def test_camera_ids_at_an_odd_address_or_inside_the_images():
+    """Ids that a kernel cannot read in place, or that the images overwrite, are copied first."""
+    w = W.scaled(W.WORKLOADS["obstacles"], 2000)
+    fl = gpu_fleet(w, W.make_inputs(w, 12), 12)
+    fl.reset(None, 12)
+    size, hfov, rng_max = (64, 48), 1.3, 8.0
+    ids = torch.arange(1999, -1, -1, dtype=torch.int32, device="cuda")
+    want = fl.render_depth(*size, hfov, rng_max, env_ids=ids)
+    raw = torch.zeros(4 * ids.numel() + 4, dtype=torch.uint8, device="cuda")
+    raw[2:-2] = ids.view(torch.uint8)
+    got = torch.empty_like(want)
+    _abi.ag_render_depth(fl.ctx, *size, hfov, rng_max, None, raw.data_ptr() + 2, ids.numel(), got)
+    assert torch.equal(got, want)
+    flat = torch.empty_like(want).view(-1)
+    inside = flat[:ids.numel()].view(torch.int32)
+    inside.copy_(ids)
+    _abi.ag_render_depth(fl.ctx, *size, hfov, rng_max, None, inside, ids.numel(), flat)
+    assert torch.equal(flat.view_as(want), want)
+    fl.close()
