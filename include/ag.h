@@ -324,8 +324,9 @@ ag_status ag_set_gains(ag_ctx* ctx, const float* gains12);
  * semi-implicit Euler, one substep per step and no obstacles (else
  * AG_ERR_UNSUPPORTED); AG_ERR_INVALID for n_steps outside 1 .. 2^30, NULL
  * p_goal or loss; AG_ERR_OOM (context still usable, nothing recorded) when the
- * checkpoints do not fit. Does not synchronise. Commands, body parameters and gains must not
- * change until ag_backward has run. */
+ * checkpoints do not fit. Does not synchronise. Command targets, body parameters and gains
+ * must not change until ag_backward has run; the modes may, since the recording
+ * keeps those it ran with. */
 ag_status ag_rollout_loss(ag_ctx* ctx, uint32_t n_steps, float w_pos, float w_omega, const float* p_goal,
                           float* loss, uint8_t* saturated);
 

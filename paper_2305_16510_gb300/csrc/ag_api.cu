@@ -459,6 +459,7 @@ ag_status ag_set_commands(ag_ctx* ctx, const uint8_t* modes, const float* target
   if (s != AG_OK) return s;
   const size_t n = ctx->cfg.n_envs;
   if (modes) {
+    if ((s = keep_recorded_order(ctx)) != AG_OK) return s;
     s = check_cuda(ctx, cudaMemcpyAsync(ctx->fb.modes, modes, n, cudaMemcpyDefault, ctx->stream), "copy modes");
     if (s != AG_OK) return s;
     s = check_cuda(ctx, agk::launch_build_order(ctx->fb, ctx->stream), "build order");

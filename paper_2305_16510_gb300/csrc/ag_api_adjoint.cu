@@ -38,7 +38,7 @@ ag_status ensure_adjoint(ag_ctx* ctx, int n_steps, int K) {
     if (e == cudaSuccess) e = alloc(ctx, &a.grad_gains, 12);
     a.p_goal = pg;
     a.loss_weights = lw;
-    if (e == cudaSuccess) e = alloc(ctx, &a.loss, n);
+    if (e == cudaSuccess) e = alloc(ctx, &a.loss, slots);  // as long as the order: see keep_recorded_order
     if (e != cudaSuccess) {  // nothing half-allocated stays: the next call starts over
       cudaGetLastError();
       void* got[] = {(void*)a.p_goal, a.saturated, (void*)a.loss_weights, a.inv_q0, a.grad_x0, a.grad_gains_env,
@@ -102,6 +102,24 @@ ag_status ensure_adjoint(ag_ctx* ctx, int n_steps, int K) {
 bool overlap(const float* a, size_t na, const float* b, size_t nb) { return a < b + nb && b < a + na; }
 
 }  // namespace
+
+namespace agh {
+
+ag_status keep_recorded_order(ag_ctx* ctx) {
+  agk::AdjointBuffers& a = ctx->adj;
+  if (!ctx->adj_recorded || a.order != ctx->fb.order) return AG_OK;
+  // the copies lie in the staging of the loss and the flags, which nothing reads between a record's end and the next
+  ag_status s = check_cuda(ctx, cudaMemcpyAsync(a.loss, a.order, a.n_slots * sizeof(uint32_t), cudaMemcpyDeviceToDevice,
+                                                ctx->stream), "keep order");
+  if (s == AG_OK)
+    s = check_cuda(ctx, cudaMemcpyAsync(a.saturated, a.modes, a.n, cudaMemcpyDeviceToDevice, ctx->stream), "keep modes");
+  if (s != AG_OK) return s;
+  a.order = reinterpret_cast<const uint32_t*>(a.loss);
+  a.modes = a.saturated;
+  return AG_OK;
+}
+
+}  // namespace agh
 
 extern "C" ag_status ag_set_gains(ag_ctx* ctx, const float* gains12) {
   ag_status s = enter(ctx);

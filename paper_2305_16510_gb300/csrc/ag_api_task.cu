@@ -164,6 +164,7 @@ ag_status ag_reach_begin(ag_ctx* ctx, const ag_reach_config* cfg, const float* g
                       "copy goals")) != AG_OK) return s;
   if ((s = check_cuda(ctx, cudaMemsetAsync(ctx->reach_steps, 0, n * sizeof(uint32_t), st), "clear step counters")) !=
       AG_OK) return s;
+  if ((s = keep_recorded_order(ctx)) != AG_OK) return s;
   if ((s = check_cuda(ctx, cudaMemsetAsync(ctx->fb.modes, (int)cfg->command_mode, n, st), "set modes")) != AG_OK)
     return s;
   if ((s = check_cuda(ctx, agk::launch_build_order(ctx->fb, st), "build order")) != AG_OK)

@@ -64,6 +64,10 @@ bool on_host(const void* p);
 // true for memory of the context's own device, aligned to 4 bytes, which its
 // kernels read and write in place (anything else is copied).
 bool on_own_device(const ag_ctx* ctx, const void* p);
+// Called before the fleet's modes and thread order are overwritten: a recorded
+// rollout whose slots they number keeps copies of both, so that its backward
+// still pairs every slot's tape with the environment that wrote it.
+ag_status keep_recorded_order(ag_ctx* ctx);
 // Rotor allocation matrix A and its pseudo-inverse A^+ in FP64, stored float32.
 void rotor_matrices(int n, double arm, double k_yaw, float A[4][8], float Ap[8][4]);
 // "" for a valid config, else a static message (no allocation).
