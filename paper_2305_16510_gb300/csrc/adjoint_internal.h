@@ -11,6 +11,14 @@ namespace agk {
 // float4 words of one tape entry of one vehicle.
 constexpr int kTapeWords = 4;
 
+// Whether a tape of `entries` entries with `slots` columns keeps a context that
+// holds `other` bytes beside it within `budget` (0 = no limit). 2^30 steps of
+// 2^28 vehicles are more bytes than 64 bits hold, so nothing is multiplied out
+// before it is known to fit.
+inline bool tape_within_budget(uint64_t budget, size_t other, size_t entries, size_t slots) {
+  return budget == 0 || (other <= budget && entries <= (budget - other) / (kTapeWords * slots * sizeof(float4)));
+}
+
 // Device buffers of one recorded rollout and its adjoint. Arrays marked
 // "slot" have n_slots columns, one per thread slot (environment order[slot],
 // none in the padding); the others are indexed by environment. With full_tape the tape holds the entries of every step and the

@@ -64,8 +64,7 @@ ag_status ensure_adjoint(ag_ctx* ctx, int n_steps, int K) {
   };
   const size_t full = (size_t)n_steps + 1;  // one entry per step and the end state
   if (ctx->adj_tape_cap < full) {
-    const uint64_t budget = ctx->cfg.hbm_budget_bytes;
-    if (budget == 0 || ctx->bytes - held + full * entry_bytes <= budget) {
+    if (agk::tape_within_budget(ctx->cfg.hbm_budget_bytes, ctx->bytes - held, full, slots)) {
       free_tape();
       if (alloc(ctx, &a.tape, full * agk::kTapeWords * slots) == cudaSuccess) {
         ctx->adj_tape_cap = full;

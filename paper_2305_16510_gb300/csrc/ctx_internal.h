@@ -74,8 +74,10 @@ void rotor_matrices(int n, double arm, double k_yaw, float A[4][8], float Ap[8][
 const char* validate(const ag_config* c);
 
 // cudaMalloc of count elements, counted against the context's device bytes.
+// A count whose bytes no size_t holds does not fit.
 template <class T> cudaError_t alloc(ag_ctx* ctx, T** p, size_t count) {
   if (count == 0) { *p = nullptr; return cudaSuccess; }
+  if (count > SIZE_MAX / sizeof(T)) return cudaErrorMemoryAllocation;
   cudaError_t e = cudaMalloc((void**)p, count * sizeof(T));
   if (e == cudaSuccess) ctx->bytes += count * sizeof(T);
   return e;
