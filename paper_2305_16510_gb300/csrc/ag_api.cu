@@ -7,6 +7,7 @@
 // per-context sticky error state, the FP64 rotor-allocation matrices, and
 // the stream-ordered copies and launches. Nothing here computes a vehicle
 // state; every step of the simulation runs in the kernels.
+#include <algorithm>
 #include <cmath>
 #include <cstdint>
 #include <cstdio>
@@ -186,11 +187,17 @@ const char* validate(const ag_config* c) {
 
 namespace {
 
+// The staging of boxes from and to memory of another kind: rows of all boxes up
+// to 256 MB, and those of one box where the budget or the device leaves no more.
+size_t box_stage_bytes(const ag_config* c, size_t boxes) {
+  return std::min<size_t>(256u << 20, boxes * 10 * c->n_envs * sizeof(float));
+}
+
 size_t buffer_bytes(const ag_config* c) {
   size_t n = c->n_envs;
   // (the order's padding slots, under 1 % of it plus 1.5 KB, are not counted)
   size_t per = sizeof(float) * (13 + 8 + 4 + 4 + 4) + sizeof(uint32_t) * 4 + 3 /* modes, collided, hits */ + 1;
-  return n * per + agk::box_record_bytes(n, c->n_obstacles) + (c->n_obstacles ? 10 * n * sizeof(float) : 0) +
+  return n * per + agk::box_record_bytes(n, c->n_obstacles) + box_stage_bytes(c, c->n_obstacles ? 1 : 0) +
          sizeof(agk::CallCounts);
 }
 
@@ -363,6 +370,7 @@ ag_status ag_create(const ag_config* cfg, void* cuda_stream, ag_ctx** out) {
   std::memset(&ctx->fb, 0, sizeof(ctx->fb));
   ctx->mask_dev = nullptr;
   ctx->box_stage = nullptr;
+  ctx->box_stage_bytes = 0;
   std::memset(&ctx->adj, 0, sizeof(ctx->adj));
   ctx->adj_ckpt_cap = 0;
   ctx->adj_tape_cap = 0;
@@ -393,7 +401,15 @@ ag_status ag_create(const ag_config* cfg, void* cuda_stream, ag_ctx** out) {
   if (e == cudaSuccess) e = alloc(ctx, &f.targets, 4 * n);
   if (e == cudaSuccess) e = alloc(ctx, &f.box_bound, (size_t)cfg->n_obstacles * n);
   if (e == cudaSuccess) e = alloc(ctx, &f.box_rest, (size_t)cfg->n_obstacles * n * 2);
-  if (e == cudaSuccess && cfg->n_obstacles) e = alloc(ctx, &ctx->box_stage, 10 * n);
+  const size_t stage_least = box_stage_bytes(cfg, cfg->n_obstacles ? 1 : 0);
+  ctx->box_stage_bytes = box_stage_bytes(cfg, cfg->n_obstacles);
+  if (cfg->hbm_budget_bytes)
+    ctx->box_stage_bytes = std::min<uint64_t>(ctx->box_stage_bytes, cfg->hbm_budget_bytes - buffer_bytes(cfg) + stage_least);
+  if (e == cudaSuccess && alloc(ctx, &ctx->box_stage, ctx->box_stage_bytes / sizeof(float)) != cudaSuccess) {
+    cudaGetLastError();
+    ctx->box_stage_bytes = stage_least;
+    e = alloc(ctx, &ctx->box_stage, stage_least / sizeof(float));
+  }
   if (e == cudaSuccess) e = alloc(ctx, &f.epoch, n);
   if (e == cudaSuccess) e = alloc(ctx, &f.collided, n);
   if (e == cudaSuccess) e = alloc(ctx, &f.reset_ids, n);
@@ -497,32 +513,20 @@ ag_status ag_set_obstacles(ag_ctx* ctx, const float* boxes) {
   if (bad) return fail_invalid(ctx, "boxes: finite centres, half-extents > 0 and unit quaternions required");
   cudaStream_t st = ctx->stream;
   if (on_own_device(ctx, boxes))
-    return check_cuda(ctx, agk::launch_pack_boxes(ctx->fb, boxes, n, 0, n_obs, st), "pack boxes");
-  for (uint32_t k = 0; k < n_obs; ++k) {  // box by box through the staging rows
-    if ((s = check_cuda(ctx, cudaMemcpyAsync(ctx->box_stage, boxes + (size_t)k * 10 * n, 10 * (size_t)n * sizeof(float),
-                                             cudaMemcpyDefault, st), "copy boxes")) != AG_OK) return s;
-    if ((s = check_cuda(ctx, agk::launch_pack_boxes(ctx->fb, ctx->box_stage, n, k, 1, st), "pack boxes")) != AG_OK)
-      return s;
-  }
-  return AG_OK;
+    return check_cuda(ctx, agk::launch_pack_boxes(ctx->fb, boxes, st), "pack boxes");
+  return check_cuda(ctx, agk::upload_boxes(ctx->fb, boxes, n, ctx->box_stage, ctx->box_stage_bytes, st), "copy boxes");
 }
 
 ag_status ag_get_obstacles(ag_ctx* ctx, float* boxes) {
   ag_status s = enter(ctx);
   if (s != AG_OK) return s;
   if (!boxes) return fail_invalid(ctx, "boxes is NULL");
-  const uint32_t n = ctx->cfg.n_envs, n_obs = ctx->cfg.n_obstacles;
-  if (n_obs == 0) return AG_OK;
+  if (ctx->cfg.n_obstacles == 0) return AG_OK;
   cudaStream_t st = ctx->stream;
   if (on_own_device(ctx, boxes))
-    return check_cuda(ctx, agk::launch_unpack_boxes(ctx->fb, boxes, 0, n_obs, st), "unpack boxes");
-  for (uint32_t k = 0; k < n_obs; ++k) {
-    if ((s = check_cuda(ctx, agk::launch_unpack_boxes(ctx->fb, ctx->box_stage, k, 1, st), "unpack boxes")) != AG_OK)
-      return s;
-    if ((s = check_cuda(ctx, cudaMemcpyAsync(boxes + (size_t)k * 10 * n, ctx->box_stage, 10 * (size_t)n * sizeof(float),
-                                             cudaMemcpyDefault, st), "copy boxes out")) != AG_OK) return s;
-  }
-  return AG_OK;
+    return check_cuda(ctx, agk::launch_unpack_boxes(ctx->fb, boxes, st), "unpack boxes");
+  return check_cuda(ctx, agk::download_boxes(ctx->fb, boxes, ctx->box_stage, ctx->box_stage_bytes, st),
+                    "copy boxes out");
 }
 
 ag_status ag_set_obstacle_randomization(ag_ctx* ctx, const float env_min[3], const float env_max[3],

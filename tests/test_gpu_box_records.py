@@ -100,3 +100,23 @@ def test_vehicle_at_a_box_centre_collides(n_obs, steps, monkeypatch):
     *_, info = env.step(torch.zeros((n, 4), device="cuda"))
     assert bool(info["collided"].all())
     env.close()
+
+
+@pytest.mark.parametrize("n,n_obs,budget", [(1001, 5, 0), (6_800_001, 1, 0), (1000, 5, 475_000)])
+def test_obstacles_from_host_memory_in_several_parts(n, n_obs, budget):
+    """All boxes at once; more rows of one box than the staging holds (256 MB);
+    two boxes at a time, which is what the budget leaves."""
+    from paper_2305_16510_gb300 import _abi
+    rng = np.random.default_rng(n)
+    boxes = rng.uniform(0.1, 5.0, (n_obs, 10, n)).astype(np.float32)
+    boxes[:, 6:10] = 0.5
+    fl = Fleet(n, n_obstacles=n_obs, hbm_budget_bytes=budget)
+    for memory in (boxes, torch.from_numpy(boxes).pin_memory()):
+        fl.set_obstacles(np.full((n_obs, 10, n), 0.5, np.float32))
+        _abi.ag_set_obstacles(fl.ctx, memory)
+        np.testing.assert_array_equal(fl.obstacles().cpu().numpy(), boxes)
+        host = np.zeros_like(boxes)
+        _abi.ag_get_obstacles(fl.ctx, host)
+        fl.synchronize()
+        np.testing.assert_array_equal(host, boxes)
+    fl.close()

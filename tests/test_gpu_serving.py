@@ -201,3 +201,23 @@ def test_request_inputs_in_host_memory_give_the_same_results(n, n_obs, with_body
     np.testing.assert_array_equal(a[0], b[0])
     np.testing.assert_array_equal(a[1], b[1])
     assert np.isfinite(a[0]).all() and (a[1] >= 1).all()
+
+
+@pytest.mark.parametrize("n,n_obs", [(150_001, 12), (1_700_001, 1)])
+def test_request_boxes_from_host_memory_in_several_parts(n, n_obs):
+    """More rows than the server stages at once (64 MiB): some boxes at a time,
+    and part of one box at a time, give what boxes in device memory give."""
+    from paper_2305_16510_gb300.serving import RequestPool
+    w = W.Workload("parts", n, 4, 1, n_obs, n, 0, 0, mode_mix=(0, 1, 2))
+    inp = W.make_inputs(w, 16)
+    boxes = np.ascontiguousarray(inp.boxes.reshape(-1, n))
+    pool = RequestPool(inp.modes, inp.targets, boxes)
+    host = _abi.ag_request()
+    host.n_envs, host.n_steps, host.n_obstacles, host.seed, host.pitch = n, 3, n_obs, 9, n
+    host.modes, host.targets, host.boxes = inp.modes.ctypes.data, inp.targets.ctypes.data, boxes.ctypes.data
+    with _server(max_active=4, chunk_steps=25, hbm_budget_bytes=2 << 30) as s:
+        a = s.wait(s.submit(pool.request(n_envs=n, n_steps=3, n_obstacles=n_obs, seed=9)))
+        b = s.wait(s.submit(host))
+    np.testing.assert_array_equal(a[0], b[0])
+    np.testing.assert_array_equal(a[1], b[1])
+    assert (a[1] > 1).any()          # the boxes were met
