@@ -195,10 +195,10 @@ size_t box_stage_bytes(const ag_config* c, size_t boxes) {
 
 size_t buffer_bytes(const ag_config* c) {
   size_t n = c->n_envs;
-  // (the order's padding slots, under 1 % of it plus 1.5 KB, are not counted)
-  size_t per = sizeof(float) * (13 + 8 + 4 + 4 + 4) + sizeof(uint32_t) * 4 + 3 /* modes, collided, hits */ + 1;
-  return n * per + agk::box_record_bytes(n, c->n_obstacles) + box_stage_bytes(c, c->n_obstacles ? 1 : 0) +
-         sizeof(agk::CallCounts);
+  size_t per = sizeof(float) * (13 + 8 + 4 + 4 + 4) + sizeof(uint32_t) * 3 + 3 /* modes, collided, hits */ + 1;
+  const size_t slots = agk::OrderLayout{c->n_envs, c->n_quad, c->n_hexa}.total();
+  return n * per + slots * sizeof(uint32_t) + agk::box_record_bytes(n, c->n_obstacles) +
+         box_stage_bytes(c, c->n_obstacles ? 1 : 0) + sizeof(agk::CallCounts) + sizeof(uint32_t) /* check_dev */;
 }
 
 }  // namespace

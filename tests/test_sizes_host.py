@@ -3,7 +3,9 @@ interface admits may exceed 64 bits, and must then be refused, not wrapped to a
 small allocation that the kernels would write past."""
 import subprocess
 
-from paper_2305_16510_gb300 import build
+import pytest
+
+from paper_2305_16510_gb300 import _abi, build
 
 PROGRAM = r"""
 #include <cstdint>
@@ -50,3 +52,36 @@ def test_sizes_beyond_64_bits_do_not_fit(tmp_path):
     assert r.returncode == 0, r.stderr
     r = subprocess.run([str(exe)], capture_output=True, text=True)
     assert (r.returncode, r.stdout.strip()) == (0, "0")
+
+
+def _order_slots(n, n_quad, n_hexa):
+    """Slots of the grouping order: windows of 16,384 environments, each with
+    room for four runs per rotor type in it, rounded up to 32 slots each."""
+    total, octo = 0, n_quad + n_hexa
+    for lo in range(0, n, 16384):
+        hi = min(lo + 16384, n)
+        types = (lo < n_quad) + (max(lo, n_quad) < min(hi, octo)) + (max(lo, octo) < hi)
+        total += (hi - lo + 31 * 4 * types) // 32 * 32
+    return total
+
+
+@pytest.mark.parametrize("n_obs", [0, 1, 7])
+@pytest.mark.parametrize("n,n_hexa,n_octo", [(1, 0, 0), (1000, 0, 0), (1000, 300, 200), (16385, 0, 1), (100_000, 33_000, 1)])
+def test_budget_counts_everything_a_context_allocates(n, n_hexa, n_octo, n_obs):
+    """state 13, motors 8, body, targets and the wrench scratch 4 rows each;
+    epoch, reset ids and reset counts; modes, collided, hits and mask bytes;
+    the order with its padding; box records and one box's staging; two
+    counters and the check counter."""
+    c = _abi.ag_config_default()
+    c.n_envs, c.n_quad, c.n_hexa, c.n_octo, c.n_obstacles = n, n - n_hexa - n_octo, n_hexa, n_octo, n_obs
+    need = (n * (33 * 4 + 3 * 4 + 4) + 4 * _order_slots(n, c.n_quad, n_hexa) + n * n_obs * 48 +
+            (40 * n if n_obs else 0) + 16 + 4)
+    c.hbm_budget_bytes = need - 1
+    with pytest.raises(_abi.AgError) as e:
+        _abi.ag_create(c)
+    assert e.value.status == _abi.AG_ERR_OOM and str(need) in str(e.value)
+    c.hbm_budget_bytes = need            # enough: what comes next is the device
+    try:
+        _abi.ag_destroy(_abi.ag_create(c))
+    except _abi.AgError as err:
+        assert err.status == _abi.AG_ERR_CUDA
