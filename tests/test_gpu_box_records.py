@@ -10,7 +10,7 @@ from paper_2305_16510_gb300 import workloads as W
 from paper_2305_16510_gb300.fleet import Fleet
 from paper_2305_16510_gb300.task import ReachEnv
 
-from harness import gpu_fleet
+from harness import box_margin, gpu_fleet
 
 pytestmark = pytest.mark.gpu
 
@@ -120,3 +120,35 @@ def test_obstacles_from_host_memory_in_several_parts(n, n_obs, budget):
         fl.synchronize()
         np.testing.assert_array_equal(host, boxes)
     fl.close()
+
+
+@pytest.mark.parametrize("steps", [1, 2])
+@pytest.mark.parametrize("n_obs", [1, 2, 3, 4, 5, 7, 33, 64])
+def test_decisions_among_walls_and_small_boxes(n_obs, steps):
+    """Calls of one step have a kernel of their own, which tests marked boxes four
+    at a time. Walls, whose spheres mark every box, and small boxes: with so
+    short a step that nothing moves, the flags are those of the float64 distances,
+    but for near ties (the squared distances are good to 1e-5 m^2)."""
+    n = 4000
+    rng = np.random.default_rng(n_obs)
+    boxes = np.zeros((n_obs, 10, n), np.float32)
+    boxes[:, 0:3] = rng.uniform(-3, 3, (n_obs, 3, n))
+    boxes[:, 3:6] = rng.choice([0.05, 0.1, 0.2], (n_obs, 3, n))
+    boxes[::2, 3:6] = np.array([4.0, 0.05, 4.0], np.float32)[None, :, None] / np.sqrt(n_obs)
+    q = rng.normal(size=(n_obs, 4, n))
+    boxes[:, 6:10] = q / np.linalg.norm(q, axis=1, keepdims=True)
+    st = np.zeros((13, n), np.float32)
+    st[0:3], st[6] = rng.uniform(-3, 3, (3, n)), 1.0
+    fl = Fleet(n, n_obstacles=n_obs, n_hexa=1300, n_octo=1300, dt=1e-30, seed=4)
+    fl.set_obstacles(boxes)
+    fl.set_state(st)
+    fl.step(steps)
+    hit = fl.events()[0].cpu().numpy() != 0
+    fl.close()
+    margin = box_margin(st[0:3].astype(np.float64), boxes.astype(np.float64), 0.2)
+    sure = np.abs(margin) > 1e-4
+    if steps == 1:
+        np.testing.assert_array_equal(hit[sure], margin[sure] <= 0)
+    else:                            # the second step tests the re-drawn vehicles too
+        assert hit[sure & (margin <= 0)].all() and not hit[sure & (margin > 0)].any()
+    assert sure.mean() > 0.99 and 20 < hit.sum() < n
