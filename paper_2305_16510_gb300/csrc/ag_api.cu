@@ -187,18 +187,12 @@ const char* validate(const ag_config* c) {
 
 namespace {
 
-// The staging of boxes from and to memory of another kind: rows of all boxes up
-// to 256 MB, and those of one box where the budget or the device leaves no more.
-size_t box_stage_bytes(const ag_config* c, size_t boxes) {
-  return std::min<size_t>(256u << 20, boxes * 10 * c->n_envs * sizeof(float));
-}
-
 size_t buffer_bytes(const ag_config* c) {
   size_t n = c->n_envs;
   size_t per = sizeof(float) * (13 + 8 + 4 + 4 + 4) + sizeof(uint32_t) * 3 + 3 /* modes, collided, hits */ + 1;
   const size_t slots = agk::OrderLayout{c->n_envs, c->n_quad, c->n_hexa}.total();
   return n * per + slots * sizeof(uint32_t) + agk::box_record_bytes(n, c->n_obstacles) +
-         box_stage_bytes(c, c->n_obstacles ? 1 : 0) + sizeof(agk::CallCounts) + sizeof(uint32_t) /* check_dev */;
+         (c->n_obstacles ? 10 * n * sizeof(float) : 0) + sizeof(agk::CallCounts) + sizeof(uint32_t) /* check_dev */;
 }
 
 }  // namespace
@@ -303,7 +297,7 @@ void free_all(ag_ctx* ctx) {
   agk::FleetBuffers& f = ctx->fb;
   void* ptrs[] = {f.state, f.motors, f.body, f.modes, f.targets, f.box_bound, f.box_rest, f.epoch, f.collided, f.reset_ids,
                   f.counts, f.cmd, f.resets, f.hits, f.order, ctx->mask_dev,
-                  ctx->box_stage, (void*)f.box_rand};
+                  ctx->box_stage, ctx->box_stage_all.rows, (void*)f.box_rand};
   for (void* p : ptrs)
     if (p) cudaFree(p);
 }
@@ -370,7 +364,8 @@ ag_status ag_create(const ag_config* cfg, void* cuda_stream, ag_ctx** out) {
   std::memset(&ctx->fb, 0, sizeof(ctx->fb));
   ctx->mask_dev = nullptr;
   ctx->box_stage = nullptr;
-  ctx->box_stage_bytes = 0;
+  ctx->box_stage_all = agk::BoxStage{nullptr, 0};
+  ctx->box_stage_tried = false;
   std::memset(&ctx->adj, 0, sizeof(ctx->adj));
   ctx->adj_ckpt_cap = 0;
   ctx->adj_tape_cap = 0;
@@ -401,15 +396,7 @@ ag_status ag_create(const ag_config* cfg, void* cuda_stream, ag_ctx** out) {
   if (e == cudaSuccess) e = alloc(ctx, &f.targets, 4 * n);
   if (e == cudaSuccess) e = alloc(ctx, &f.box_bound, (size_t)cfg->n_obstacles * n);
   if (e == cudaSuccess) e = alloc(ctx, &f.box_rest, (size_t)cfg->n_obstacles * n * 2);
-  const size_t stage_least = box_stage_bytes(cfg, cfg->n_obstacles ? 1 : 0);
-  ctx->box_stage_bytes = box_stage_bytes(cfg, cfg->n_obstacles);
-  if (cfg->hbm_budget_bytes)
-    ctx->box_stage_bytes = std::min<uint64_t>(ctx->box_stage_bytes, cfg->hbm_budget_bytes - buffer_bytes(cfg) + stage_least);
-  if (e == cudaSuccess && alloc(ctx, &ctx->box_stage, ctx->box_stage_bytes / sizeof(float)) != cudaSuccess) {
-    cudaGetLastError();
-    ctx->box_stage_bytes = stage_least;
-    e = alloc(ctx, &ctx->box_stage, stage_least / sizeof(float));
-  }
+  if (e == cudaSuccess && cfg->n_obstacles) e = alloc(ctx, &ctx->box_stage, 10 * n);
   if (e == cudaSuccess) e = alloc(ctx, &f.epoch, n);
   if (e == cudaSuccess) e = alloc(ctx, &f.collided, n);
   if (e == cudaSuccess) e = alloc(ctx, &f.reset_ids, n);
@@ -487,6 +474,22 @@ ag_status ag_set_commands(ag_ctx* ctx, const uint8_t* modes, const float* target
   return s;
 }
 
+// The stage of a transfer of all boxes: rows of all of them up to 256 MB, made at
+// the first such call where the device and the budget have room, else the one
+// box's rows that every context among boxes holds.
+static agk::BoxStage box_stage(ag_ctx* ctx) {
+  const size_t one = 10 * (size_t)ctx->cfg.n_envs * sizeof(float);
+  if (!ctx->box_stage_all.rows && !ctx->box_stage_tried) {
+    ctx->box_stage_tried = true;
+    const uint64_t budget = ctx->cfg.hbm_budget_bytes;
+    size_t bytes = std::min<size_t>(256u << 20, ctx->cfg.n_obstacles * one);
+    if (budget) bytes = std::min<uint64_t>(bytes, budget > ctx->bytes ? budget - ctx->bytes : 0);
+    if (bytes >= 2 * one) ctx->box_stage_all = {agk::alloc_box_stage(bytes), bytes};
+    if (ctx->box_stage_all.rows) ctx->bytes += bytes;
+  }
+  return ctx->box_stage_all.rows ? ctx->box_stage_all : agk::BoxStage{ctx->box_stage, one};
+}
+
 ag_status ag_set_obstacles(ag_ctx* ctx, const float* boxes) {
   agk::NvtxRange range("ag_set_obstacles");
   ag_status s = enter(ctx);
@@ -513,20 +516,20 @@ ag_status ag_set_obstacles(ag_ctx* ctx, const float* boxes) {
   if (bad) return fail_invalid(ctx, "boxes: finite centres, half-extents > 0 and unit quaternions required");
   cudaStream_t st = ctx->stream;
   if (on_own_device(ctx, boxes))
-    return check_cuda(ctx, agk::launch_pack_boxes(ctx->fb, boxes, st), "pack boxes");
-  return check_cuda(ctx, agk::upload_boxes(ctx->fb, boxes, n, ctx->box_stage, ctx->box_stage_bytes, st), "copy boxes");
+    return check_cuda(ctx, agk::launch_pack_boxes(ctx->fb, boxes, n, 0, n_obs, st), "pack boxes");
+  return check_cuda(ctx, agk::upload_boxes(ctx->fb, boxes, n, box_stage(ctx), st), "copy boxes");
 }
 
 ag_status ag_get_obstacles(ag_ctx* ctx, float* boxes) {
   ag_status s = enter(ctx);
   if (s != AG_OK) return s;
   if (!boxes) return fail_invalid(ctx, "boxes is NULL");
-  if (ctx->cfg.n_obstacles == 0) return AG_OK;
+  const uint32_t n_obs = ctx->cfg.n_obstacles;
+  if (n_obs == 0) return AG_OK;
   cudaStream_t st = ctx->stream;
   if (on_own_device(ctx, boxes))
-    return check_cuda(ctx, agk::launch_unpack_boxes(ctx->fb, boxes, st), "unpack boxes");
-  return check_cuda(ctx, agk::download_boxes(ctx->fb, boxes, ctx->box_stage, ctx->box_stage_bytes, st),
-                    "copy boxes out");
+    return check_cuda(ctx, agk::launch_unpack_boxes(ctx->fb, boxes, 0, n_obs, st), "unpack boxes");
+  return check_cuda(ctx, agk::download_boxes(ctx->fb, boxes, box_stage(ctx), st), "copy boxes out");
 }
 
 ag_status ag_set_obstacle_randomization(ag_ctx* ctx, const float env_min[3], const float env_max[3],

@@ -19,8 +19,9 @@ struct ag_ctx {
   int device;
   agk::FleetBuffers fb;
   uint8_t* mask_dev;         // [n] staging for ag_reset masks
-  float* box_stage;          // rows of boxes on their way to or from memory of another kind (NULL without boxes)
-  size_t box_stage_bytes;
+  float* box_stage;          // [10][n] one box's rows on their way to or from memory of another kind (NULL without boxes)
+  agk::BoxStage box_stage_all;  // several boxes' rows, made at the first transfer that wants them
+  bool box_stage_tried;
   uint64_t seed;             // Philox key of collision resets
   bool failed;
   std::string err;

@@ -106,18 +106,33 @@ cudaError_t launch_plain_step(const FleetBuffers& fb, const StepParams& P, int i
 // Builds fb.order from the current modes and rotor types (one launch).
 cudaError_t launch_build_order(const FleetBuffers& fb, cudaStream_t st);
 
-// Box records from an array of device memory in the layout of
-// ag_set_obstacles (row f of box j at src[(j * 10 + f) * n + env]), and back.
-cudaError_t launch_pack_boxes(const FleetBuffers& fb, const float* src, cudaStream_t st);
-cudaError_t launch_unpack_boxes(const FleetBuffers& fb, float* dst, cudaStream_t st);
-// The same from and to any other memory, through `stage` in device memory, as
-// many boxes at a time as it holds (rows of `pitch` elements; download: n). With
-// one box at a time, 64 boxes of 1,000 environments take 864 us to read and 690
-// to set, together 30 and 354; the eight requests of a batch with 16 boxes from
-// host memory 3,047 us against 1,235.
-cudaError_t upload_boxes(const FleetBuffers& fb, const float* boxes, size_t pitch, float* stage, size_t stage_bytes,
-                         cudaStream_t st);
-cudaError_t download_boxes(const FleetBuffers& fb, float* boxes, float* stage, size_t stage_bytes, cudaStream_t st);
+// Box records of boxes k0 .. k0 + count - 1 from the layout of ag_set_obstacles
+// (row f of box k0 + j at src[(j * 10 + f) * pitch + env]), and back (pitch n).
+cudaError_t launch_pack_boxes(const FleetBuffers& fb, const float* src, size_t pitch, uint32_t k0, uint32_t count,
+                              cudaStream_t st);
+cudaError_t launch_unpack_boxes(const FleetBuffers& fb, float* dst, uint32_t k0, uint32_t count, cudaStream_t st);
+
+// Device memory for rows of boxes on their way to or from memory that a kernel
+// does not reach in place: at least one box's rows, better all of them.
+struct BoxStage {
+  float* rows;
+  size_t bytes;
+  uint32_t boxes(uint32_t n) const {
+    const size_t fit = bytes / (10 * sizeof(float) * n);
+    return fit < 1 ? 1u : fit > 64 ? 64u : (uint32_t)fit;
+  }
+};
+// All boxes of fb from any memory (rows of `pitch` elements), and to any memory
+// (pitch n), as many at a time as the stage holds. One at a time, 64 boxes of
+// 1,000 environments take 864 us to read and 690 to set, together 30 and 354; the
+// eight requests of a batch with 16 boxes from host memory 3,047 us against 1,235.
+cudaError_t upload_boxes(const FleetBuffers& fb, const float* boxes, size_t pitch, const BoxStage& stage, cudaStream_t st);
+cudaError_t download_boxes(const FleetBuffers& fb, float* boxes, const BoxStage& stage, cudaStream_t st);
+// A stage of several boxes, made when the first transfer wants it (cudaMalloc of
+// 160 MB takes 0.5 ms, which a program that sets its boxes from device memory does
+// not pay); NULL if the device has no room for it.
+float* alloc_box_stage(size_t bytes);
+
 // Bytes of the box records of n envs with n_obs boxes each.
 inline size_t box_record_bytes(size_t n, size_t n_obs) { return n * n_obs * 3 * sizeof(float4); }
 

@@ -154,26 +154,25 @@ __global__ void __launch_bounds__(kOrderThreads) k_order_window(FleetBuffers fb)
   }
 }
 
-// Box records of environments env0 .. env0 + count - 1 from the caller's rows and back: thread (env, box).
+// Box records k0 .. from the caller's rows and back: thread (env, box).
 __global__ void __launch_bounds__(256) k_pack_boxes(FleetBuffers fb, const float* __restrict__ src, size_t pitch,
-                                                    uint32_t k0, uint32_t env0, uint32_t count) {
-  const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= count) return;
+                                                    uint32_t k0) {
+  const uint32_t env = blockIdx.x * blockDim.x + threadIdx.x;
+  if (env >= fb.n) return;
   float v[10];
 #pragma unroll
-  for (int f = 0; f < 10; ++f) v[f] = src[((size_t)blockIdx.y * 10 + f) * pitch + i];
-  pack_box(fb, k0 + blockIdx.y, env0 + i, v);
+  for (int f = 0; f < 10; ++f) v[f] = src[((size_t)blockIdx.y * 10 + f) * pitch + env];
+  pack_box(fb, k0 + blockIdx.y, env, v);
 }
 
-__global__ void __launch_bounds__(256) k_unpack_boxes(FleetBuffers fb, float* __restrict__ dst, size_t pitch,
-                                                      uint32_t k0, uint32_t env0, uint32_t count) {
-  const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= count) return;
-  const size_t at = (size_t)(k0 + blockIdx.y) * fb.n + env0 + i;
+__global__ void __launch_bounds__(256) k_unpack_boxes(FleetBuffers fb, float* __restrict__ dst, uint32_t k0) {
+  const uint32_t env = blockIdx.x * blockDim.x + threadIdx.x;
+  if (env >= fb.n) return;
+  const size_t at = (size_t)(k0 + blockIdx.y) * fb.n + env;
   const float4 b = fb.box_bound[at], h = fb.box_rest[2 * at], q = fb.box_rest[2 * at + 1];
   const float v[10] = {b.x, b.y, b.z, h.x, h.y, h.z, h.w, q.x, q.y, q.z};
 #pragma unroll
-  for (int f = 0; f < 10; ++f) dst[((size_t)blockIdx.y * 10 + f) * pitch + i] = v[f];
+  for (int f = 0; f < 10; ++f) dst[((size_t)blockIdx.y * 10 + f) * fb.n + env] = v[f];
 }
 
 // ag_reset: resample masked environments, clear collided flags, list them.
@@ -357,60 +356,55 @@ cudaError_t launch_build_order(const FleetBuffers& fb, cudaStream_t st) {
   return cudaGetLastError();
 }
 
-cudaError_t launch_pack_boxes(const FleetBuffers& fb, const float* src, cudaStream_t st) {
-  k_pack_boxes<<<dim3((fb.n + 255) / 256, fb.n_obs), 256, 0, st>>>(fb, src, fb.n, 0, 0, fb.n);
+cudaError_t launch_pack_boxes(const FleetBuffers& fb, const float* src, size_t pitch, uint32_t k0, uint32_t count,
+                              cudaStream_t st) {
+  k_pack_boxes<<<dim3((fb.n + 255) / 256, count), 256, 0, st>>>(fb, src, pitch, k0);
   return cudaGetLastError();
 }
 
-cudaError_t launch_unpack_boxes(const FleetBuffers& fb, float* dst, cudaStream_t st) {
-  k_unpack_boxes<<<dim3((fb.n + 255) / 256, fb.n_obs), 256, 0, st>>>(fb, dst, fb.n, 0, 0, fb.n);
+cudaError_t launch_unpack_boxes(const FleetBuffers& fb, float* dst, uint32_t k0, uint32_t count, cudaStream_t st) {
+  k_unpack_boxes<<<dim3((fb.n + 255) / 256, count), 256, 0, st>>>(fb, dst, k0);
   return cudaGetLastError();
 }
 
-namespace {
-
-// Calls part(k0, boxes, env0, envs) over the largest parts whose rows fit the
-// stage: several boxes of all environments, else a range of environments of one.
-template <class F> cudaError_t each_box_part(const FleetBuffers& fb, size_t stage_bytes, const F& part) {
-  const size_t columns = stage_bytes / (10 * sizeof(float));  // of one box
-  if (columns == 0) return cudaErrorInvalidValue;
-  const uint32_t envs = (uint32_t)std::min<size_t>(fb.n, columns);
-  const uint32_t boxes = (uint32_t)std::min<size_t>(fb.n_obs, columns / envs);
-  cudaError_t e = cudaSuccess;
-  for (uint32_t k = 0; k < fb.n_obs; k += boxes)
-    for (uint32_t i = 0; i < fb.n && e == cudaSuccess; i += envs)
-      e = part(k, std::min(boxes, fb.n_obs - k), i, std::min(envs, fb.n - i));
-  return e;
-}
-
-// `rows` rows of `width` floats, in one piece where neither side has a gap between them.
-cudaError_t copy_rows(float* dst, size_t dst_pitch, const float* src, size_t src_pitch, size_t width, size_t rows,
-                      cudaStream_t st) {
-  if (dst_pitch == width && src_pitch == width)
-    return cudaMemcpyAsync(dst, src, width * rows * sizeof(float), cudaMemcpyDefault, st);
-  return cudaMemcpy2DAsync(dst, dst_pitch * sizeof(float), src, src_pitch * sizeof(float), width * sizeof(float), rows,
-                           cudaMemcpyDefault, st);
-}
-
-}  // namespace
-
-cudaError_t upload_boxes(const FleetBuffers& fb, const float* boxes, size_t pitch, float* stage, size_t stage_bytes,
-                         cudaStream_t st) {
-  return each_box_part(fb, stage_bytes, [&](uint32_t k0, uint32_t count, uint32_t env0, uint32_t envs) {
-    cudaError_t e = copy_rows(stage, envs, boxes + (size_t)k0 * 10 * pitch + env0, pitch, envs, (size_t)count * 10, st);
+cudaError_t upload_boxes(const FleetBuffers& fb, const float* boxes, size_t pitch, const BoxStage& stage, cudaStream_t st) {
+  const uint32_t most = stage.boxes(fb.n);
+  for (uint32_t k = 0; k < fb.n_obs; k += most) {
+    const uint32_t count = std::min(most, fb.n_obs - k);
+    const float* src = boxes + (size_t)k * 10 * pitch;
+    cudaError_t e = pitch == fb.n ? cudaMemcpyAsync(stage.rows, src, (size_t)count * 10 * fb.n * sizeof(float),
+                                                    cudaMemcpyDefault, st)
+                                  : cudaMemcpy2DAsync(stage.rows, fb.n * sizeof(float), src, pitch * sizeof(float),
+                                                      fb.n * sizeof(float), (size_t)count * 10, cudaMemcpyDefault, st);
+    if (e == cudaSuccess) e = launch_pack_boxes(fb, stage.rows, fb.n, k, count, st);
     if (e != cudaSuccess) return e;
-    k_pack_boxes<<<dim3((envs + 255) / 256, count), 256, 0, st>>>(fb, stage, envs, k0, env0, envs);
-    return cudaGetLastError();
-  });
+  }
+  return cudaSuccess;
 }
 
-cudaError_t download_boxes(const FleetBuffers& fb, float* boxes, float* stage, size_t stage_bytes, cudaStream_t st) {
-  return each_box_part(fb, stage_bytes, [&](uint32_t k0, uint32_t count, uint32_t env0, uint32_t envs) {
-    k_unpack_boxes<<<dim3((envs + 255) / 256, count), 256, 0, st>>>(fb, stage, envs, k0, env0, envs);
-    cudaError_t e = cudaGetLastError();
+cudaError_t download_boxes(const FleetBuffers& fb, float* boxes, const BoxStage& stage, cudaStream_t st) {
+  const uint32_t most = stage.boxes(fb.n);
+  for (uint32_t k = 0; k < fb.n_obs; k += most) {
+    const uint32_t count = std::min(most, fb.n_obs - k);
+    cudaError_t e = launch_unpack_boxes(fb, stage.rows, k, count, st);
+    if (e == cudaSuccess)
+      e = cudaMemcpyAsync(boxes + (size_t)k * 10 * fb.n, stage.rows, (size_t)count * 10 * fb.n * sizeof(float),
+                          cudaMemcpyDefault, st);
     if (e != cudaSuccess) return e;
-    return copy_rows(boxes + (size_t)k0 * 10 * fb.n + env0, fb.n, stage, envs, envs, (size_t)count * 10, st);
-  });
+  }
+  return cudaSuccess;
+}
+
+float* alloc_box_stage(size_t bytes) {
+  cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;  // an allocation is no part of a capture
+  cudaThreadExchangeStreamCaptureMode(&mode);
+  float* p = nullptr;
+  if (cudaMalloc((void**)&p, bytes) != cudaSuccess) {
+    cudaGetLastError();
+    p = nullptr;
+  }
+  cudaThreadExchangeStreamCaptureMode(&mode);
+  return p;
 }
 
 cudaError_t launch_reset(const FleetBuffers& fb, const uint8_t* mask, uint32_t seed_lo, uint32_t seed_hi,

@@ -167,12 +167,12 @@ size_t align256(size_t b) { return (b + 255) & ~size_t(255); }
 
 // Device bytes one request needs (state, motors, body, targets, modes, epoch,
 // collided, reset count, order (its first use is as the initial reset's id
-// list) and box records).
+// list), box records and the staging of one box's rows).
 size_t request_bytes(size_t n, size_t n_obs) {
   size_t b = 0;
   b += align256(13 * n * 4) + align256(8 * n * 4) + align256(4 * n * 4) + align256(4 * n * 4);
   b += align256(n) + align256(n * 4) + align256(n) + align256(4) + align256(OrderLayout{(uint32_t)n, (uint32_t)n, 0}.total() * sizeof(uint32_t));
-  b += align256(n_obs * n * 16) + align256(n_obs * n * 32);
+  b += align256(n_obs * n * 16) + align256(n_obs * n * 32) + align256(n_obs ? 10 * n * 4 : 0);
   return b;
 }
 
@@ -185,6 +185,7 @@ struct ServeRequest {
   std::chrono::steady_clock::time_point t_submit, t_done;
   size_t offset = 0;
   agk::FleetBuffers fb{};
+  float* box_stage = nullptr;  // [10][n] one box's rows on their way from host memory
   uint32_t remaining = 0;
   bool started = false;
   bool done = false;
@@ -201,8 +202,10 @@ struct ag_server {
   // two chunks can be in flight: chunk k uses buffer k % 2
   cudaEvent_t chunk_start[2] = {nullptr, nullptr}, chunk_done[2] = {nullptr, nullptr};
   unsigned char* slab = nullptr;
-  float* box_stage = nullptr;  // rows of a request's boxes on their way from host memory (one request at a time, in stream order)
-  size_t box_stage_bytes = 0;
+  // several boxes' rows on their way from host memory, made for the first request that brings them; requests
+  // use it one after another, in stream order
+  agk::BoxStage box_stage{nullptr, 64u << 20};
+  bool box_stage_tried = false;
   agk::SlabAllocator* alloc = nullptr;
   agk::ServeDesc* table_host[2] = {nullptr, nullptr};  // pinned
   agk::ServeDesc* table_dev[2] = {nullptr, nullptr};
@@ -250,6 +253,7 @@ void carve(ag_server* s, ServeRequest* r) {
   f.reset_ids = f.order;  // written by the initial reset, before the order is built
   f.box_bound = (float4*)take(n_obs * n * 16);
   f.box_rest = (float4*)take(n_obs * n * 32);
+  r->box_stage = (float*)take(n_obs ? 10 * n * 4 : 0);
   f.n = (uint32_t)n;
   f.n_quad = (uint32_t)n;
   f.n_obs = (uint32_t)n_obs;
@@ -303,8 +307,15 @@ cudaError_t start_request(ag_server* s, ServeRequest* r) {
       e = cudaGetLastError();
     }
   }
-  if (e == cudaSuccess && in.n_obstacles)
-    e = agk::upload_boxes(f, in.boxes, pitch, s->box_stage, s->box_stage_bytes, st);
+  if (e == cudaSuccess && in.n_obstacles) {
+    if (!s->box_stage_tried) {
+      s->box_stage_tried = true;
+      s->box_stage.rows = agk::alloc_box_stage(s->box_stage.bytes);
+    }
+    const size_t one = 10 * n * sizeof(float);
+    const bool shared = s->box_stage.rows && s->box_stage.bytes > one;
+    e = agk::upload_boxes(f, in.boxes, pitch, shared ? s->box_stage : agk::BoxStage{r->box_stage, one}, st);
+  }
   if (e == cudaSuccess) e = cudaMemsetAsync(f.epoch, 0, n * 4, st);
   if (e == cudaSuccess) e = agk::launch_reset(f, nullptr, (uint32_t)(in.seed & 0xFFFFFFFFu), (uint32_t)(in.seed >> 32), st);
   if (e == cudaSuccess) e = agk::launch_build_order(f, st);
@@ -481,12 +492,9 @@ ag_status ag_server_create(const ag_server_config* cfg, ag_server** out) {
     if (e == cudaSuccess) e = cudaMalloc((void**)&s->table_dev[b], sizeof(agk::ServeDesc) * cfg->max_active);
   }
   if (e == cudaSuccess) e = cudaMalloc((void**)&s->slab, cfg->hbm_budget_bytes);
-  s->box_stage_bytes = std::min<uint64_t>(64u << 20, cfg->hbm_budget_bytes);
-  if (e == cudaSuccess) e = cudaMalloc((void**)&s->box_stage, s->box_stage_bytes);
   if (e != cudaSuccess) {
     cudaGetLastError();
     if (s->slab) cudaFree(s->slab);
-    if (s->box_stage) cudaFree(s->box_stage);
     for (int b = 0; b < 2; ++b) {
       if (s->table_host[b]) cudaFreeHost(s->table_host[b]);
       if (s->table_dev[b]) cudaFree(s->table_dev[b]);
@@ -582,7 +590,7 @@ ag_status ag_server_destroy(ag_server* s) {
   for (auto& kv : s->all) delete kv.second;
   delete s->alloc;
   cudaFree(s->slab);
-  cudaFree(s->box_stage);
+  if (s->box_stage.rows) cudaFree(s->box_stage.rows);
   for (int b = 0; b < 2; ++b) {
     cudaFreeHost(s->table_host[b]);
     cudaFree(s->table_dev[b]);

@@ -102,10 +102,10 @@ def test_vehicle_at_a_box_centre_collides(n_obs, steps, monkeypatch):
     env.close()
 
 
-@pytest.mark.parametrize("n,n_obs,budget", [(1001, 5, 0), (6_800_001, 1, 0), (1000, 5, 475_000)])
+@pytest.mark.parametrize("n,n_obs,budget", [(1001, 5, 0), (700_001, 10, 0), (1000, 5, 516_000), (1000, 5, 475_000)])
 def test_obstacles_from_host_memory_in_several_parts(n, n_obs, budget):
-    """All boxes at once; more rows of one box than the staging holds (256 MB);
-    two boxes at a time, which is what the budget leaves."""
+    """All boxes at once; nine and then one (more rows than 256 MB); two and one
+    at a time, which is what the budgets leave."""
     from paper_2305_16510_gb300 import _abi
     rng = np.random.default_rng(n)
     boxes = rng.uniform(0.1, 5.0, (n_obs, 10, n)).astype(np.float32)

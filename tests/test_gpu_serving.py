@@ -205,8 +205,8 @@ def test_request_inputs_in_host_memory_give_the_same_results(n, n_obs, with_body
 
 @pytest.mark.parametrize("n,n_obs", [(150_001, 12), (1_700_001, 1)])
 def test_request_boxes_from_host_memory_in_several_parts(n, n_obs):
-    """More rows than the server stages at once (64 MiB): some boxes at a time,
-    and part of one box at a time, give what boxes in device memory give."""
+    """More rows than the server stages at once (64 MiB): some boxes at a time, and
+    one at a time in the request's own memory, give what boxes in device memory give."""
     from paper_2305_16510_gb300.serving import RequestPool
     w = W.Workload("parts", n, 4, 1, n_obs, n, 0, 0, mode_mix=(0, 1, 2))
     inp = W.make_inputs(w, 16)
