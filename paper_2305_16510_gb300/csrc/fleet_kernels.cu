@@ -88,10 +88,15 @@ __global__ void __launch_bounds__(128, !BOXES && QUAD_ONLY && INTEG == kIntegSIE
 // window of 4,096 needs four times the padding (8 % with three rotor types,
 // which cost a 4M mixed fleet 0.9 %).
 // One block per window. Each warp takes a contiguous share of the window's
-// environments, 32 at a time, and counts them by key (__match_any_sync, one
+// environments, 32 at a time, and ranks them by key (__match_any_sync, one
 // add per key and 32 environments); a scan over the warps gives every warp its
-// place in each key's run, and a second pass over the modes writes the slots.
+// place in each key's run, and the environments go to their slots. All ROUNDS
+// modes of a thread are requested, and all matches made, before any is counted:
+// a kernel that asked for each mode as it came to it, twice, took 18.6 us a call of
+// ag_set_commands for 16,384 to 1M quads, this one 12.5 to 14.5. Fleets of up to
+// 1,024 and 4,096 environments take 1 and 4 rounds; with 16 they wait 2 us longer.
 constexpr int kOrderThreads = 1024, kOrderWarps = kOrderThreads / 32;
+constexpr int kOrderRounds = kOrderWindow / kOrderThreads;  // environments per thread of a whole window
 
 __host__ __device__ inline OrderLayout order_layout(const FleetBuffers& fb) { return {fb.n, fb.n_quad, fb.n_hexa}; }
 
@@ -101,8 +106,9 @@ __device__ __forceinline__ uint32_t order_key(const FleetBuffers& fb, uint32_t i
   return (uint32_t)(nrot == 4 ? 0 : (nrot == 6 ? 1 : 2)) * 4u + m;
 }
 
+template <int ROUNDS>
 __global__ void __launch_bounds__(kOrderThreads) k_order_window(FleetBuffers fb) {
-  __shared__ uint32_t place[kOrderWarps][12];  // counts, then the next place of the warp in each key's run
+  __shared__ uint32_t place[kOrderWarps][13];  // counts (the last: of no environment), then the warp's place in each key's run
   __shared__ uint32_t run[12];                 // length, then the first slot of each key's run
   const OrderLayout layout = order_layout(fb);
   const uint32_t first = blockIdx.x * kOrderWindow, count = layout.count(blockIdx.x), slots = layout.slots(blockIdx.x);
@@ -110,13 +116,24 @@ __global__ void __launch_bounds__(kOrderThreads) k_order_window(FleetBuffers fb)
   const uint32_t warp = threadIdx.x >> 5, lane = threadIdx.x & 31u;
   const uint32_t share = (count + kOrderThreads - 1) / kOrderThreads * 32u;  // environments per warp
   const uint32_t lo = warp * share, hi = min(lo + share, count);
+  uint32_t key[ROUNDS], rank[ROUNDS];  // of environment lo + 32 j + lane in its warp's share
+#pragma unroll
+  for (int j = 0; j < ROUNDS; ++j) {
+    const uint32_t i = lo + 32u * j + lane;
+    key[j] = i < hi ? order_key(fb, first + i) : 12u;
+  }
   for (uint32_t k = threadIdx.x; k < slots; k += kOrderThreads) order[k] = kNoEnv;
-  if (lane < 12) place[warp][lane] = 0;
+  if (lane < 13) place[warp][lane] = 0;
   __syncwarp();
-  for (uint32_t i = lo; i < hi; i += 32) {
-    const uint32_t key = i + lane < hi ? order_key(fb, first + i + lane) : 12u;
-    const unsigned same = __match_any_sync(0xFFFFFFFFu, key);
-    if (key < 12u && (int)lane == __ffs(same) - 1) place[warp][key] += __popc(same);
+#pragma unroll
+  for (int j = 0; j < ROUNDS; ++j) rank[j] = __match_any_sync(0xFFFFFFFFu, key[j]);
+#pragma unroll
+  for (int j = 0; j < ROUNDS; ++j) {
+    const unsigned same = rank[j];
+    const uint32_t before = place[warp][key[j]];
+    __syncwarp();
+    rank[j] = before + __popc(same & ((1u << lane) - 1u));
+    if ((int)lane == __ffs(same) - 1) place[warp][key[j]] = before + __popc(same);
     __syncwarp();
   }
   __syncthreads();
@@ -141,17 +158,9 @@ __global__ void __launch_bounds__(kOrderThreads) k_order_window(FleetBuffers fb)
     }
   }
   __syncthreads();
-  for (uint32_t i = lo; i < hi; i += 32) {
-    const uint32_t key = i + lane < hi ? order_key(fb, first + i + lane) : 12u;
-    const unsigned same = __match_any_sync(0xFFFFFFFFu, key);
-    const uint32_t at = key < 12u ? place[warp][key] : 0u;
-    __syncwarp();
-    if (key < 12u) {
-      if ((int)lane == __ffs(same) - 1) place[warp][key] = at + __popc(same);
-      order[run[key] + at + __popc(same & ((1u << lane) - 1u))] = first + i + lane;
-    }
-    __syncwarp();
-  }
+#pragma unroll
+  for (int j = 0; j < ROUNDS; ++j)
+    if (key[j] < 12u) order[run[key[j]] + place[warp][key[j]] + rank[j]] = first + lo + 32u * j + lane;
 }
 
 // Box records k0 .. from the caller's rows and back: thread (env, box).
@@ -352,7 +361,10 @@ cudaError_t launch_fused_step(const FleetBuffers& fb_in, const StepParams& P, in
 }
 
 cudaError_t launch_build_order(const FleetBuffers& fb, cudaStream_t st) {
-  k_order_window<<<order_layout(fb).windows(), kOrderThreads, 0, st>>>(fb);
+  const auto kernel = fb.n <= kOrderThreads       ? k_order_window<1>
+                      : fb.n <= 4 * kOrderThreads ? k_order_window<4>
+                                                  : k_order_window<kOrderRounds>;
+  kernel<<<order_layout(fb).windows(), kOrderThreads, 0, st>>>(fb);
   return cudaGetLastError();
 }
 

@@ -57,3 +57,21 @@ def test_adjoint_does_not_depend_on_a_vehicles_slot(n):
     for a, b in zip(*outs):
         np.testing.assert_array_equal(a, b)
     assert np.isfinite(outs[0][1]).all() and (np.abs(outs[0][1]).sum(axis=0) > 0).all()
+
+
+@pytest.mark.parametrize("n", [1024, 3000, 4095, 4096, 4097, 9000, 16384 + 4097])
+def test_order_around_the_sizes_of_its_kernels(n, monkeypatch):
+    """Fleets of up to 1,024 and 4,096 environments are ordered in fewer rounds."""
+    w = _workload(n, True)
+    inp = W.make_inputs(w, 3)
+    outs = []
+    for order in ("grouped", "identity"):
+        monkeypatch.setenv("AG_FUSED_ORDER", order)
+        fl = gpu_fleet(w, inp, 3)
+        fl.set_commands(modes=inp.modes[::-1].copy())   # another order over the first one
+        fl.reset(None, 3)
+        fl.step(3)
+        outs.append((fl.state().cpu().numpy(), fl.motors().cpu().numpy()))
+        fl.close()
+    for a, b in zip(*outs):
+        np.testing.assert_array_equal(a, b)
