@@ -102,36 +102,41 @@ __global__ void k_fill_rows(float* dst, uint32_t n, float v0, float v1, float v2
 }
 
 // Up to three device arrays of 32-bit words copied in one launch: block
-// (x, y) takes a share of array y, in 16-byte words where both ends allow.
-// ag_set_state's three copies were three operations on the stream: 131,072
-// quads of two modes x 100 steps from given states take 112.2 us a pass instead
-// of 117.3. Large fleets keep the copies, which move more bytes per second (4M
-// vehicles, 50 steps: 1767 us against 1787 with this kernel).
+// (x, y) takes a share of array y, in 16-byte words where both ends allow. Bound
+// by memory: eight words per thread in flight, and four blocks per SM and array
+// at most (152 SMs), since more, shorter blocks cost up to a third (2^19 vehicles
+// 22.7 us a call with a block per 16 KB, 16.6 so). ag_set_state's three copies
+// take 12.4 us at 2^17 vehicles (6.4 with this kernel), 28.5 at 450,001 (14.5),
+// 18.7 at 2^19, 64.9 at 2^21 (60.5) and 227 at 8,000,001 (215), but 442 at 2^24
+// (446) and 1,042 at 40M (1,061), which draws the line at 2^23. From an address
+// that is not a multiple of 16 they take 8.3 us at 65,536 (6.4), 20.7 at 450,001
+// (12.8) and 14.6 at 2^19 (16.7), but 34.9 at 2^20 (36.5) and 58.8 at 2^21 (68.7).
 struct CopyJob { const uint32_t* src; uint32_t* dst; size_t words; };
 struct CopyJobs { CopyJob job[3]; };
-constexpr int kCopyBlock = 256, kCopyUnroll = 4;
-constexpr size_t kCopyMostEnvs = 1 << 19;  // 46 MB of state, motors and epochs
+constexpr int kCopyBlock = 256, kCopyUnroll = 8;
+constexpr size_t kCopyMostBlocks = 4 * 152;
+constexpr size_t kCopyMostWide = 1 << 23, kCopyMostNarrow = 1 << 19;  // vehicles
+
+template <class W>
+__device__ __forceinline__ void copy_words(const W* src, W* dst, size_t n) {
+  const size_t step = (size_t)gridDim.x * kCopyBlock;
+  for (size_t i = (size_t)blockIdx.x * kCopyBlock + threadIdx.x; i < n; i += step * kCopyUnroll) {
+    W v[kCopyUnroll];
+#pragma unroll
+    for (int u = 0; u < kCopyUnroll; ++u)
+      if (i + u * step < n) v[u] = src[i + u * step];
+#pragma unroll
+    for (int u = 0; u < kCopyUnroll; ++u)
+      if (i + u * step < n) dst[i + u * step] = v[u];
+  }
+}
 
 __global__ void __launch_bounds__(kCopyBlock) k_copy(CopyJobs jobs) {
   const CopyJob j = jobs.job[blockIdx.y];
-  const size_t step = (size_t)gridDim.x * kCopyBlock, first = (size_t)blockIdx.x * kCopyBlock + threadIdx.x;
-  size_t done = 0;
-  if (((reinterpret_cast<uintptr_t>(j.src) | reinterpret_cast<uintptr_t>(j.dst)) & 15u) == 0) {
-    const uint4* src = reinterpret_cast<const uint4*>(j.src);
-    uint4* dst = reinterpret_cast<uint4*>(j.dst);
-    const size_t n = j.words / 4;
-    for (size_t i = first; i < n; i += step * kCopyUnroll) {
-      uint4 v[kCopyUnroll];
-#pragma unroll
-      for (int u = 0; u < kCopyUnroll; ++u)
-        if (i + u * step < n) v[u] = src[i + u * step];
-#pragma unroll
-      for (int u = 0; u < kCopyUnroll; ++u)
-        if (i + u * step < n) dst[i + u * step] = v[u];
-    }
-    done = n * 4;
-  }
-  for (size_t i = done + first; i < j.words; i += step) j.dst[i] = j.src[i];
+  const bool wide = ((reinterpret_cast<uintptr_t>(j.src) | reinterpret_cast<uintptr_t>(j.dst)) & 15u) == 0;
+  const size_t done = wide ? j.words / 4 * 4 : 0;
+  if (wide) copy_words(reinterpret_cast<const uint4*>(j.src), reinterpret_cast<uint4*>(j.dst), done / 4);
+  copy_words(j.src + done, j.dst + done, j.words - done);
 }
 
 // Precondition checks of ag_set_body and ag_set_obstacles: each counts the
@@ -694,13 +699,14 @@ ag_status ag_set_state(ag_ctx* ctx, const float* state, const float* motors, con
   if (s != AG_OK) return s;
   if (!state) return fail_invalid(ctx, "state is NULL");
   const size_t n = ctx->cfg.n_envs;
-  if (motors && n <= kCopyMostEnvs && on_own_device(ctx, state) && on_own_device(ctx, motors) &&
-      (!epoch || on_own_device(ctx, epoch))) {
+  const bool wide = ((reinterpret_cast<uintptr_t>(state) | reinterpret_cast<uintptr_t>(motors)) & 15u) == 0;
+  if (motors && n <= (wide ? kCopyMostWide : kCopyMostNarrow) && on_own_device(ctx, state) &&
+      on_own_device(ctx, motors) && (!epoch || on_own_device(ctx, epoch))) {
     const CopyJobs jobs = {{{(const uint32_t*)state, (uint32_t*)ctx->fb.state, 13 * n},
                             {(const uint32_t*)motors, (uint32_t*)ctx->fb.motors, 8 * n},
                             {epoch, ctx->fb.epoch, n}}};
-    const size_t share = (size_t)kCopyBlock * kCopyUnroll * 4;  // words of the largest array per block
-    const unsigned blocks = (unsigned)((13 * n + share - 1) / share < 8192 ? (13 * n + share - 1) / share : 8192);
+    const size_t share = (size_t)kCopyBlock * kCopyUnroll * (wide ? 4 : 1);  // words of the largest array per block
+    const unsigned blocks = (unsigned)std::min((13 * n + share - 1) / share, kCopyMostBlocks);
     k_copy<<<dim3(blocks, epoch ? 3 : 2), kCopyBlock, 0, ctx->stream>>>(jobs);
     return check_cuda(ctx, cudaGetLastError(), "copy state in");
   }

@@ -35,3 +35,18 @@ def test_set_state_from_device_arrays_of_any_alignment(n, with_epoch):
         np.testing.assert_array_equal(fl.motors().cpu().numpy(), motors)
         np.testing.assert_array_equal(fl.epoch().cpu().numpy(), epoch if with_epoch else np.zeros(n, np.int32))
     fl.close()
+
+
+@pytest.mark.parametrize("n", [8191, 600_001, (1 << 20) + 3, (1 << 23) + 1])
+def test_set_state_around_the_lines_between_copies_and_kernel(n):
+    """Blocks that take several turns; above 2^19 vehicles at an odd address and
+    above 2^23 at any the copies serve."""
+    torch.manual_seed(n)
+    for words in (0, 1):
+        s = torch.rand(13 * n + words, device="cuda")[words:].view(13, n)
+        m = torch.rand(8 * n + words, device="cuda")[words:].view(8, n)
+        e = torch.randint(1, 1000, (n,), dtype=torch.int32, device="cuda")
+        fl = Fleet(n)
+        _abi.ag_set_state(fl.ctx, s, m, e)
+        assert torch.equal(fl.state(), s) and torch.equal(fl.motors(), m) and torch.equal(fl.epoch(), e)
+        fl.close()
