@@ -241,9 +241,9 @@ __global__ void __launch_bounds__(256) k_plain_integrate(FleetBuffers fb, StepPa
   store_state(fb.state, n, i, s);
 }
 
-// Collision test of every environment against all its boxes, from the
-// caller's rows (the allocation-free step) or the context's records; the
-// per-env hit byte goes to `collided_now`.
+// Collision test of every environment against its boxes: every box of the
+// caller's rows (the allocation-free step), or the context's records, spheres
+// first as in the fused step; the per-env hit byte goes to `collided_now`.
 __global__ void __launch_bounds__(256) k_plain_collide(FleetBuffers fb, StepParams P, uint8_t* collided_now) {
   const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= fb.n) return;
@@ -257,8 +257,8 @@ __global__ void __launch_bounds__(256) k_plain_collide(FleetBuffers fb, StepPara
                                      Q4{bx[6 * n], bx[7 * n], bx[8 * n], bx[9 * n]}));
     }
   } else {
-    const EnvBoxes boxes(fb, i);
-    for (uint32_t k = 0; k < fb.n_obs; ++k) hit |= touches(P.r2, boxes.dist2(p, (int)k));
+    float clearance2;
+    hit = EnvBoxesT<true, true>(fb, i).any_hit(p, sqrtf(P.r2), P.r2, (int)fb.n_obs, kBoxSlack, false, clearance2);
   }
   collided_now[i] = hit ? 1 : 0;
 }
