@@ -26,9 +26,11 @@
 // recomputes one segment's entries at a time.
 //
 // Thread slot s handles environment order[s] (grouped by rotor type and
-// command mode, as in the fused step): a warp runs one mode's code. Tape,
-// checkpoints and the norm of q_0 are kept in slot order, so their rows are
-// read and written coalesced whatever the modes are.
+// command mode, as in the fused step): a warp runs one mode's code. The tape and
+// the norm of q_0 are kept in slot order, so their rows are read and written
+// coalesced whatever the modes are. Checkpoints are kept by environment: they
+// grow with the horizon, and the padding slots of a fleet of one would make them
+// 96 times as large.
 //
 // Attitude adjoint. The adjoint of the unit quaternion is carried as the
 // 3-vector g of the right perturbation q -> q (1, delta / 2): the step's
@@ -170,8 +172,8 @@ template <bool FULL_TAPE> struct Record {
     int to_ckpt = 0;
     for (int t = 0; t < ab.n_steps; ++t) {
       if (!FULL_TAPE && to_ckpt-- == 0) {
-        store_vehicle(ckpt, ckpt + 13 * (size_t)ns, ns, slot, x);
-        ckpt += 21 * (size_t)ns;
+        store_vehicle(ckpt, ckpt + 13 * (size_t)n, n, env, x);
+        ckpt += 21 * (size_t)n;
         to_ckpt = ab.K - 1;
       }
       const VState start = x.s;
@@ -541,8 +543,8 @@ template <bool FULL_TAPE> struct Sweep {
         const int t0 = seg * K, len = H - t0 < K ? H - t0 : K;
         float4* const tape = ab.tape + slot;
         Vehicle<NROT> v;
-        const float* ck = ab.ckpt + (size_t)seg * 21 * ns;
-        load_vehicle(ck, ck + 13 * ns, (uint32_t)ns, slot, v);
+        const float* ck = ab.ckpt + (size_t)seg * 21 * n;
+        load_vehicle(ck, ck + 13 * n, (uint32_t)n, env, v);
         for (int t = 0; t < len; ++t) {
           const VState start = v.s;
           float wf;

@@ -21,9 +21,10 @@ inline bool tape_within_budget(uint64_t budget, size_t other, size_t entries, si
 
 // Device buffers of one recorded rollout and its adjoint. Arrays marked
 // "slot" have n_slots columns, one per thread slot (environment order[slot],
-// none in the padding); the others are indexed by environment. With full_tape the tape holds the entries of every step and the
-// end state; else it holds one segment's K entries, and checkpoint s holds
-// the state (13 rows) and motors (8 rows) at step s * K.
+// none in the padding); the others are indexed by environment. With full_tape
+// the tape holds the entries of every step and the end state; else it holds one
+// segment's K entries, and checkpoint s holds the state (13 rows) and motors (8
+// rows) at step s * K.
 struct AdjointBuffers {
   float* state;                // [13][n] fleet state (advanced by the record)
   float* motors;               // [8][n]
@@ -33,7 +34,7 @@ struct AdjointBuffers {
   const uint32_t* order;       // [n_slots] thread slot -> environment, grouped by rotor type and mode
   const float* goal_in;        // [3][n] the record's goals (the caller's array, or p_goal)
   float* p_goal;               // [3][n] kept for the sweep, written by the record
-  float* ckpt;                 // [S][21] slot (NULL with full_tape)
+  float* ckpt;                 // [S][21][n] (NULL with full_tape)
   float4* tape;                // [n_steps + 1][4] (full_tape) or [K][4], slot
   float* inv_q0;               // slot: 1 / |q_0| of the given initial quaternion
   float* loss;                 // [n]

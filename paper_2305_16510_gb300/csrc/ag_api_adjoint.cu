@@ -88,10 +88,10 @@ ag_status ensure_adjoint(ag_ctx* ctx, int n_steps, int K) {
       cudaStreamSynchronize(ctx->stream);
       cudaFree(a.ckpt);
       a.ckpt = nullptr;
-      ctx->bytes -= ctx->adj_ckpt_cap * 21 * slots * sizeof(float);
+      ctx->bytes -= ctx->adj_ckpt_cap * 21 * n * sizeof(float);
       ctx->adj_ckpt_cap = 0;
     }
-    e = alloc(ctx, &a.ckpt, n_ckpt * 21 * slots);
+    e = alloc(ctx, &a.ckpt, n_ckpt * 21 * n);
     if (e != cudaSuccess) { cudaGetLastError(); a.ckpt = nullptr; ctx->err = "checkpoints do not fit"; return AG_ERR_OOM; }
     ctx->adj_ckpt_cap = n_ckpt;
   }
