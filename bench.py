@@ -59,9 +59,10 @@ FLOP_PER_VEHICLE_STEP_MIXED = 584.4
 # substep the controller (state 52, mode 1, targets 16, body 16 in; command
 # 16 out), allocation (command 16, motors 16 in; motors 16, wrench 16 out)
 # and integrator (state 52, wrench 16, body 16 in; state 52 out), 301 B x 4;
-# per step the collision test (position 12, 16 boxes x 40 in; hit byte out)
-# and the reset pass (hit byte in).
-PLAIN_BYTES_PER_VEHICLE_STEP = 301 * 4 + 12 + 16 * 40 + 1 + 1
+# per step the collision test (position 12, 16 circumscribed spheres x 16 in,
+# the few boxes within reach not counted; hit byte out) and the reset pass (hit
+# byte in).
+PLAIN_BYTES_PER_VEHICLE_STEP = 301 * 4 + 12 + 16 * 16 + 1 + 1
 HBM_PEAK_GBS = 6788.3  # measured GB300 copy bandwidth (MEASURED_PEAKS.json, hbm_gbs)
 
 
@@ -90,10 +91,10 @@ def alu_peak_tflops(info: dict) -> float:
 BYTES_PER_VEHICLE_LAUNCH = 4 * (26 + 8 + 4 + 4) + 1 + 8 + 4 * 160 + 1 + 4
 # DRAM traffic of one full-size fused launch (1,048,576 envs, 1,000 steps):
 # dram__bytes_read.sum + dram__bytes_write.sum from a one-pass ncu capture of
-# exactly this launch (413.52 MB + 60.44 MB). It scales with the fleet size
+# exactly this launch (414.87 MB + 60.38 MB). It scales with the fleet size
 # (each env is loaded and stored once per launch, of each box its 16-byte
 # sphere and of the few near ones the record), not with the step count.
-TRAFFIC_BYTES_FULL_LAUNCH = 413.523200e6 + 60.444928e6
+TRAFFIC_BYTES_FULL_LAUNCH = 414.867456e6 + 60.380672e6
 # Algorithmic bytes of one reach-task step per quad: read action 16, goal 12,
 # step counter 4, state 52, motors 16, body 16, epoch 4, mode 1 (121 B);
 # written state 52, motors 16, epoch 4, collided flag 1, command 16,
@@ -541,9 +542,10 @@ def task_part(seed: int, world: int) -> dict:
 
 # ----------------------------------------------------------------- adjoint --
 def adjoint_part(seed: int, world: int, alu_peak: float) -> dict:
-    """Differentiable rollout at 65,536 quads x 256 steps (position mode, SIE,
-    checkpoint every 32): recorded forward + hand-written adjoint. Each half
-    is timed with CUDA events on the fleet's stream."""
+    """Differentiable rollout at 65,536 quads x 256 steps (position mode, SIE;
+    the whole horizon's tape fits, so no checkpoints are kept): recorded forward
+    + hand-written adjoint. Each half is timed with CUDA events on the fleet's
+    stream."""
     import torch
     from paper_2305_16510_gb300 import _abi, workloads as W
     w = W.WORKLOADS["adjoint"]
@@ -591,7 +593,7 @@ def adjoint_part(seed: int, world: int, alu_peak: float) -> dict:
                                       "reverse": FLOP_PER_VEHICLE_STEP_ADJ_REV},
             "alu_frac_record": units * FLOP_PER_VEHICLE_STEP_ADJ_FWD / fwd_s / 1e12 / alu_peak,
             "alu_frac_backward": units * FLOP_PER_VEHICLE_STEP_ADJ_REV / bwd_s / 1e12 / alu_peak,
-            "workload": "65,536 quads, position mode, SIE, horizon 256, checkpoint every 32 steps, "
+            "workload": "65,536 quads, position mode, SIE, horizon 256, whole-horizon tape, "
                         "gradients w.r.t. x0 (13/vehicle) and 12 gains"}
 
 

@@ -19,13 +19,13 @@
  *   - Arrays are structure-of-arrays over environments: field r of env i sits
  *     at index r * n_envs + i, in float32 unless stated.
  *   - Pointer arguments may point to host memory (pageable or pinned) or to
- *     device memory of the context's device; the library copies with
- *     cudaMemcpyAsync(cudaMemcpyDefault). The caller owns them; they are only
- *     borrowed for the duration of the call, except that copies FROM a
- *     pageable host buffer have completed when the call returns, and copies
- *     INTO any buffer have completed once the context's stream has been
- *     synchronised (ag_synchronize) — pinned/device destinations may still be
- *     written after the call returns.
+ *     device memory of the context's device. Aligned arrays of the context's
+ *     device may be read and written in place by the library's kernels; others
+ *     are copied with cudaMemcpyAsync(cudaMemcpyDefault). Either happens in the
+ *     order of the context's stream. The caller owns them: copies FROM a
+ *     pageable host buffer have completed when the call returns, while pinned
+ *     and device arrays may still be read, and any buffer written, until the
+ *     context's stream has passed the call (ag_synchronize).
  *   - Calls are asynchronous on the context's CUDA stream unless stated.
  *   - Errors: AG_ERR_INVALID leaves the context unchanged. After a CUDA error
  *     the context is failed and every later call except ag_last_error and
@@ -451,7 +451,9 @@ typedef struct {
   ag_config physics;         /* per-step physics of every request */
   uint32_t max_active;       /* requests on the device at once, 1..AG_SERVER_MAX_ACTIVE */
   uint32_t chunk_steps;      /* steps per launch (1 .. 2^30) */
-  uint64_t hbm_budget_bytes; /* device memory for request buffers (>= 1 MiB) */
+  uint64_t hbm_budget_bytes; /* device memory for request buffers (>= 1 MiB); 64 MiB
+                                more stage boxes once a request brings them from
+                                host memory, where the device has room */
 } ag_server_config;
 
 typedef struct {
@@ -487,11 +489,12 @@ ag_status ag_server_create(const ag_server_config* cfg, ag_server** out);
 
 /* Queues a request (thread-safe, non-blocking) and returns its id. The input
  * arrays (host or device) must stay valid until ag_server_wait has returned
- * for this id. The loop uploads them when it admits the request: device (or
- * pinned) arrays are copied asynchronously, while pageable host arrays make
- * the loop wait for their copy before it queues the next chunk. Their contents are not checked (submission stays cheap): they
- * must meet the preconditions of ag_set_commands, ag_set_body and
- * ag_set_obstacles. AG_ERR_INVALID for a malformed request (n_envs outside
+ * for this id. The loop takes them in when it admits the request: arrays
+ * that all lie in the server's device memory are read in place by a kernel,
+ * pinned ones are copied asynchronously, and pageable host arrays make the loop
+ * wait for their copy before it queues the next chunk. Their contents are not
+ * checked (submission stays cheap): they must meet the preconditions of
+ * ag_set_commands, ag_set_body and ag_set_obstacles. AG_ERR_INVALID for a malformed request (n_envs outside
  * 1 .. AG_MAX_ENVS, other counts, NULL arrays, pitch), AG_ERR_OOM if it
  * could never fit the budget, AG_ERR_STATE
  * if the server has failed. */

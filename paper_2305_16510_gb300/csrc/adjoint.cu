@@ -198,7 +198,7 @@ template <bool FULL_TAPE> struct Record {
 // One warp per block: the fleet's warps spread evenly over the SMs (a
 // 65,536-vehicle fleet puts 13 or 14 on each of 152 SMs, where 128-thread
 // blocks would put 12 on some and 16 on others). Writing the tape here costs
-// little beside the step: 65,536 quads x 256 steps take 192 us at 5.3 TB/s of
+// little beside the step: 65,536 quads x 256 steps take 193 us at 5.6 TB/s of
 // tape, against 176 us without it and another 194 us to recompute it later.
 constexpr int kRecordBlock = 32;
 template <bool FULL_TAPE>
@@ -596,10 +596,10 @@ template <bool FULL_TAPE> struct Sweep {
 
 // One warp per block and at most 128 registers: four warps fit per SM
 // sub-partition, 16 per SM, so a 65,536-vehicle fleet (2,048 warps) is
-// resident in one wave on 152 SMs; nothing spills. Bound by instruction issue
-// (75 % of cycles, and the sub-partitions that hold four warps, not three,
+// resident in one wave on 152 SMs; three words spill. Bound by instruction issue
+// (72 % of cycles, and the sub-partitions that hold four warps, not three,
 // finish last); the tape leaves DRAM at half its rate. 65,536 quads x 256
-// steps: 262 us for 206 M warp instructions, against 501 us for 365 M (and
+// steps: 267 us for 202 M warp instructions, against 501 us for 365 M (and
 // 194 us for a launch that recomputed the tape) when the sweep rebuilt the
 // whole step and carried the adjoints of q and R.
 // The warp's sum of each gain's adjoint (a fixed tree over its lanes) goes to

@@ -114,9 +114,10 @@ struct NoBoxSource {
 // decision only and takes near = kBoxSlack; the others take kBoxNear, or
 // kBoxNearShort in calls of up to kShortCall steps, where a vehicle gets no
 // further, so that the clearance is exact up to near and at least the distance
-// to the other spheres (674,653 quads, 10 boxes, 2 / 6 / 20 steps: 195.9 ->
-// 192.1, 223.5 -> 218.9 and 299.2 -> 294.9 us a pass with the shorter reach;
-// 0.1 m 191.6 / 218.1 / 296.1, 0.05 m 191.4 / 218.5 / 298.2).
+// to the other spheres. 674,653 quads among 10 boxes, a reset and 2 / 6 / 20 / 32 /
+// 64 / 256 steps: 144.0 / 185.5 / 288.5 / 374.5 / 601 / 1,978 us with the shorter
+// reach throughout, 146.6 / 188.5 / 289.7 / 372.0 / 597 / 1,955 with the longer;
+// they meet between 20 and 32 steps. (0.1 and 0.05 m do as 0.2 m does.)
 // The sphere's distance is taken low by 3e-4 of the centre distance, which
 // covers the hardware square root and a quaternion whose norm is off by the
 // 1e-4 that ag_set_obstacles admits, and kBoxSlack covers the rest of the
@@ -132,17 +133,23 @@ struct NoBoxSource {
 constexpr float kBoxSlack = 1e-3f, kBoxNearShort = 0.2f, kBoxNear = 0.5f;  // m
 constexpr int kShortCall = 32;
 
+// Boxes that are large and flat gain nothing: every vehicle of a room lies within
+// a wall's sphere, so a test reads 64 bytes of a wall instead of 40 and twice the
+// instructions. Calls of many steps among nothing but walls (5 x 5 x 0.05 m) take
+// longer than with a test of every box from rows in pairs (65,536 quads x 8 walls x
+// 200 steps 325 us against 279, x 6 of 16 boxes 382 against 380).
 // GROUPED: the spheres are loaded in whole groups (8, or 16 while more than 8
 // are left) before any is looked at, so that a group waits for memory once. It
-// serves the single-step kernel, where every thread tests (131,072 quads with
+// serves the single-step kernels, where every thread tests (131,072 quads with
 // 3 / 8 / 16 / 32 boxes: 23.3 / 27.6 / 34.7 / 52.5 us a pass); in the launches
 // of many steps, where few do, the plain loop leaves more registers to the
 // step (1M x 1,000 steps: 50.5 ms against 51.6).
 // DENSE: while more than two boxes are marked, four are tested at a time (the last
 // one again where fewer are left), so that their loads are in flight together. It
-// serves the single-step fused kernel; in the task step it costs 3 % among 16
-// small boxes (19.1 -> 19.7 us), and inside the loops of the many-step kernel the
-// longer code misses the instruction cache (1M x 1,000 steps 11 % slower).
+// serves the single-step fused kernel and the unfused test; in the task step it
+// costs 3 % among 16 small boxes (19.1 -> 19.7 us), and inside the loops of the
+// many-step kernel the longer code misses the instruction cache (no_instruction 0.24
+// -> 1.15 stalls per issue, 1M x 1,000 steps 10 % slower).
 template <bool GROUPED, bool DENSE = false> struct EnvBoxesT {
   const float4* bound;  // this environment's column of box_bound
   const float4* rest;   // and of box_rest

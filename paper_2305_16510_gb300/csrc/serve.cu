@@ -52,6 +52,8 @@ struct ServeDesc {
 
 constexpr int kServeBlock = 128;
 
+// The bound of 4 blocks holds the kernel to 128 registers, 16 warps per SM; 48
+// bytes per thread spill (192 loaded).
 template <int INTEG, bool DRAG>
 __global__ void __launch_bounds__(kServeBlock, 4) k_serve_step(const ServeDesc* __restrict__ table, int n_req,
                                                            StepParams P, int substeps) {

@@ -98,7 +98,10 @@ __device__ __forceinline__ VState reach_fly(const ReachArgs& a, const StepParams
 // Without boxes the step is memory-latency bound: a bound of 12 blocks (24
 // warps) per SM measured best (50.8 us a pass over 1,048,576 quads), against
 // 10 (53.2), 14 (51.3), 16 (52.2, 64 registers) and 18 (53.3); with the state
-// requested after the command's angles it took 57.4. With boxes 8 blocks (16
+// requested after the command's angles it took 57.4. RK4 is within 3 % of its best
+// there: 1,048,576 quads x 4 substeps 73.9 us (10 blocks 72.7, 14 76.4), x 1 substep
+// 49.4 (52.4, 54.2), mixed airframes x 4 80.6 (78.2, 79.6) and with drag 81.2 (78.6,
+// 82.5), though those two kernels spill 40 and 72 bytes. With boxes 8 blocks (16
 // warps, 128 registers).
 template <int INTEG, bool QUAD_ONLY, bool DRAG, bool BOXES>
 __global__ void __launch_bounds__(kTaskBlock, BOXES ? 8 : 12)
